@@ -725,6 +725,9 @@ __device__ __forceinline__ void epilogue_row_spec(const ConvArgs &args, uint32_t
       dst[0] = h[0];
     }
   }
+  // a last 64-bit word of which only the low half-word holds channels
+  const int nhalf = (nvalid + LH - 1) / LH;
+  if (args.out_word64 && (nhalf & 1) && row_valid) row32[nhalf] = 0u;
 }
 
 __host__ __device__ constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }

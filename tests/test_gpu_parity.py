@@ -330,3 +330,20 @@ def test_conv_packed_only_outputs_partial_groups(samd_lib, fo_bits, fo_signed):
         assert np.array_equal(got[:n], want), (K, R, word_bits, spacer)
         assert np.array_equal(got[n:], np_words(torch.full((guard,), 0x5A5A5A5A, dtype=samd.word_dtype(fo)), word_bits))
     assert_status_clean()
+
+
+# 64-bit output words of 1-, 2-, 4- and 8-bit lanes are written as 32-bit
+# halves: a last word whose channels end in its low half must still be whole.
+@pytest.mark.parametrize("fo_bits,K", [(1, 16), (1, 70), (2, 16), (2, 40), (4, 24), (4, 290), (8, 20), (8, 33)])
+def test_conv_packed_only_last_64bit_word_is_whole(samd_lib, fo_bits, K):
+    shape = samd.ConvShape(1, 16, 6, 5, K)
+    a_v, w_v, a_w, w_w, fa, fw = conv_case(shape, 4, False, 3, True, synth.seed_for("w64", K, fo_bits))
+    fo = samd.fmt(fo_bits, False, 0, 64)
+    shift = harness_shift(4, 3, fo_bits, shape.C * shape.R * shape.S)
+    n = samd.samd_packed_words(fo, shape.N * shape.Ho * shape.Wo, K)
+    buf = torch.full((n + 8,), 0x5A5A5A5A5A5A5A5A, dtype=torch.int64, device="cuda")
+    samd.samd_conv2d(shape.desc(), fa, a_w, fw, w_w, None, fo, buf, shift, samd.conv_workspace(shape, fa, fw))
+    got = np_words(buf, 64)
+    assert np.array_equal(got[:n], oracle_requant_pack(oracle_conv_nhwc(a_v, w_v, shape), shift, fo))
+    assert (got[n:] == 0x5A5A5A5A5A5A5A5A).all()
+    assert_status_clean()
