@@ -697,7 +697,6 @@ samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const 
   a.Wo = p.Wo;
   a.M = p.M;
   a.wpr = p.wpr;
-  a.words_total = p.words_total;
   a.nchunks = p.nchunks;
   a.NBc = p.NBc;
   a.n_mma = p.n_mma;

@@ -147,7 +147,6 @@ struct ConvArgs {
   int N, C, H, W, K, R, S, stride, pad, Ho, Wo;
   long long M;
   int wpr;          // activation words per pixel
-  int words_total;  // R * S * wpr: reduction length in packed words (GATHER)
   int nchunks;      // weight tiles per output tile
   int NBc;          // output channels per channel block
   int n_mma;        // NBc rounded up to 16
@@ -437,65 +436,61 @@ __device__ __forceinline__ void load_window(const uint8_t *row, int o4, int nw, 
   }
 }
 
-// Gathers the packed words of one pixel's chunk into shared memory with
-// cp.async: word kw of the reduction is word (kw mod wpr) of the input pixel
-// at tap kw / wpr; taps outside the image and words past the end are
-// zero-filled (source size 0).
+// Gathers one output pixel's operand chunks (implicit im2col): chunk (j, r, q)
+// is channel chunk j, the words [j WC, min((j + 1) WC, wpr)), of the input
+// pixel under tap (r, q); taps outside the image are zero-filled (source size
+// 0). The position of the chunk is kept by counters that advance one chunk at
+// a time, in the order of the reduction: taps inside channel chunks (windows)
+// or channel chunks inside taps (whole 16-byte vectors).
 template <typename W, int WC>
 struct AGather {
   const W *act;
-  int H, W_, wpr, S, stride, pad, words_total, taps;
-  int n, oh, ow;
+  int H, W_, wpr, R, S, nck;
+  bool win;
   bool row_valid;
-  bool vec;  // every chunk lies inside one pixel at a kVec-aligned offset
+  int ih0, iw0, pix0;    // input pixel under tap (0, 0) of this thread's output pixel
+  int j = 0, r = 0, q = 0;
 
-  __device__ __forceinline__ const W *pixel(int tap, bool &valid) const {
-    int r = tap / S, s = tap - (tap / S) * S;
-    int ih = oh * stride - pad + r, iw = ow * stride - pad + s;
-    valid = row_valid && ih >= 0 && ih < H && iw >= 0 && iw < W_;
-    return act + ((static_cast<long long>(n) * H + ih) * W_ + iw) * wpr;
+  // Next chunk; true after the output tile's last one.
+  __device__ __forceinline__ bool advance() {
+    if (!win) {
+      if (++j < nck) return false;
+      j = 0;
+    }
+    if (++q < S) return false;
+    q = 0;
+    if (++r < R) return false;
+    r = 0;
+    if (!win) return true;
+    if (++j < nck) return false;
+    j = 0;
+    return true;
   }
 
-  __device__ __forceinline__ void issue(int chunk, uint32_t dst) const {
-    const int kw0 = chunk * WC;
-    int tap = kw0 / wpr, wi = kw0 - tap * wpr;
-    bool valid;
-    const W *px = pixel(tap, valid);
-    if (vec) {
-      stage_chunk<W, WC>(dst, reinterpret_cast<const char *>(valid ? px + wi : act), valid ? 1u : 0u);
-      return;
-    }
-#pragma unroll
-    for (int q = 0; q < WC; ++q) {
-      const bool in = valid && kw0 + q < words_total;
-      const W *src = in ? px + wi : act;
-      if constexpr (sizeof(W) == 8)
-        ptx::cp_async_8(dst + 8 * q, src, in ? 8u : 0u);
-      else
-        ptx::cp_async_4(dst + 4 * q, src, in ? 4u : 0u);
-      if (++wi == wpr) {
-        wi = 0;
-        ++tap;
-        px = pixel(tap, valid);
-      }
-    }
+  __device__ __forceinline__ const W *chunk(bool &valid) const {
+    valid = row_valid && static_cast<unsigned>(ih0 + r) < static_cast<unsigned>(H) &&
+            static_cast<unsigned>(iw0 + q) < static_cast<unsigned>(W_);
+    return act + (static_cast<long long>(pix0 + r * W_ + q) * wpr + j * WC);
   }
 
-  // Chunks that are not whole 16-byte vectors (issue_win): chunk c is
-  // channel chunk j = c / taps of the pixel at tap c % taps, the words
-  // [j WC, min((j + 1) WC, wpr)) of that pixel, copied as the 16-byte pieces
-  // of the aligned window around them, so that every copy is 16 bytes wide
-  // whatever the pixel's alignment. Pieces past the chunk are zero-filled;
-  // a piece that reaches past the end of the activation tensor (act_end)
-  // copies only the bytes before it. Returns the chunk's offset into the
-  // staged row in 32-bit units (load_window). act is 16-byte aligned.
-  __device__ __forceinline__ int issue_win(int chunk, uint32_t dst, uintptr_t act_end) const {
-    const int j = chunk / taps;
-    const int wi = j * WC;
-    const int nw = wpr - wi < WC ? wpr - wi : WC;
+  // A chunk that is a whole number of aligned 16-byte vectors.
+  __device__ __forceinline__ void issue(uint32_t dst) const {
     bool valid;
-    const W *px = pixel(chunk - j * taps, valid);
-    const uintptr_t a = valid ? reinterpret_cast<uintptr_t>(px + wi) : reinterpret_cast<uintptr_t>(act);
+    const W *src = chunk(valid);
+    stage_chunk<W, WC>(dst, reinterpret_cast<const char *>(valid ? src : act), valid ? 1u : 0u);
+  }
+
+  // Any other chunk is copied as the 16-byte pieces of the aligned window
+  // around it, so that every copy is 16 bytes wide whatever the pixel's
+  // alignment. Pieces past the chunk are zero-filled; a piece that reaches
+  // past the end of the activation tensor (act_end) copies only the bytes
+  // before it. Returns the chunk's offset into the staged row in 32-bit units
+  // (load_window). act is 16-byte aligned.
+  __device__ __forceinline__ int issue_win(uint32_t dst, uintptr_t act_end) const {
+    const int nw = wpr - j * WC < WC ? wpr - j * WC : WC;
+    bool valid;
+    const W *px = chunk(valid);
+    const uintptr_t a = valid ? reinterpret_cast<uintptr_t>(px) : reinterpret_cast<uintptr_t>(act);
     const uintptr_t a0 = a & ~static_cast<uintptr_t>(15);
     const uintptr_t end = a + static_cast<uintptr_t>(nw) * sizeof(W);
 #pragma unroll
@@ -977,20 +972,20 @@ __device__ __forceinline__ void epilogue_row(const ConvArgs &args, uint32_t tadd
   }
 }
 
+// A role's wait on one of the kernel's barriers, by whole warps.
+__device__ __forceinline__ void role_wait(uint32_t bar, uint32_t parity, int *status) {
+  ptx::mbar_wait(bar, parity, status, static_cast<int>(SAMD_ETIMEOUT), kWaitLimitNs);
+}
+
 // The epilogue warps' meeting point of a pooled tile: every warp of the
 // tile's group arrives on `bar` once its part of the step is done, then
-// waits, bounded, for the phase; false if the wait gave up.
-__device__ __forceinline__ bool epi_group_sync(uint32_t bar, uint32_t &phase, volatile int *status) {
+// waits, bounded, for the phase.
+__device__ __forceinline__ void epi_group_sync(uint32_t bar, uint32_t &phase, int *status) {
   __syncwarp();
-  bool ok = true;
-  if ((threadIdx.x & 31) == 0) {
-    ptx::mbar_arrive(bar);
-    ok = ptx::mbar_wait_bounded(bar, phase & 1u, status, kWaitLimitNs);
-  }
+  if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(bar);
+  role_wait(bar, phase & 1u, status);
   ++phase;
-  ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
   __syncwarp();
-  return ok;
 }
 
 // Epilogue of one pooled tile for output lanes of OB = 1, 2, 4 or 8 bits
@@ -1000,11 +995,11 @@ __device__ __forceinline__ bool epi_group_sync(uint32_t bar, uint32_t &phase, vo
 // accumulator, meet the other epilogue warps, then write the lane-wise max of
 // every 2x2 window of the tile's row pairs (the maximum commutes with the
 // monotone requantize, so this is the pool of the requantized output), and
-// meet again before the buffer is reused. False if a wait gave up.
+// meet again before the buffer is reused.
 template <int OB, bool OS>
-__device__ __noinline__ bool epilogue_pool_tile(const ConvArgs &args, uint32_t taddr, int trow, uint32_t mt, int nb,
+__device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t taddr, int trow, uint32_t mt, int nb,
                                                 uint32_t *pbuf, uint32_t acc_empty, uint32_t group_bar,
-                                                uint32_t &phase, volatile int *status, int gw, int gi) {
+                                                uint32_t &phase, int *status, int gw, int gi) {
   constexpr int LH = 32 / OB;  // lanes per word
   constexpr int NH = 32 / LH;  // words per 32 channels
   constexpr int32_t lo = OS ? -(1 << (OB - 1)) : 0, hi = OS ? (1 << (OB - 1)) - 1 : (1 << OB) - 1;
@@ -1046,7 +1041,7 @@ __device__ __noinline__ bool epilogue_pool_tile(const ConvArgs &args, uint32_t t
   ptx::tc_fence_before();
   __syncwarp();
   if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(acc_empty);
-  if (!epi_group_sync(group_bar, phase, status)) return false;
+  epi_group_sync(group_bar, phase, status);
   // the 2x2 windows of this tile's row pairs
   const uint32_t img = fdiv(mt, args.fd_tpi);
   const int g = static_cast<int>(mt - img * args.fd_tpi.d);
@@ -1065,23 +1060,23 @@ __device__ __noinline__ bool epilogue_pool_tile(const ConvArgs &args, uint32_t t
     const long long orow = (static_cast<long long>(img) * Ho2 + g * q + i) * Wo2 + j;
     out[orow * args.out_wpr + w] = swar_lane_max<uint32_t, OB>(top, bot, flip);
   }
-  return epi_group_sync(group_bar, phase, status);
+  epi_group_sync(group_bar, phase, status);
 }
 
-__device__ __forceinline__ bool epilogue_pool_dispatch(const ConvArgs &args, uint32_t taddr, int trow, uint32_t mt,
+__device__ __forceinline__ void epilogue_pool_dispatch(const ConvArgs &args, uint32_t taddr, int trow, uint32_t mt,
                                                        int nb, uint32_t *pbuf, uint32_t acc_empty, uint32_t group_bar,
-                                                       uint32_t &phase, volatile int *status, int gw, int gi) {
+                                                       uint32_t &phase, int *status, int gw, int gi) {
 #define SAMD_POOL_TILE(OB, OS) \
   epilogue_pool_tile<OB, OS>(args, taddr, trow, mt, nb, pbuf, acc_empty, group_bar, phase, status, gw, gi)
   switch (args.out_bits * 2 + (args.out_signed ? 1 : 0)) {
-    case 2: return SAMD_POOL_TILE(1, false);
-    case 3: return SAMD_POOL_TILE(1, true);
-    case 4: return SAMD_POOL_TILE(2, false);
-    case 5: return SAMD_POOL_TILE(2, true);
-    case 8: return SAMD_POOL_TILE(4, false);
-    case 9: return SAMD_POOL_TILE(4, true);
-    case 16: return SAMD_POOL_TILE(8, false);
-    default: return SAMD_POOL_TILE(8, true);
+    case 2: SAMD_POOL_TILE(1, false); return;
+    case 3: SAMD_POOL_TILE(1, true); return;
+    case 4: SAMD_POOL_TILE(2, false); return;
+    case 5: SAMD_POOL_TILE(2, true); return;
+    case 8: SAMD_POOL_TILE(4, false); return;
+    case 9: SAMD_POOL_TILE(4, true); return;
+    case 16: SAMD_POOL_TILE(8, false); return;
+    default: SAMD_POOL_TILE(8, true); return;
   }
 #undef SAMD_POOL_TILE
 }
@@ -1191,7 +1186,7 @@ __device__ __forceinline__ void issue_taps(uint32_t d, uint32_t dn, uint64_t a, 
 //               first, store-free pass over the first tile fetches the
 //               epilogue's code early. Pooled tiles (ConvArgs::pool) are
 //               drained, requantized and pooled by the warps of a group.
-// Every wait is bounded; a role that gives up records SAMD_ETIMEOUT and stops.
+// Every wait is bounded; one that gives up records SAMD_ETIMEOUT (role_wait).
 template <typename W, int BITS, bool SIGNED, bool HALO, bool FP8, bool FULL, int HV>
 __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                                            const ConvArgs args) {
@@ -1224,7 +1219,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   // four of epilogue set g (one-half tiles, group_bar(g))
   auto group_bar = [&](int g) { return ptx::smem_addr(bars + 2 * STB + 2 * NO + 5 + g); };
 
-  volatile int *status = args.status;
+  int *const status = args.status;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // No global read precedes the setup barrier: a failure recorded by an
   // earlier launch is seen by the first wait that has to wait.
@@ -1255,10 +1250,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
 
-  const long long total_tiles = static_cast<long long>(args.grid_m) * args.nblocks;
-  const long long first_tile = blockIdx.x, tile_step = gridDim.x;
+  // fewer than 2^31 tiles, and a CTA's last step stays below 2^31 + gridDim.x (checked on the host)
+  const uint32_t total_tiles = static_cast<uint32_t>(args.grid_m) * static_cast<uint32_t>(args.nblocks);
+  const uint32_t first_tile = blockIdx.x, tile_step = gridDim.x;
   const int nchunks = args.nchunks;  // weight tiles per output tile
-  bool ok = true;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1273,25 +1268,33 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         // the CTA does not exit with a copy in flight, whatever the other roles do
         for (int c = 0; c < nchunks; ++c) ptx::mbar_wait_bounded(full_b(c), 0, &quiet, kWaitLimitNs);
       } else {
-        long long cb = 0;
-        for (long long tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
-          const int nb = static_cast<int>(tile / args.grid_m);
-          for (int c = 0; c < nchunks; ++c, ++cb) {
-            const int s = static_cast<int>(cb % STB);
-            const long long round = cb / STB;
-            if (round > 0 &&
-                !ptx::mbar_wait_bounded(empty_b(s), static_cast<uint32_t>((round - 1) & 1), status, kWaitLimitNs)) {
-              ok = false;
-              break;
-            }
+        // Ring position and round parity advance by increments (a 64-bit
+        // division by the runtime ring size costs this thread about as much
+        // as the rest of the step).
+        int s = 0, loaded = 0;  // loaded: tiles issued so far, counted up to the ring's size
+        uint32_t par = 1;       // parity of the previous round's release
+        for (uint32_t tile = first_tile; tile < total_tiles; tile += tile_step) {
+          const int row0 = static_cast<int>(fdiv(tile, args.fd_gm)) * args.mma_n;
+          for (int c = 0; c < nchunks; ++c) {
+            if (loaded == STB)
+              role_wait(empty_b(s), par, status);
+            else
+              ++loaded;
             ptx::mbar_arrive_expect_tx(full_b(s), b_bytes);
-            ptx::tma_load_2d(ptx::smem_addr(sB + s * b_bytes), &tmap_b, c * BK, nb * args.mma_n, full_b(s));
+            ptx::tma_load_2d(ptx::smem_addr(sB + s * b_bytes), &tmap_b, c * BK, row0, full_b(s));
+            if (++s == STB) {
+              s = 0;
+              par ^= 1;
+            }
           }
         }
-        if (!ok) {  // leave no copy in flight: wait (bounded) for the last ring's worth
-          for (long long k = (cb > STB ? cb - STB : 0); k < cb; ++k)
-            ptx::mbar_wait_bounded(full_b(static_cast<int>(k % STB)), static_cast<uint32_t>((k / STB) & 1), &quiet,
-                                   kWaitLimitNs / 10);
+        // the CTA does not exit with a copy in flight: the ring's last round,
+        // oldest first (slots q < s were filled in this round, whose full
+        // phase has parity par ^ 1, the others in the round before)
+        for (int k = 0; k < loaded; ++k) {
+          int q = loaded == STB ? s + k : k;
+          if (q >= STB) q -= STB;
+          ptx::mbar_wait_bounded(full_b(q), q < s ? par ^ 1u : par, &quiet, kWaitLimitNs / 10);
         }
       }
     }
@@ -1303,11 +1306,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     // turns every descriptor into a per-thread value that has to be moved to
     // the uniform datapath before each MMA, which costs more than the MMA.
     const uint32_t idesc = ptx::idesc_f16_f32(BM, args.mma_n);
-    auto wait = [&](uint32_t bar, uint32_t parity) {
-      bool w_ok = true;
-      if (lane == 0) w_ok = ptx::mbar_wait_bounded(bar, parity, status, kWaitLimitNs);
-      return __shfl_sync(0xffffffffu, w_ok ? 1 : 0, 0) != 0;
-    };
+    auto wait = [&](uint32_t bar, uint32_t parity) { role_wait(bar, parity, status); };
     // Ring positions advance by increments (no division in this loop).
     int sb = 0, so = 0;
     uint32_t bpar = 0, opar = 0;
@@ -1319,27 +1318,29 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     const uint32_t dn = static_cast<uint32_t>(args.mma_n);          // the second half's accumulator columns
     const uint32_t a_skip16 = HALO ? static_cast<uint32_t>(args.row_step - args.S) * a_row16 : 0u;
     if (resident)  // resident weights: wait for all of them once
-      for (int c = 0; c < nchunks && ok; ++c)
-        if (!wait(full_b(c), 0)) ok = false;
-    long long i = 0;
-    for (long long tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++i) {
+      for (int c = 0; c < nchunks; ++c) wait(full_b(c), 0);
+    uint32_t i = 0;
+    for (uint32_t tile = first_tile; tile < total_tiles; tile += tile_step, ++i) {
       const int a = static_cast<int>(i & 1);
-      if (i >= 2 && !wait(accempty(a), static_cast<uint32_t>(((i >> 1) - 1) & 1))) {
-        ok = false;
-        break;
-      }
+      if (i >= 2) wait(accempty(a), ((i >> 1) - 1) & 1u);
       ptx::tc_fence_after();  // the epilogue's reads of this accumulator are complete
       const uint32_t tmem_d = tmem_base + static_cast<uint32_t>(a * HV * args.mma_n);
       uint32_t acc = 0;
-      for (int j = 0; j < nops && ok; ++j) {
-        if (!wait(opfull(so), opar)) {
-          ok = false;
-          break;
+      int jt = 0, jc = 0;  // window gather: tap and channel chunk of item j
+      for (int j = 0; j < nops; ++j) {
+        wait(opfull(so), opar);
+        // words of the packed chunk: channel chunk j (halo) or jc (window
+        // gather) of a pixel; the chunks of a vector gather are whole
+        int words = WC;
+        if (HALO) {
+          words = args.wpr - j * WC;
+        } else if (args.gather_win) {
+          words = args.wpr - jc * WC;
+          if (++jt == args.taps) {
+            jt = 0;
+            ++jc;
+          }
         }
-        // words of the packed chunk: channel chunk j (halo) or j / taps
-        // (window gather) of a pixel, else words j WC.. of the whole reduction
-        int words = HALO ? args.wpr - j * WC
-                         : (args.gather_win ? args.wpr - (j / args.taps) * WC : args.words_total - j * WC);
         if (words > WC) words = WC;
         int npos = words * U::L;
         if (npos > BK) npos = BK;  // FULL: the last word's lanes past 64 are padding
@@ -1359,10 +1360,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           uint64_t adesc = a0;
           int ts = 0;
           for (int t = 0; t < taps_here; ++t) {
-            if (!wait(full_b(sb), bpar)) {
-              ok = false;
-              break;
-            }
+            wait(full_b(sb), bpar);
             const uint64_t bdesc = T::desc(sB_addr + sb * b_bytes);
             if (ptx::elect_one()) {
               mma_ksteps<FP8, HV>(ksteps, tmem_d, dn, adesc, a_half16, bdesc, idesc, acc);
@@ -1390,10 +1388,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           opar ^= 1;
         }
       }
-      if (ok) {
-        if (ptx::elect_one()) ptx::mma_commit(accfull(a));
-        __syncwarp();
-      }
+      if (ptx::elect_one()) ptx::mma_commit(accfull(a));
+      __syncwarp();
     }
     if (ptx::elect_one()) ptx::mma_commit(drain_bar);
     __syncwarp();
@@ -1406,11 +1402,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     // ---- operand producers ----
     const int t = threadIdx.x - 64;  // 0 .. kProdThreads - 1
     const W *act = static_cast<const W *>(args.act);
-    auto wait_lane0 = [&](uint32_t bar, uint32_t parity) {
-      bool w_ok = true;
-      if (lane == 0) w_ok = ptx::mbar_wait_bounded(bar, parity, status, kWaitLimitNs);
-      return __shfl_sync(0xffffffffu, w_ok ? 1 : 0, 0) != 0;
-    };
     if constexpr (HALO) {
       const int halo_rows = args.nseg * args.seg_rows;
       // halo row hr -> virtual offset from the tile's first position, or -1
@@ -1420,8 +1411,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         return q < args.seg_used ? g * args.Wp + q : -1;
       };
       // items k = (tile i, channel chunk j), in the MMA's order
-      auto gather = [&](long long tile, int j, int slot) {
-        const uint32_t mt = static_cast<uint32_t>(tile) - fdiv(static_cast<uint32_t>(tile), args.fd_gm) * args.fd_gm.d;
+      auto gather = [&](uint32_t tile, int j, int slot) {
+        const uint32_t mt = tile - fdiv(tile, args.fd_gm) * args.fd_gm.d;
         const uint32_t v0 = tile_first_pos(args, mt, BMT);
         const uint32_t dst0 = ptx::smem_addr(sG + slot * args.g_stride);
         for (int hr = t; hr < halo_rows; hr += kProdThreads) {
@@ -1451,7 +1442,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           }
         }
       };
-      auto advance = [&](long long &tile, int &j) {
+      auto advance = [&](uint32_t &tile, int &j) {
         if (++j == args.nck) {
           j = 0;
           tile += tile_step;
@@ -1464,7 +1455,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       // A thread reads back only the rows it gathered itself, so refilling
       // the slot it finished with one item earlier needs no barrier.
       const int D = args.gdepth;
-      long long gtile = first_tile;  // issue side
+      uint32_t gtile = first_tile;  // issue side
       int gj = 0, gslot = 0;
       auto issue = [&]() {
         if (gtile < total_tiles) gather(gtile, gj, gslot);
@@ -1473,9 +1464,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         if (++gslot == D) gslot = 0;
       };
       for (int d = 0; d + 1 < D; ++d) issue();
-      long long ctile = first_tile;  // widening side
+      uint32_t ctile = first_tile;  // widening side
       int cj = 0, cslot = 0;
-      for (long long k = 0; ctile < total_tiles; ++k) {
+      int hb = 0;           // halo buffer of item k
+      bool reused = false;  // buffers are in their second or a later round
+      uint32_t hpar = 1;    // parity of the previous round's release
+      while (ctile < total_tiles) {
         issue();
         if (D == 4)
           ptx::cp_async_wait<3>();
@@ -1483,11 +1477,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           ptx::cp_async_wait<2>();
         else
           ptx::cp_async_wait<1>();  // item k of this thread's rows has landed
-        const int hb = static_cast<int>(k % NO);
-        if (k >= NO && !wait_lane0(opempty(hb), static_cast<uint32_t>(((k / NO) - 1) & 1))) {
-          ok = false;
-          break;
-        }
+        if (reused) role_wait(opempty(hb), hpar, status);
         const uint8_t *stg = sG + cslot * args.g_stride;
         for (int hr = t; hr < halo_rows; hr += kProdThreads) {
           if (voff(hr) < 0) continue;  // a row no tap reads
@@ -1500,6 +1490,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         if (lane == 0) ptx::mbar_arrive(opfull(hb));
         advance(ctile, cj);
         if (++cslot == D) cslot = 0;
+        if (++hb == NO) {
+          hb = 0;
+          reused = true;
+          hpar ^= 1;
+        }
       }
       ptx::cp_async_wait<0>();
     } else {
@@ -1509,55 +1504,49 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       const int grp = t / BM;
       const int row = (HV == 2 ? grp * BM : 0) + t % BM;  // row of the A tile
       constexpr int kItemStep = HV == 2 ? 1 : 2;
+      const bool win = args.gather_win != 0;
       AGather<W, WC> g;
       g.act = act;
       g.H = args.H;
       g.W_ = args.W;
       g.wpr = args.wpr;
+      g.R = args.R;
       g.S = args.S;
-      g.stride = args.stride;
-      g.pad = args.pad;
-      g.words_total = args.words_total;
-      g.taps = args.taps;
-      g.vec = args.gather_vec != 0;
-      auto set_tile = [&](long long tile) {
-        const uint32_t tl = static_cast<uint32_t>(tile);
-        const uint32_t mt = tl - fdiv(tl, args.fd_gm) * args.fd_gm.d;
+      g.nck = args.nck;
+      g.win = win;
+      auto set_tile = [&](uint32_t tile) {
+        const uint32_t mt = tile - fdiv(tile, args.fd_gm) * args.fd_gm.d;
         const uint32_t m = mt * BMT + row;
         g.row_valid = m < static_cast<uint64_t>(args.M);
         const uint32_t mm = g.row_valid ? m : 0u;
         const uint32_t tq = fdiv(mm, args.fd_wo);
-        g.ow = static_cast<int>(mm - tq * args.fd_wo.d);
         const uint32_t nq = fdiv(tq, args.fd_ho);
-        g.oh = static_cast<int>(tq - nq * args.fd_ho.d);
-        g.n = static_cast<int>(nq);
+        g.iw0 = static_cast<int>(mm - tq * args.fd_wo.d) * args.stride - args.pad;
+        g.ih0 = static_cast<int>(tq - nq * args.fd_ho.d) * args.stride - args.pad;
+        g.pix0 = (static_cast<int>(nq) * args.H + g.ih0) * args.W + g.iw0;
       };
       const uint32_t g_row = static_cast<uint32_t>(args.g_row);  // staging row pitch
       const uint32_t kSlotBytes = BM * g_row;
       const uint32_t slot0 = ptx::smem_addr(sG) + grp * (kGatherDepth * kSlotBytes) + (t % BM) * g_row;
-      const bool win = args.gather_win != 0;
       const uintptr_t act_end = reinterpret_cast<uintptr_t>(args.act) + static_cast<uintptr_t>(args.act_bytes);
       uint32_t o4s = 0;  // window offsets of the kGatherDepth slots, 2 bits each
-      // issue side: this group's item (itile, ic), kGatherDepth ahead of the consume side
-      long long itile = first_tile;
-      int ic = 0;
+      // Items (tile, chunk) are counted, not divided: the issue side runs
+      // kGatherDepth of this group's items ahead of the consume side.
+      uint32_t itile = first_tile;
       auto step = [&]() {
-        if (++ic == nchunks) {
-          ic = 0;
-          itile += tile_step;
-        }
+        if (g.advance()) itile += tile_step;
       };
       if (HV == 1 && grp == 1) step();
       if (itile < total_tiles) set_tile(itile);
       auto issue_next = [&](int slot) {
         if (itile < total_tiles) {
           if (win) {
-            const int o4 = g.issue_win(ic, slot0 + slot * kSlotBytes, act_end);
+            const int o4 = g.issue_win(slot0 + slot * kSlotBytes, act_end);
             o4s = (o4s & ~(3u << (2 * slot))) | (static_cast<uint32_t>(o4) << (2 * slot));
           } else {
-            g.issue(ic, slot0 + slot * kSlotBytes);
+            g.issue(slot0 + slot * kSlotBytes);
           }
-          const long long prev = itile;
+          const uint32_t prev = itile;
           step();
           if (kItemStep == 2) step();
           if (itile != prev && itile < total_tiles) set_tile(itile);
@@ -1566,32 +1555,48 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       };
 #pragma unroll 1
       for (int d = 0; d < kGatherDepth; ++d) issue_next(d);
-      const long long items = ((total_tiles - first_tile + tile_step - 1) / tile_step) * nchunks;
+      const long long items = static_cast<long long>((total_tiles - first_tile + tile_step - 1) / tile_step) * nchunks;
       int slot = 0;
+      int ct = 0, cj = 0;   // windows: tap and channel chunk of the item consumed next
+      auto cstep = [&]() {
+        if (++ct == args.taps) {
+          ct = 0;
+          if (++cj == args.nck) cj = 0;
+        }
+      };
+      int sa = 0;           // A tile of the item
+      bool reused = false;  // the A tiles are in their second or a later round
+      uint32_t apar = 1;    // parity of the previous round's release
+      if (HV == 1 && grp == 1) {
+        cstep();
+        sa = 1;
+      }
       for (long long k = HV == 2 ? 0 : grp; k < items; k += kItemStep) {
         ptx::cp_async_wait<kGatherDepth - 1>();
         W cur[WC];
         const uint8_t *srow = sG + grp * (kGatherDepth * kSlotBytes) + slot * kSlotBytes + (t % BM) * g_row;
         if (win) {
-          const int chunk = static_cast<int>(k % nchunks);
-          const int wi = (chunk / args.taps) * WC;
+          const int wi = cj * WC;
           const int nw = args.wpr - wi < WC ? args.wpr - wi : WC;
           load_window<W, WC>(srow, static_cast<int>((o4s >> (2 * slot)) & 3u), nw, cur);
+          cstep();
+          if (kItemStep == 2) cstep();
         } else {
           load_staged<W, WC>(srow, cur);
         }
-        const int sa = static_cast<int>(k % NO);
-        const long long round = k / NO;
-        if (round > 0 && !wait_lane0(opempty(sa), static_cast<uint32_t>((round - 1) & 1))) {
-          ok = false;
-          break;
-        }
+        if (reused) role_wait(opempty(sa), apar, status);
         U::unpack_row(cur, sOp + sa * args.op_stride, row);
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(opfull(sa));
         issue_next(slot);  // refill the slot just read
         if (++slot == kGatherDepth) slot = 0;
+        sa += kItemStep;
+        if (sa >= NO) {
+          sa -= NO;
+          reused = true;
+          apar ^= 1;
+        }
       }
       ptx::cp_async_wait<0>();
     }
@@ -1611,7 +1616,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     // set * kParts .. set * kParts + kParts - 1 (HV = 2: its half; HV = 4:
     // two of the four parts); with HV = 1 the sets take alternate tiles
     constexpr int kParts = HV == 4 ? 2 : 1;
-    long long i = HV >= 2 ? 0 : set;
+    uint32_t i = HV >= 2 ? 0 : set;
     // The first pass over the first tile runs with its stores off and without
     // waiting for the accumulator (whatever it reads is discarded): the row
     // epilogue is the largest code of the kernel, and this way its
@@ -1631,47 +1636,30 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         const uint32_t gbar = group_bar(HV == 2 ? 0 : set);
         constexpr int kStep = HV == 2 ? 1 : 2;
         uint32_t gphase = 0;
-        long long ip = HV == 2 ? 0 : set;
-        for (long long tile = first_tile + (HV == 2 ? 0 : set) * tile_step; tile < total_tiles;
+        uint32_t ip = HV == 2 ? 0 : set;
+        for (uint32_t tile = first_tile + (HV == 2 ? 0 : set) * tile_step; tile < total_tiles;
              tile += kStep * tile_step, ip += kStep) {
           const int acc_i = HV == 2 ? static_cast<int>(ip & 1) : set;
-          bool w_ok = true;
-          if (lane == 0)
-            w_ok = ptx::mbar_wait_bounded(accfull(acc_i), static_cast<uint32_t>((ip >> 1) & 1), status, kWaitLimitNs);
-          if (!__shfl_sync(0xffffffffu, w_ok ? 1 : 0, 0)) {
-            ok = false;
-            break;
-          }
+          role_wait(accfull(acc_i), (ip >> 1) & 1u, status);
           ptx::tc_fence_after();
-          const uint32_t tl = static_cast<uint32_t>(tile);
-          const uint32_t nbu = fdiv(tl, args.fd_gm);
-          const uint32_t mt = tl - nbu * args.fd_gm.d;
+          const uint32_t nbu = fdiv(tile, args.fd_gm);
+          const uint32_t mt = tile - nbu * args.fd_gm.d;
           const uint32_t taddr = tmem_base + static_cast<uint32_t>((acc_i * HV + (HV == 2 ? set : 0)) * args.mma_n) +
                                  (static_cast<uint32_t>(quad * 32) << 16);
-          if (!epilogue_pool_dispatch(args, taddr, (HV == 2 ? set * BM : 0) + row, mt, static_cast<int>(nbu), pbuf,
-                                      accempty(acc_i), gbar, gphase, status, gw, gi)) {
-            ok = false;
-            break;
-          }
+          epilogue_pool_dispatch(args, taddr, (HV == 2 ? set * BM : 0) + row, mt, static_cast<int>(nbu), pbuf,
+                                 accempty(acc_i), gbar, gphase, status, gw, gi);
         }
       }
     }
-    for (long long tile = first_tile + (HV >= 2 ? 0 : set) * tile_step; !pooled && tile < total_tiles;) {
+    for (uint32_t tile = first_tile + (HV >= 2 ? 0 : set) * tile_step; !pooled && tile < total_tiles;) {
       const int acc_i = HV >= 2 ? static_cast<int>(i & 1) : set;  // accumulator of this tile
       if (!warm) {
-        bool w_ok = true;
-        if (lane == 0)
-          w_ok = ptx::mbar_wait_bounded(accfull(acc_i), static_cast<uint32_t>((i >> 1) & 1), status, kWaitLimitNs);
-        if (!__shfl_sync(0xffffffffu, w_ok ? 1 : 0, 0)) {
-          ok = false;
-          break;
-        }
+        role_wait(accfull(acc_i), (i >> 1) & 1u, status);
         ptx::tc_fence_after();
       }
-      const uint32_t tl = static_cast<uint32_t>(tile);
-      const uint32_t nbu = fdiv(tl, args.fd_gm);
+      const uint32_t nbu = fdiv(tile, args.fd_gm);
       const int nb = static_cast<int>(nbu);
-      const uint32_t mt = tl - nbu * args.fd_gm.d;
+      const uint32_t mt = tile - nbu * args.fd_gm.d;
 #pragma unroll 1
       for (int hh = 0; hh < kParts; ++hh) {
         const int part = HV >= 2 ? set * kParts + hh : 0;
@@ -1713,7 +1701,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, args.tmem_cols);
   }
-  if (!ok) atomicOr(const_cast<int *>(status), static_cast<int>(SAMD_ETIMEOUT));
 }
 
 // cudaFuncSetAttribute once per (kernel, device); defined in conv2d.cu.

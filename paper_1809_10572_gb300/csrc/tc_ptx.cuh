@@ -72,7 +72,7 @@ __device__ __forceinline__ bool elect_one() {
 
 // Wait for the phase with the given parity to complete. Gives up after
 // `limit_ns` of wall time, or as soon as another CTA has recorded a failure
-// in *status; either way it returns false and the caller stops its work.
+// in *status, and returns false.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, volatile int *status,
                                                   uint64_t limit_ns) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -81,6 +81,25 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     if (mbar_try_wait_hint(bar, parity, 20000u)) return true;
     if (*status != 0) return false;
     if (global_timer_ns() - t0 > limit_ns) return false;
+  }
+}
+
+// The kernel roles' wait, executed by whole warps (every lane polls): a wait
+// that gives up records `code` in *status and returns like any other, so that
+// the callers' control flow does not depend on the outcome and stays uniform
+// (the compiler keeps ring positions and descriptors in uniform registers).
+// The loops of a failed launch run on to their end without waiting longer
+// than one poll; their results are undefined, as the status says.
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int *status, int code, uint64_t limit_ns) {
+  if (__builtin_expect(!mbar_try_wait(bar, parity), 0)) {
+    const uint64_t t0 = global_timer_ns();
+    while (!mbar_try_wait_hint(bar, parity, 20000u)) {
+      if (*static_cast<volatile int *>(status) != 0) break;
+      if (global_timer_ns() - t0 > limit_ns) {
+        atomicOr(status, code);
+        break;
+      }
+    }
   }
 }
 
