@@ -215,6 +215,12 @@ long long max_abs(samd_fmt f) { return f.is_signed ? (1LL << (f.bits - 1)) : ((1
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 constexpr int kMaxHaloRows = 1024;
+// A halo layer computes the whole virtual grid; a gather layer gathers and
+// widens every operand row once per tap instead. At 7x7 (1.31 grid positions
+// per output) the halo form is still the faster one: 3x3, 512 channels, u6 x
+// s2, batch 64: 58.8 -> 32.9 us; 14x14 (1.15), 512 channels, u4 x s4, batch
+// 16: 35.1 -> 22.4 us.
+constexpr double kMaxHaloWaste = 1.35;
 constexpr int kHaloGatherDepth = 2;  // packed staging slots of the halo producers (2..4)
 // minimum 128-pixel tiles per CTA of a launch (samd_conv2d_set_min_tiles_per_cta)
 std::atomic<int> g_min_tiles_per_cta{4};
@@ -222,7 +228,21 @@ std::atomic<int> g_min_tiles_per_cta{4};
 // Tiling, reduction order, operand type and exactness mode for one
 // convolution. fo.bits == 0 means no packed output. Returns SAMD_EUNSUP when
 // no mode keeps every accumulator below 2^24.
-samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, Plan &p, bool pool = false) {
+samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, Plan &p, bool pool = false,
+                      bool two_sided = false);
+
+// Fused 2x2 max-pool: the shapes it takes are those of a grid padded on both
+// sides (include/samd.h states them); the placement then follows the shared
+// padding like any other halo layer's.
+bool pool_plan_exists(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, int *hv) {
+  Plan q;
+  if (make_plan(d, fa, fw, fo, q, true, true) != SAMD_OK) return false;
+  *hv = q.hv;
+  return true;
+}
+
+samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, Plan &p, bool pool,
+                      bool two_sided) {
   p.La = lanes_per_word(fa);
   if (p.La == 0) return SAMD_EINVAL;
   const long long taps = static_cast<long long>(d->R) * d->S * d->C;
@@ -306,8 +326,14 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
     p.nchunks = p.nck * p.taps;
     p.Kpad = p.nchunks * BK;
   }
-  p.Hv = d->H + 2 * d->pad;
-  p.Wp = d->W + 2 * d->pad;
+  // The virtual grid shares its padding: the pad columns at the right end of
+  // a row are those at the left of the next row, and the pad rows below an
+  // image those above the next one (all zero), whenever the filter reaches
+  // no further than them (pad < S, pad < R). 14x14 images then waste 15% of
+  // the grid's positions instead of 31%, 7x7 ones 31% instead of 65%, and
+  // 56x56 ones 3.6% instead of 7.3%.
+  p.Hv = d->H + (d->pad < d->R && !two_sided ? d->pad : 2 * d->pad);
+  p.Wp = d->W + (d->pad < d->S && !two_sided ? d->pad : 2 * d->pad);
   const int nchunks_gather = p.nchunks;
   // One configuration: operand mode (halo or gather) and tile halves hv.
   // Returns false if it does not fit, or if `need_resident` and the weights
@@ -348,7 +374,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       const size_t halo_bytes = round_up(static_cast<size_t>(halo_rows) * p.row_bytes, 1024);
       const size_t stage_g = round_up(static_cast<size_t>(halo_rows) * srow, 16);
       const int ntiles_b = p.nck * p.taps;
-      if (halo_rows > kMaxHaloRows || waste > 1.16) return false;
+      if (halo_rows > kMaxHaloRows || waste > (two_sided ? 1.16 : kMaxHaloWaste)) return false;
       // The packed staging ring: with depth D the gathers run D - 1 items
       // ahead of the widening. Depth 2 is used: per-role timelines show the
       // halo producers finishing a tile's operands microseconds before its
@@ -446,9 +472,11 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   // halves or on residency, so the same prepared weights serve both forms).
   if (pool) {
     if (!p.halo) return SAMD_EUNSUP;
+    int hv_pool = 0;
+    if (!two_sided && !pool_plan_exists(d, fa, fw, fo, &hv_pool)) return SAMD_EUNSUP;
     placed = false;
     for (int hv = 2; hv >= 1 && !placed; --hv) {
-      if ((hv == 2 && !two) || 2 * p.Wp > BM * hv) continue;
+      if ((hv == 2 && !two) || 2 * p.Wp > BM * hv || (hv_pool && hv != hv_pool)) continue;
       for (int need_res = 1; need_res >= 0 && !placed; --need_res) placed = place(true, hv, need_res != 0);
     }
     if (!placed) return SAMD_EUNSUP;
@@ -496,7 +524,11 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       off_e = round_up(p.off_g + static_cast<size_t>(depth) * p.g_stride, 16);
       if (1024 + round_up(off_e + pool_bytes, 16) + bar_bytes(p.stages, p.hbufs) <= kBudget) break;
     }
-    if (depth < 2) return SAMD_EUNSUP;
+    if (depth < 2) {
+      // a smaller halo may have made room for more weights and left too
+      // little for the pool buffer: the placement that was found above fits
+      return two_sided ? SAMD_EUNSUP : make_plan(d, fa, fw, fo, p, true, true);
+    }
     p.pool = 1;
     p.gdepth = depth;
     p.grid_m = static_cast<long long>(d->N) * p.pool_tpi;

@@ -347,3 +347,15 @@ def test_conv_packed_only_last_64bit_word_is_whole(samd_lib, fo_bits, K):
     assert np.array_equal(got[:n], oracle_requant_pack(oracle_conv_nhwc(a_v, w_v, shape), shift, fo))
     assert (got[n:] == 0x5A5A5A5A5A5A5A5A).all()
     assert_status_clean()
+
+
+# Stride-1 layers share padding between neighbouring rows and images of the
+# position grid (pad < filter size); small images take the grid too.
+@pytest.mark.parametrize("shape", [samd.ConvShape(3, 24, 7, 7, 40), samd.ConvShape(2, 70, 14, 14, 24),
+                                   samd.ConvShape(2, 8, 14, 13, 16, R=5, S=5, pad=4), samd.ConvShape(3, 16, 9, 8, 16, R=3, S=3, pad=2),
+                                   samd.ConvShape(2, 16, 12, 11, 16, R=2, S=2, pad=1), samd.ConvShape(2, 16, 12, 11, 16, R=2, S=3, pad=2),
+                                   samd.ConvShape(2, 16, 20, 9, 300, R=3, S=3, pad=0)],
+                         ids=lambda v: f"{v.N}x{v.C}x{v.H}x{v.W}-K{v.K}r{v.R}s{v.S}p{v.pad}")
+@pytest.mark.parametrize("ba,sa", [(4, False), (6, True)])
+def test_conv_shared_padding(samd_lib, shape, ba, sa):
+    run_conv_check(shape, ba, sa, 3, True, fo_t=(ba, sa, 0, 32), seed=synth.seed_for("pad", shape, ba))

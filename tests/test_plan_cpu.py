@@ -32,3 +32,27 @@ def test_every_plan_fits_and_does_not_overlap():
                      "staged epilogue"):
             count = int(r.stdout.split(mode)[1].split()[0].strip("(),"))
             assert count > 0, (mode, r.stdout)
+
+
+@pytest.mark.parametrize("N,H,W,R,S,pad", [(2, 3, 4, 3, 3, 1), (3, 1, 1, 3, 3, 1), (2, 5, 4, 5, 5, 2), (2, 4, 3, 3, 3, 2),
+                                           (2, 4, 5, 2, 2, 1), (2, 4, 5, 3, 5, 1), (2, 6, 5, 3, 3, 0), (1, 3, 3, 5, 5, 4)])
+def test_shared_padding_grid_reads_what_two_sided_padding_reads(N, H, W, R, S, pad):
+    """The planner's virtual grid keeps pad columns on one side of a row and
+    pad rows on one side of an image (pad < R, S): the position one tap row or
+    column on always holds the input value that tap reads, or padding."""
+    assert pad < R and pad < S
+    Hv, Wp = H + pad, W + pad
+    Ho, Wo = H + 2 * pad - R + 1, W + 2 * pad - S + 1
+    assert Ho <= Hv and Wo <= Wp
+    for n in range(N):
+        for oh in range(Ho):
+            for ow in range(Wo):
+                for r in range(R):
+                    for s in range(S):
+                        ih, iw = oh + r - pad, ow + s - pad
+                        want = (n, ih, iw) if 0 <= ih < H and 0 <= iw < W else None
+                        v = (n * Hv + oh) * Wp + ow + r * Wp + s
+                        img, rem = divmod(v, Hv * Wp)
+                        gh, gw = rem // Wp - pad, rem % Wp - pad
+                        got = (img, gh, gw) if img < N and 0 <= gh < H and 0 <= gw < W else None
+                        assert got == want
