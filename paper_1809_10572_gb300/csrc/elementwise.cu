@@ -17,8 +17,7 @@
 // lane's carry or borrow from its first spacer bit; the other ops use the
 // temporary-spacer forms with masks over the spacer-separated fields.
 //
-// Requantize into another format takes the per-lane path: one thread per
-// output word, bit-field extract, integer op, clamp, insert.
+// Requantize into another format is in requant.cu.
 #include "samd_internal.cuh"
 
 namespace samd {
@@ -238,44 +237,6 @@ __global__ void __launch_bounds__(kThreads)
     W x = a[w];
     W y = kBinary ? b[w] : x;
     out[w] = apply_op<W, BITS, OP>(x, y, is_signed, sat, shift, keep);
-  }
-}
-
-// Per-lane path: any spacer, any output format. One thread per output word.
-struct LaneFmt {
-  int bits, is_signed, lane_w, L;
-};
-
-template <typename WI, typename WO>
-__global__ void __launch_bounds__(kThreads)
-    ew_lane_kernel(int op, LaneFmt fa, const WI *__restrict__ a, const WI *__restrict__ b, LaneFmt fo,
-                   WO *__restrict__ out, int64_t n, int64_t nwords_out, int shift, int sat) {
-  const uint32_t ma = (1u << fa.bits) - 1, mo = (1u << fo.bits) - 1;
-  const int lo = lane_lo(fo.bits, fo.is_signed), hi = lane_hi(fo.bits, fo.is_signed);
-  for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nwords_out;
-       w += (int64_t)gridDim.x * blockDim.x) {
-    WO word = 0;
-    for (int l = 0; l < fo.L; ++l) {
-      int64_t e = w * fo.L + l;
-      if (e >= n) break;
-      int64_t wi = e / fa.L;
-      int li = static_cast<int>(e - wi * fa.L);
-      int x = lane_value(static_cast<uint32_t>(a[wi] >> (li * fa.lane_w)) & ma, fa.bits, fa.is_signed);
-      int y = 0;
-      if (op == SAMD_ADD || op == SAMD_SUB || op == SAMD_MUL)
-        y = lane_value(static_cast<uint32_t>(b[wi] >> (li * fa.lane_w)) & ma, fa.bits, fa.is_signed);
-      int v;
-      switch (op) {
-        case SAMD_ADD: v = x + y; break;
-        case SAMD_SUB: v = x - y; break;
-        case SAMD_MUL: v = x * y; break;
-        case SAMD_RELU: v = x < 0 ? 0 : x; break;
-        default: v = x >> shift; break;  // arithmetic shift: floor(x / 2^shift)
-      }
-      if (op == SAMD_REQUANT || sat) v = clamp_int(v, lo, hi);
-      word |= WO(static_cast<uint32_t>(v) & mo) << (l * fo.lane_w);
-    }
-    out[w] = word;
   }
 }
 
@@ -518,21 +479,6 @@ cudaError_t swar_dispatch(samd_op op, int bits, const void *a, const void *b, vo
   }
 }
 
-LaneFmt lane_fmt(samd_fmt f) {
-  return LaneFmt{f.bits, f.is_signed, f.bits + f.spacer, lanes_per_word(f)};
-}
-
-template <typename WI, typename WO>
-cudaError_t lane_dispatch(samd_op op, samd_fmt fa, const void *a, const void *b, samd_fmt fo, void *out, int64_t n,
-                          int shift, int sat, cudaStream_t s) {
-  int64_t nwo = words_per_row(fo, n);
-  int grid = grid_for(nwo, kThreads, sm_count() * 16);
-  ew_lane_kernel<WI, WO><<<grid, kThreads, 0, s>>>(static_cast<int>(op), lane_fmt(fa), static_cast<const WI *>(a),
-                                                   static_cast<const WI *>(b), lane_fmt(fo), static_cast<WO *>(out),
-                                                   n, nwo, shift, sat);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 cudaError_t launch_elementwise(samd_op op, samd_fmt fa, const void *a, const void *b, samd_fmt fo, void *out,
@@ -548,13 +494,7 @@ cudaError_t launch_elementwise(samd_op op, samd_fmt fa, const void *a, const voi
       return swar_dispatch<uint32_t>(op, fa.bits, a, b, out, nwords, fa.is_signed, saturate, shift, s);
     return swar_dispatch<uint64_t>(op, fa.bits, a, b, out, nwords, fa.is_signed, saturate, shift, s);
   }
-  if (fa.word_bits == 32 && fo.word_bits == 32)
-    return lane_dispatch<uint32_t, uint32_t>(op, fa, a, b, fo, out, n, shift, saturate, s);
-  if (fa.word_bits == 32)
-    return lane_dispatch<uint32_t, uint64_t>(op, fa, a, b, fo, out, n, shift, saturate, s);
-  if (fo.word_bits == 32)
-    return lane_dispatch<uint64_t, uint32_t>(op, fa, a, b, fo, out, n, shift, saturate, s);
-  return lane_dispatch<uint64_t, uint64_t>(op, fa, a, b, fo, out, n, shift, saturate, s);
+  return launch_requant(fa, a, fo, out, n, shift, s);  // the one op that may change the format
 }
 
 }  // namespace samd

@@ -174,6 +174,7 @@ cudaError_t launch_pack(samd_fmt f, const int8_t *src, void *dst, int64_t rows, 
 cudaError_t launch_unpack(samd_fmt f, const void *src, int8_t *dst, int64_t rows, int64_t inner, cudaStream_t s);
 cudaError_t launch_elementwise(samd_op op, samd_fmt fa, const void *a, const void *b, samd_fmt fo, void *out,
                                int64_t n, int shift, int saturate, cudaStream_t s);
+cudaError_t launch_requant(samd_fmt fa, const void *a, samd_fmt fo, void *out, int64_t n, int shift, cudaStream_t s);
 cudaError_t launch_maxpool2x2_nhwc(samd_fmt f, const void *in, void *out, int N, int C, int H, int W,
                                    cudaStream_t s);
 

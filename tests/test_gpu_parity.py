@@ -359,3 +359,27 @@ def test_conv_packed_only_last_64bit_word_is_whole(samd_lib, fo_bits, K):
 @pytest.mark.parametrize("ba,sa", [(4, False), (6, True)])
 def test_conv_shared_padding(samd_lib, shape, ba, sa):
     run_conv_check(shape, ba, sa, 3, True, fo_t=(ba, sa, 0, 32), seed=synth.seed_for("pad", shape, ba))
+
+
+# Requantize between formats: sizes around one period of the two lane grids
+# (4 times the least common multiple of their lanes, or once), guard words
+# after the output, shifts up to past the lane width.
+@pytest.mark.parametrize("word_bits", (32, 64))
+@pytest.mark.parametrize("bits_o", BITS)
+@pytest.mark.parametrize("bits", BITS)
+def test_requant_format_change_periods(samd_lib, bits, bits_o, word_bits):
+    for (signed, signed_o), shift in zip(itertools.product(SIGNS, SIGNS), (0, 1, bits, 31)):
+        fa, fo = samd.fmt(bits, signed, 0, word_bits), samd.fmt(bits_o, signed_o, 0, word_bits)
+        if samd.samd_lanes_per_word(fa) == samd.samd_lanes_per_word(fo) and signed == signed_o:
+            continue
+        for n in (1, 31, 127, 128, 129, 160, 161, 32 * 641 + 3):
+            xv, xb = values_and_bytes(synth.seed_for("rqp", bits, bits_o, signed, signed_o, n), (n,), bits, signed)
+            xw = gpu_pack(xb, fa, 1, n)
+            nw = samd.samd_packed_words(fo, 1, n)
+            out = torch.full((nw + 4,), 0x5A5A5A5A, dtype=samd.word_dtype(fo), device="cuda")
+            samd.samd_elementwise("requant", fa, xw, None, fo, out, n, shift, 0)
+            got = np_words(out, word_bits)
+            want = oracle.pack(oracle.requant(xv, shift, bits_o, signed_o)[None], bits_o, signed_o, 0, word_bits)
+            assert np.array_equal(got[:nw], want), (signed, signed_o, shift, n)
+            assert (got[nw:] == 0x5A5A5A5A).all()
+    assert_status_clean()
