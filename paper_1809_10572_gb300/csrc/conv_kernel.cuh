@@ -122,23 +122,6 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t c) {
   return d;
 }
 
-// n / d for 0 <= n < 2^31 by one multiply-high, an add and a shift:
-// l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1, q = (umulhi(m, n) + n) >> l.
-struct FastDiv {
-  uint32_t m;
-  int l;
-  uint32_t d;
-};
-
-inline FastDiv make_fastdiv(uint32_t d) {
-  int l = 0;
-  while ((uint64_t(1) << l) < d) ++l;
-  const uint64_t m = ((uint64_t(1) << 32) * ((uint64_t(1) << l) - d)) / d + 1;
-  return FastDiv{static_cast<uint32_t>(m), l, d};
-}
-
-__device__ __forceinline__ uint32_t fdiv(uint32_t n, const FastDiv &f) { return (__umulhi(f.m, n) + n) >> f.l; }
-
 struct ConvArgs {
   const void *act;
   int32_t *acc_out;
