@@ -201,6 +201,7 @@ struct Plan {
   int gdepth;  // HALO: packed staging slots (items gathered gdepth - 1 ahead of the widening)
   int hbufs;   // HALO: widened halo buffers (2 or 3)
   int e_stage; // kEpiStageBytes at off_e stage the epilogue's 3/5/6-bit packed rows
+  int e_flat;  // ConvArgs::e_flat
   int pool, pool_rows, pool_nw, pool_pitch, pool_tpi;  // fused 2x2 max-pool (ConvArgs::pool)
   long long M;
   long long bound;  // R*S*C * max|a| * max|w|: no accumulator exceeds it
@@ -214,7 +215,6 @@ long long max_abs(samd_fmt f) { return f.is_signed ? (1LL << (f.bits - 1)) : ((1
 
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-constexpr int kMaxHaloRows = 1024;
 // A halo layer computes the whole virtual grid; a gather layer gathers and
 // widens every operand row once per tap instead. At 7x7 (1.31 grid positions
 // per output) the halo form is still the faster one: 3x3, 512 channels, u6 x
@@ -230,6 +230,13 @@ std::atomic<int> g_min_tiles_per_cta{4};
 // no mode keeps every accumulator below 2^24.
 samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, Plan &p, bool pool = false,
                       bool two_sided = false);
+
+// Words between two staged rows of a pooled tile: the row's words of its
+// channel block, made odd (outputs of 1, 2, 4 or 8 bits in 32-bit words).
+int pool_pitch(int NBc, samd_fmt fo) {
+  const int Lo = lanes_per_word(fo);
+  return Lo > 0 ? ((NBc + Lo - 1) / Lo) | 1 : 1;
+}
 
 // Fused 2x2 max-pool: the shapes it takes are those of a grid padded on both
 // sides (include/samd.h states them); the placement then follows the shared
@@ -481,19 +488,39 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
     }
     if (!placed) return SAMD_EUNSUP;
   }
-  // 3-, 5- and 6-bit packed outputs (32-bit words, no spacer) stage their
-  // rows in shared memory when a channel block's row holds at least one
-  // whole packing period (lcm(32, L) channels: 160 for L = 5 or 10, 96 for
-  // L = 6) and the buffer fits beside the placement chosen above (which it
-  // never changes), so that stores are contiguous within a row. Shorter rows
-  // (64 channels: 7 to 13 words) measured faster stored directly.
-  p.e_stage = 0;
-  const int period_ch = fo.bits == 5 ? 96 : 160;
-  if ((fo.bits == 3 || fo.bits == 5 || fo.bits == 6) && fo.spacer == 0 && fo.word_bits == 32 &&
-      p.NBc >= period_ch && p.smem_bytes + round_up(kEpiStageBytes, 16) <= kBudget) {
-    p.e_stage = 1;
-    p.off_bar = static_cast<uint32_t>(round_up(p.off_e + kEpiStageBytes, 16));
-    p.smem_bytes = 1024 + p.off_bar + bar_bytes(p.stages, p.halo ? p.hbufs : p.stages_a);
+  // 3-, 5- and 6-bit packed outputs (32-bit words, no spacer) are staged in
+  // shared memory where the buffer fits beside the placement chosen above: a
+  // warp's 32 whole rows when one channel block holds them (a gather layer
+  // gives up A tiles in flight, down to two, to make room), else 32 words of
+  // each row at a time when a block's row holds at least 96 (5 bits) or 160
+  // channels; shorter parts of rows measured faster stored directly.
+  p.e_stage = p.e_flat = 0;
+  if ((fo.bits == 3 || fo.bits == 5 || fo.bits == 6) && fo.spacer == 0 && fo.word_bits == 32 && !pool) {
+    auto fits = [&](size_t bytes) { return p.smem_bytes + round_up(bytes, 16) <= kBudget; };
+    auto reserve = [&](size_t bytes) {
+      p.off_bar = static_cast<uint32_t>(round_up(p.off_e + bytes, 16));
+      p.smem_bytes = 1024 + p.off_bar + bar_bytes(p.stages, p.halo ? p.hbufs : p.stages_a);
+    };
+    const int Lo = lanes_per_word(fo);
+    const size_t flat_bytes = static_cast<size_t>(kEpiWarps) * 32 * 4 * ((d->K + Lo - 1) / Lo);
+    if (p.nblocks == 1) {
+      const Plan whole = p;
+      while (!fits(flat_bytes) && !p.halo && p.stages_a > 2) {
+        // one A tile less moves everything behind the A tiles down
+        --p.stages_a;
+        finish(p.stages_a * static_cast<size_t>(p.op_stride), 2 * static_cast<size_t>(p.g_stride), p.stages_a);
+      }
+      if (fits(flat_bytes)) {
+        p.e_flat = 1;
+        reserve(flat_bytes);
+      } else {
+        p = whole;
+      }
+    }
+    if (!p.e_flat && p.NBc >= (fo.bits == 5 ? 96 : 160) && fits(kEpiStageBytes)) {
+      p.e_stage = 1;
+      reserve(kEpiStageBytes);
+    }
   }
   // Fused 2x2 max-pool (placed above): even output sizes, outputs of 1, 2, 4
   // or 8 bits in 32-bit words. A tile is q = 128 hv / (2 Wp) row pairs of
@@ -509,13 +536,11 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       return SAMD_EUNSUP;
     int q = (BM * p.hv) / (2 * p.Wp);
     if (q > Ho / 2) q = Ho / 2;
-    const int Lo = 32 / fo.bits;
     p.pool_rows = 2 * q;
     p.pool_tpi = (Ho / 2 + q - 1) / q;
-    p.pool_nw = (p.NBc + Lo - 1) / Lo;
-    p.pool_pitch = p.pool_nw | 1;
+    p.pool_nw = (p.NBc + 32 / fo.bits - 1) / (32 / fo.bits);
+    p.pool_pitch = pool_pitch(p.NBc, fo);
     const size_t pool_bytes = static_cast<size_t>(2 * BM) * p.pool_pitch * 4;
-    if (p.e_stage) return SAMD_EUNSUP;  // not reached: e_stage is for 3/5/6-bit outputs
     // the buffer goes after the packed staging ring, made shallower if need
     // be (the ring's depth does not change the weight layout)
     int depth = p.gdepth;
@@ -556,7 +581,7 @@ bool layout_ok(const Plan &p) {
          p.off_e <= p.off_bar && 1023 + p.off_bar + bars <= p.smem_bytes && p.op_stride % 1024 == 0 &&
          p.off_b % 1024 == 0 && p.b_bytes % 1024 == 0 && p.off_bar % 8 == 0 && 2 * p.hv * p.mma_n <= 512 &&
          (p.hv == 1 || p.hv == 2 || (p.hv == 4 && p.halo && p.fp8 && p.mma_n <= 64)) && (!p.halo || (p.gdepth >= 2 && p.gdepth <= 4 && (p.hbufs == 2 || p.hbufs == 3))) &&
-         (!p.e_stage || p.off_e + kEpiStageBytes <= p.off_bar) &&
+         (!p.e_stage || p.off_e + kEpiStageBytes <= p.off_bar) && !(p.e_stage && p.e_flat) && (!p.e_flat || p.nblocks == 1) &&
          (!p.pool || (p.halo && 2 * p.Wp <= BM * p.hv && !p.e_stage && p.pool_pitch >= p.pool_nw &&
                       p.off_e + static_cast<size_t>(2 * BM) * p.pool_pitch * 4 <= p.off_bar));
 }
@@ -757,7 +782,8 @@ samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const 
     a.out_fast = fast ? Lo : 0;
   }
   a.shift = shift;
-  a.out_scale = ldexpf(1.0f, -shift);
+  a.acc_scale = 1.0f;
+  a.out_scale = ldexpf(a.acc_scale, -shift);
   a.fast_req = (!p.split && (p.bound >> shift) < (1LL << 22)) ? 1 : 0;
   a.fast_acc = (!p.split && p.bound < (1LL << 22)) ? 1 : 0;
   a.Hv = p.Hv;
@@ -790,6 +816,7 @@ samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const 
   a.hbufs = p.hbufs;
   a.off_e = p.off_e;
   a.e_stage = p.e_stage;
+  a.e_flat = p.e_flat;
   a.pool = p.pool;
   a.pool_rows = p.pool ? p.pool_rows : 0;
   a.pool_nw = p.pool ? p.pool_nw : 0;

@@ -46,11 +46,12 @@ constexpr int kGatherDepth = 4;                    // packed chunks in flight pe
 constexpr int kProdWarps = 8;                      // operand producers
 constexpr int kEpiWarps = 8;                       // epilogue
 constexpr int kProdThreads = 32 * kProdWarps;
+constexpr int kMaxHaloRows = 1024;                 // of one tile (kMaxHaloRows / kProdThreads rows per producer thread)
 constexpr int kThreads = 32 * (2 + kProdWarps + kEpiWarps);
 constexpr int kFirstEpiWarp = 2 + kProdWarps;
-// Optional epilogue staging (ConvArgs::e_stage): per epilogue warp 32 rows of
-// one packing period (at most 32 words), rows kEpiPitch words apart (odd, so
-// that 32 lanes writing one word of their own rows hit 32 banks).
+// Optional epilogue staging (ConvArgs::e_stage): per epilogue warp 32 words of
+// 32 rows, kEpiPitch words apart (odd, so that 32 lanes writing one word of
+// their own rows hit 32 banks).
 constexpr int kEpiPitch = 33;
 constexpr uint32_t kEpiStageBytes = kEpiWarps * 32 * kEpiPitch * 4;
 
@@ -150,7 +151,8 @@ struct ConvArgs {
   int out_bits, out_signed, out_lane_w, out_L, out_word64, out_wpr;
   int out_fast;     // output lanes per word when they divide 32 (whole words per 32 channels), else 0
   int shift;
-  float out_scale;  // 2^-shift
+  float acc_scale;  // an accumulator times acc_scale is its integer sum (2^op_exp)
+  float out_scale;  // acc_scale * 2^-shift
   int fast_req;     // |acc| / 2^shift < 2^22: requantize through floor_scaled_biased
   int fast_acc;     // |acc| < 2^22: int32 outputs through floor_scaled_biased
   // HALO (stride 1): virtual output grid of N x Hv x Wp positions. A tile of
@@ -171,7 +173,8 @@ struct ConvArgs {
   // shared memory carve-up (bytes from the 1024-byte-aligned base)
   uint32_t op_stride;  // one halo buffer or one A tile
   uint32_t off_b, b_bytes, off_g, g_stride, off_e, off_bar;
-  int e_stage;  // 1: kEpiStageBytes at off_e stage the 3/5/6-bit packed rows (epilogue_row_period_staged)
+  int e_stage;  // 1: kEpiStageBytes at off_e stage 32 words of each 3/5/6-bit packed row (epilogue_row_words)
+  int e_flat;   // 1: 32 whole rows per epilogue warp at off_e instead (one channel block)
   // Fused 2x2 max-pool (pool = 1; halo layers): tile mt is pool_rows output
   // rows (pool_rows / 2 row pairs) of one image from an even row on, at
   // virtual position img * Hv * Wp + g * pool_rows * Wp (img = mt / tiles
@@ -550,39 +553,66 @@ struct RowPacker {
   }
 };
 
-// Epilogue of one accumulator row (one output pixel m) of channel block nb:
-// fp32 accumulators -> exact integers -> optional int32 store, optional
-// requantize-and-pack. Called by whole warps (tcgen05.ld is collective; rows
-// outside the output only skip the stores).
+// One requantized lane as an offset pattern: clamp_fo(floor(acc / 2^shift))
+// plus half the range of a signed format (0 for an unsigned one), by one fma
+// and one add-clamp: `addend` takes the fma's bias off and adds the offset,
+// min with the largest pattern, relu for the smallest. Flipping the top bits
+// of a word's signed lanes then gives their two's complement.
+__device__ __forceinline__ uint32_t requant_lane(uint32_t acc, float scale, int32_t addend, int32_t omax) {
+  return static_cast<uint32_t>(__viaddmin_s32_relu(floor_scaled_biased(__uint_as_float(acc), scale), addend, omax));
+}
+__device__ __forceinline__ constexpr int32_t requant_addend(int bits, bool is_signed) {
+  return (is_signed ? 1 << (bits - 1) : 0) - kMagicBits;
+}
+
+// What the epilogue of a row works on: rows are output pixels (m; ~0 for a
+// row outside the output, which only skips the stores), nvalid the channels
+// of this block from ch0 on. The first, store-free pass asks for one column
+// group only (warm).
+struct EpiRow {
+  uint32_t taddr;   // TMEM address of the warp's rows, first column
+  uint32_t m;
+  int ch0, nvalid;
+  __device__ __forceinline__ bool valid() const { return m != ~0u; }
+};
+__device__ __forceinline__ EpiRow epi_row(const ConvArgs &args, uint32_t taddr, uint32_t m, int nb, bool warm) {
+  EpiRow e{taddr, m, nb * args.NBc, 0};
+  e.nvalid = args.K - e.ch0 < args.NBc ? args.K - e.ch0 : args.NBc;
+  if (warm) {
+    e.m = ~0u;
+    e.nvalid = 1;
+  }
+  return e;
+}
+
+// Epilogue of one accumulator row of a channel block: fp32 accumulators ->
+// exact integers -> optional int32 store, optional requantize-and-pack.
+// Called by whole warps (tcgen05.ld is collective).
 //
-// The common case (packed output only, no split digits, |acc| / 2^shift <
-// 2^22) requantizes each accumulator with one fma in place.
+// Formats with spacers or 64-bit words of 3, 5, 6 or 7 bits: packed output
+// only, no split digits, |acc| / 2^shift < 2^22.
 template <typename WO>
-__device__ __forceinline__ void epilogue_row_fast(const ConvArgs &args, uint32_t taddr, bool row_valid, long long m,
-                                                  int nb) {
-  const int ch0 = nb * args.NBc;
-  const int nvalid = args.K - ch0 < args.NBc ? args.K - ch0 : args.NBc;
-  const int lo = lane_lo(args.out_bits, args.out_signed), hi = lane_hi(args.out_bits, args.out_signed);
-  const int32_t blo = kMagicBits + lo, bhi = kMagicBits + hi;
-  const uint32_t omask = (1u << args.out_bits) - 1;
+__device__ __forceinline__ void epilogue_row_fast(const ConvArgs &args, const EpiRow &e) {
+  const int32_t addend = requant_addend(args.out_bits, args.out_signed != 0), omax = (1 << args.out_bits) - 1;
+  const uint32_t flip = args.out_signed ? 1u << (args.out_bits - 1) : 0u;
   const float scale = args.out_scale;
   const int L = args.out_L, lw = args.out_lane_w;
   RowPacker<WO> pk;
-  pk.dst = static_cast<WO *>(args.packed_out) + (m * args.out_wpr + ch0 / L);
-  for (int col = 0; col < nvalid; col += 32) {
+  WO *const row = static_cast<WO *>(args.packed_out) + (static_cast<long long>(e.m) * args.out_wpr + e.ch0 / L);
+  pk.dst = row;
+  for (int col = 0; col < e.nvalid; col += 32) {
     uint32_t y[32];
-    ptx::tmem_ld_32x32b_x32(taddr + col, y);
-    ptx::tmem_wait_ld();
-    const int cnt = nvalid - col < 32 ? nvalid - col : 32;
+    ptx::tmem_ld_32x32b_x32(e.taddr + col, y);
+    ptx::tmem_wait_ld(y);
+    const int cnt = e.nvalid - col < 32 ? e.nvalid - col : 32;
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
-      int32_t t = floor_scaled_biased(__uint_as_float(y[k]), scale);
-      t = t < blo ? blo : (t > bhi ? bhi : t);
-      y[k] = k < cnt ? static_cast<uint32_t>(t) & omask : 0u;
+      y[k] = requant_lane(y[k], scale, addend, omax) ^ flip;
+      if (k >= cnt) y[k] = 0u;
     }
-    if (!row_valid) continue;
+    if (!e.valid()) continue;
     if (args.out_fast) {  // L divides 32: whole words per 32-channel group
-      WO *dst = static_cast<WO *>(args.packed_out) + (m * args.out_wpr + (ch0 + col) / L);
+      WO *dst = row + col / L;
       switch (args.out_fast) {
         case 4:
           if constexpr (sizeof(WO) == 4) pack_regs<4>(y, lw, cnt, dst);
@@ -597,73 +627,69 @@ __device__ __forceinline__ void epilogue_row_fast(const ConvArgs &args, uint32_t
         if (k < cnt) pk.put(y[k], L, lw);
     }
   }
-  if (!args.out_fast && row_valid) pk.flush();
+  if (!args.out_fast && e.valid()) pk.flush();
 }
 
 // The fast epilogue for output lanes of OB = 1, 2, 4, 7 or 8 bits without
 // spacers (7 only in 32-bit words): the words of a 32-channel group are built
 // 32 bits at a time (for OB dividing 32 a 64-bit word is its two 32-bit
 // halves, low half first, so the bytes are the same) with compile-time
-// shifts. Unsigned lanes are summed in the
-// biased domain and the bias sum is removed once per word; signed lanes are
-// masked to their two's complement bits first.
+// shifts: three operations a lane.
 template <int OB, bool OS>
-__device__ __forceinline__ void epilogue_row_spec(const ConvArgs &args, uint32_t taddr, bool row_valid, long long m,
-                                                  int nb) {
+__device__ __forceinline__ void epilogue_row_spec(const ConvArgs &args, const EpiRow &e) {
   constexpr int LH = 32 / OB;  // lanes per 32-bit half-word (a divisor of 32: OB = 1, 2, 4, 7, 8)
   constexpr int NH = 32 / LH;  // half-words per 32-channel group
   static_assert(32 % LH == 0, "whole half-words per 32-channel group");
-  constexpr int32_t lo = OS ? -(1 << (OB - 1)) : 0, hi = OS ? (1 << (OB - 1)) - 1 : (1 << OB) - 1;
-  constexpr int32_t blo = kMagicBits + lo, bhi = kMagicBits + hi;
-  constexpr uint32_t omask = (1u << OB) - 1;
-  constexpr uint32_t bias_sum = [] {
-    uint32_t b = 0;
-    for (int l = 0; l < LH; ++l) b += static_cast<uint32_t>(kMagicBits) << (l * OB);
-    return b;
-  }();
-  const int ch0 = nb * args.NBc;
-  const int nvalid = args.K - ch0 < args.NBc ? args.K - ch0 : args.NBc;
+  constexpr int32_t addend = requant_addend(OB, OS), omax = (1 << OB) - 1;
+  constexpr uint32_t flip = OS ? LaneMsb<uint32_t, OB>::kValue : 0u;
   const float scale = args.out_scale;
   // 32-bit half-words of this row: output channel c sits in half-word c / LH
   uint32_t *row32 = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(args.packed_out) +
-                                                 static_cast<size_t>(m) * args.out_wpr * (args.out_word64 ? 8 : 4)) +
-                    ch0 / LH;
+                                                 static_cast<size_t>(e.m) * args.out_wpr * (args.out_word64 ? 8 : 4)) +
+                    e.ch0 / LH;
   // 4-bit lanes: two 32-channel groups make one 32-byte store (a warp's
   // 32-byte rows then cover whole 128-byte lines, in the L1 data path the
   // MMAs' operand reads share)
-  const bool pair32 = NH == 4 && nvalid % 64 == 0 && (reinterpret_cast<uintptr_t>(row32) & 31) == 0;
+  const bool pair32 = NH == 4 && e.nvalid % 64 == 0 && (reinterpret_cast<uintptr_t>(row32) & 31) == 0;
   uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-  for (int col = 0; col < nvalid; col += 32) {
-    uint32_t r[32];
-    ptx::tmem_ld_32x32b_x32(taddr + col, r);
-    ptx::tmem_wait_ld();
-    const int cnt = nvalid - col < 32 ? nvalid - col : 32;
+  // 16 columns are packed while the next 16 are on their way (the block's MMA
+  // columns are a multiple of 16; past them the first ones are read again)
+  uint32_t ra[16], rb[16];
+  auto load = [&](int col, uint32_t (&r)[16]) {
+    ptx::tmem_ld_32x32b_x16(e.taddr + (col < args.n_mma ? col : 0), r);
+  };
+  load(0, ra);
+  ptx::tmem_wait_ld(ra);
+  for (int col = 0; col < e.nvalid; col += 32) {
+    const int cnt = e.nvalid - col < 32 ? e.nvalid - col : 32;
     uint32_t h[NH];
+    auto half = [&](const uint32_t (&r)[16], auto first) {  // columns first .. first + 15 of the group
 #pragma unroll
-    for (int j = 0; j < NH; ++j) {
-      uint32_t w = 0;
-#pragma unroll
-      for (int l = 0; l < LH; ++l) {
-        int32_t t = floor_scaled_biased(__uint_as_float(r[j * LH + l]), scale);
-        t = t < blo ? blo : (t > bhi ? bhi : t);
-        if constexpr (OS)
-          w |= (static_cast<uint32_t>(t) & omask) << (l * OB);
-        else
-          w += static_cast<uint32_t>(t) << (l * OB);
+      for (int k = 0; k < 16; ++k) {
+        const int c = decltype(first)::value + k;
+        const uint32_t v = requant_lane(r[k], scale, addend, omax) << ((c % LH) * OB);
+        h[c / LH] = c % LH == 0 ? v : h[c / LH] + v;
       }
-      h[j] = OS ? w : w - bias_sum;
-    }
+    };
+    load(col + 16, rb);
+    half(ra, std::integral_constant<int, 0>{});
+    ptx::tmem_wait_ld(rb);
+    load(col + 32, ra);
+    half(rb, std::integral_constant<int, 16>{});
+#pragma unroll
+    for (int j = 0; j < NH; ++j) h[j] ^= flip;
+    ptx::tmem_wait_ld(ra);
     if constexpr (NH == 4) {
       if (pair32) {
         if ((col & 32) == 0) {
           p0 = h[0], p1 = h[1], p2 = h[2], p3 = h[3];
-        } else if (row_valid) {
+        } else if (e.valid()) {
           ptx::st_global_v8(row32 + (col - 32) / LH, p0, p1, p2, p3, h[0], h[1], h[2], h[3]);
         }
         continue;
       }
     }
-    if (!row_valid) continue;
+    if (!e.valid()) continue;
     uint32_t *dst = row32 + col / LH;
     if (cnt < 32) {  // the last group of a channel count that is not a multiple of 32
 #pragma unroll
@@ -704,129 +730,109 @@ __device__ __forceinline__ void epilogue_row_spec(const ConvArgs &args, uint32_t
     }
   }
   // a last 64-bit word of which only the low half-word holds channels
-  const int nhalf = (nvalid + LH - 1) / LH;
-  if (args.out_word64 && (nhalf & 1) && row_valid) row32[nhalf] = 0u;
+  const int nhalf = (e.nvalid + LH - 1) / LH;
+  if (args.out_word64 && (nhalf & 1) && e.valid()) row32[nhalf] = 0u;
 }
-
-__host__ __device__ constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }
 
 // The fast epilogue for 32-bit output words whose L = 32 / OB lanes do not
-// divide 32 (OB = 3, 5, 6: L = 10, 6, 5). Word boundaries repeat every
-// lcm(32, L) channels, so one such period (G groups of 32 columns) is
-// unrolled and every lane's word and shift are compile-time. Lanes past the
-// last channel read the biased zero, so a final partial word is zero-filled.
+// divide 32 (OB = 3, 5, 6: L = 10, 6, 5): two or four words (20 or 24 columns)
+// at a time, the next ones' columns on their way meanwhile, loaded in pieces that never reach past the block's MMA columns.
+// The loop's body is small on purpose: unrolled over the 160 or 96 columns
+// after which word boundaries repeat on a 32-column grid, the two or so warps
+// of a scheduler spent most of their time fetching it (2700 instructions a
+// row of 256 6-bit channels at 0.2 a cycle).
+//
+// Rows leave in one of three ways. Flat (e_flat: one channel block): the
+// warp's valid rows are consecutive output pixels, so their words are one
+// contiguous run; they are staged side by side and copied with 16-byte
+// accesses. By rows (e_stage): 32 words of each row are staged at a time and
+// written row by row. Else each thread stores its own row's words.
 template <int OB, bool OS>
-__device__ __forceinline__ void epilogue_row_period(const ConvArgs &args, uint32_t taddr, bool row_valid,
-                                                    long long m, int nb) {
+__device__ __forceinline__ void epilogue_row_words(const ConvArgs &args, const EpiRow &e, uint32_t *stg) {
   constexpr int L = 32 / OB;
-  constexpr int G = L / gcd_c(32, L);  // lcm(32, L) / 32
-  constexpr int32_t lo = OS ? -(1 << (OB - 1)) : 0, hi = OS ? (1 << (OB - 1)) - 1 : (1 << OB) - 1;
-  constexpr int32_t blo = kMagicBits + lo, bhi = kMagicBits + hi;
-  constexpr uint32_t omask = (1u << OB) - 1;  // the low bits of kMagicBits + y are those of y
-  const int ch0 = nb * args.NBc;
-  const int nvalid = args.K - ch0 < args.NBc ? args.K - ch0 : args.NBc;
-  const float scale = args.out_scale;
-  uint32_t *dst = static_cast<uint32_t *>(args.packed_out) + (m * args.out_wpr + ch0 / L);
-  // The last 32-column group may run past the block's channels: its lanes
-  // read the biased zero, and words that lie wholly past the last channel
-  // belong to the next row, so only the block's words are stored.
-  int wleft = (nvalid + L - 1) / L;
-  for (int c0 = 0; c0 < nvalid; c0 += 32 * G) {
-    uint32_t cur = 0;
-    bool open = false;
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const int col = c0 + 32 * g;
-      if (col >= nvalid) break;
-      uint32_t r[32];
-      ptx::tmem_ld_32x32b_x32(taddr + col, r);
-      ptx::tmem_wait_ld();
-#pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const int q = 32 * g + k;  // channel within the period (compile-time after unrolling)
-        const int l = q % L;
-        int32_t t = floor_scaled_biased(__uint_as_float(r[k]), scale);
-        t = t < blo ? blo : (t > bhi ? bhi : t);
-        if (col + k >= nvalid) t = kMagicBits;
-        cur |= (static_cast<uint32_t>(t) & omask) << (l * OB);
-        open = true;
-        if (l == L - 1) {
-          if (row_valid && wleft > 0) *dst = cur;
-          ++dst;
-          --wleft;
-          cur = 0;
-          open = false;
-        }
-      }
-    }
-    if (open && row_valid && wleft > 0) *dst = cur;  // the row's last, partial word
-  }
-}
-
-// epilogue_row_period with the stores staged: a warp's 32 rows of one
-// period (PW = lcm(32, L) / L words per row, 16 or 32) go to the warp's
-// shared-memory area first, and the warp then writes them out row by row,
-// PW consecutive words of 32 / PW rows per store instruction, instead of
-// every thread storing its own row one word at a time (32 rows, 32 sectors,
-// per instruction). Every word of a period is computed (channels past the
-// block's last read as the biased zero; 32-column groups wholly past it are
-// skipped), and only the block's words are stored.
-template <int OB, bool OS>
-__device__ __forceinline__ void epilogue_row_period_staged(const ConvArgs &args, uint32_t taddr, bool row_valid,
-                                                           long long m, int nb, uint32_t *stg) {
-  constexpr int L = 32 / OB;
-  constexpr int G = L / gcd_c(32, L);  // lcm(32, L) / 32
-  constexpr int PW = 32 * G / L;       // words per row and period
-  constexpr int RPI = 32 / PW;         // rows per store instruction
-  static_assert(PW * RPI == 32, "a period is 16 or 32 words");
-  constexpr int32_t lo = OS ? -(1 << (OB - 1)) : 0, hi = OS ? (1 << (OB - 1)) - 1 : (1 << OB) - 1;
-  constexpr int32_t blo = kMagicBits + lo, bhi = kMagicBits + hi;
-  constexpr uint32_t omask = (1u << OB) - 1;
+  constexpr int kWords = L == 10 ? 2 : 4;      // words of a group
+  constexpr int kCols = kWords * L;            // 20 or 24 columns
+  constexpr int kPiece = L == 6 ? 8 : 4;       // columns of one TMEM load; divides 16, as the block's MMA columns are
+  constexpr int32_t addend = requant_addend(OB, OS), omax = (1 << OB) - 1;
+  constexpr uint32_t flip = OS ? LaneMsb<uint32_t, OB>::kValue : 0u;
+  static_assert(kCols % kPiece == 0, "whole pieces");
   const int lane = threadIdx.x & 31;
-  const int ch0 = nb * args.NBc;
-  const int nvalid = args.K - ch0 < args.NBc ? args.K - ch0 : args.NBc;
-  const int nwords = (nvalid + L - 1) / L;  // the block's words in a row
   const float scale = args.out_scale;
-  const unsigned vmask = __ballot_sync(0xffffffffu, row_valid);
-  uint32_t *const out = static_cast<uint32_t *>(args.packed_out) + ch0 / L;
-  uint32_t *const mine = stg + lane * kEpiPitch;
-  for (int c0 = 0, wbase = 0; c0 < nvalid; c0 += 32 * G, wbase += PW) {
-    uint32_t cur = 0;
-    bool open = false;
-    int wcur = 0;  // words of this period staged so far
+  const int nwords = (e.nvalid + L - 1) / L;
+  const int last_lanes = e.nvalid - (nwords - 1) * L;
+  const uint32_t last_mask = (1u << (last_lanes * OB)) - 1;  // L * OB <= 30 bits
+  uint32_t *const out = static_cast<uint32_t *>(args.packed_out);
+  uint32_t *const own = out + (static_cast<size_t>(e.m) * args.out_wpr + e.ch0 / L);
+  const unsigned vmask = __ballot_sync(0xffffffffu, e.valid());
+  const bool flat = args.e_flat != 0, by_rows = args.e_stage != 0;
+  uint32_t *const mine = flat ? stg + __popc(vmask & ((1u << lane) - 1)) * nwords : stg + lane * kEpiPitch;
+  auto load = [&](int c0, uint32_t (&r)[kCols]) {
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const int col = c0 + 32 * g;
-      if (col >= nvalid) break;
-      uint32_t r[32];
-      ptx::tmem_ld_32x32b_x32(taddr + col, r);
-      ptx::tmem_wait_ld();
+    for (int q = 0; q < kCols; q += kPiece) {
+      const int col = c0 + q < args.n_mma ? c0 + q : 0;  // past the last column: any, not stored
+      if constexpr (kPiece == 4)
+        ptx::tmem_ld_32x32b_x4(e.taddr + col, r + q);
+      else
+        ptx::tmem_ld_32x32b_x8(e.taddr + col, r + q);
+    }
+  };
+  auto group = [&](int c0, int w0, const uint32_t (&r)[kCols]) {
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const int q = 32 * g + k;  // channel within the period (compile-time after unrolling)
-        const int l = q % L;
-        int32_t t = floor_scaled_biased(__uint_as_float(r[k]), scale);
-        t = t < blo ? blo : (t > bhi ? bhi : t);
-        if (col + k >= nvalid) t = kMagicBits;
-        cur |= (static_cast<uint32_t>(t) & omask) << (l * OB);
-        open = true;
-        if (l == L - 1) {
-          mine[wcur++] = cur;
-          cur = 0;
-          open = false;
+    for (int j = 0; j < kWords; ++j) {
+      uint32_t w = 0;
+#pragma unroll
+      for (int l = 0; l < L; ++l) w += requant_lane(r[j * L + l], scale, addend, omax) << (l * OB);
+      w ^= flip;
+      const int wi = w0 + j;
+      if (wi == nwords - 1) w &= last_mask;  // the row's last, partial word
+      if (wi < nwords) {
+        if (flat) {
+          if (e.valid()) mine[wi] = w;
+        } else if (by_rows) {
+          mine[wi & 31] = w;
+        } else if (e.valid()) {
+          own[wi] = w;
         }
       }
     }
-    if (open) mine[wcur] = cur;  // the row's last, partial word
-    __syncwarp();
-    const int nw = nwords - wbase < PW ? nwords - wbase : PW;  // this period's words inside the block
-    const int wi = lane % PW;
+    if (by_rows && (((w0 + kWords) & 31) == 0 || c0 + kCols >= e.nvalid)) {
+      __syncwarp();
+      const int wb = w0 & ~31;  // first word of this flush
+      const bool has = wb + lane < nwords;
 #pragma unroll 4
-    for (int r0 = 0; r0 < 32; r0 += RPI) {
-      const int rr = r0 + lane / PW;
-      const long long mr = __shfl_sync(0xffffffffu, m, rr);
-      if (((vmask >> rr) & 1u) && wi < nw) out[mr * args.out_wpr + wbase + wi] = stg[rr * kEpiPitch + wi];
+      for (int rr = 0; rr < 32; ++rr) {
+        const uint32_t mr = __shfl_sync(0xffffffffu, e.m, rr);
+        if (has && mr != ~0u)
+          out[static_cast<size_t>(mr) * args.out_wpr + e.ch0 / L + wb + lane] = stg[rr * kEpiPitch + lane];
+      }
+      __syncwarp();
     }
+  };
+  // the next group's columns are on their way while one is packed
+  uint32_t ra[kCols], rb[kCols];
+  load(0, ra);
+  ptx::tmem_wait_ld(ra);
+  for (int c0 = 0, w0 = 0; c0 < e.nvalid; c0 += 2 * kCols, w0 += 2 * kWords) {
+    load(c0 + kCols, rb);
+    group(c0, w0, ra);
+    ptx::tmem_wait_ld(rb);
+    if (c0 + kCols >= e.nvalid) break;
+    load(c0 + 2 * kCols, ra);
+    group(c0 + kCols, w0 + kWords, rb);
+    ptx::tmem_wait_ld(ra);
+  }
+  if (flat && vmask != 0u) {
+    __syncwarp();
+    const uint32_t m0 = __shfl_sync(0xffffffffu, e.m, __ffs(vmask) - 1);
+    uint32_t *const dst = out + static_cast<size_t>(m0) * args.out_wpr;
+    const int total = __popc(vmask) * nwords;
+    int i = 0;
+    if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+      i = total & ~3;
+      for (int k = 4 * lane; k < i; k += 128)
+        *reinterpret_cast<uint4 *>(dst + k) = *reinterpret_cast<const uint4 *>(stg + k);
+    }
+    for (int k = i + lane; k < total; k += 32) dst[k] = stg[k];
     __syncwarp();
   }
 }
@@ -834,42 +840,46 @@ __device__ __forceinline__ void epilogue_row_period_staged(const ConvArgs &args,
 // Every other case, 16 columns at a time: split digits (acc = 16 hi + lo),
 // int32 outputs, accumulators too large for the fma path.
 template <typename WO>
-__device__ __forceinline__ void epilogue_row_general(const ConvArgs &args, uint32_t taddr, bool row_valid,
-                                                     long long m, int nb) {
-  const int ch0 = nb * args.NBc;
-  const int nvalid = args.K - ch0 < args.NBc ? args.K - ch0 : args.NBc;
-  const bool vec_ok = (args.K % 4 == 0) && (ch0 % 4 == 0);
+__device__ __forceinline__ void epilogue_row_general(const ConvArgs &args, const EpiRow &e) {
+  const bool vec_ok = (args.K % 4 == 0) && (e.ch0 % 4 == 0);
+  const bool vec8_ok = (args.K % 8 == 0) && (e.ch0 % 8 == 0) && (reinterpret_cast<uintptr_t>(args.acc_out) & 31) == 0;
   const int lo = lane_lo(args.out_bits, args.out_signed), hi = lane_hi(args.out_bits, args.out_signed);
   const uint32_t omask = (1u << args.out_bits) - 1;
   const int L = args.out_L, lw = args.out_lane_w;
   RowPacker<WO> pk;
-  pk.dst = static_cast<WO *>(args.packed_out) + (m * args.out_wpr + ch0 / (L > 0 ? L : 1));
-  for (int col = 0; col < nvalid; col += 16) {
+  pk.dst = static_cast<WO *>(args.packed_out) + (static_cast<long long>(e.m) * args.out_wpr + e.ch0 / (L > 0 ? L : 1));
+  for (int col = 0; col < e.nvalid; col += 16) {
     uint32_t r[16];
     int v[16];
-    ptx::tmem_ld_32x32b_x16(taddr + col, r);
+    ptx::tmem_ld_32x32b_x16(e.taddr + col, r);
     if (args.split) {  // acc = 16 * hi + lo
       uint32_t r2[16];
-      ptx::tmem_ld_32x32b_x16(taddr + args.n_mma + col, r2);
-      ptx::tmem_wait_ld();
+      ptx::tmem_ld_32x32b_x16(e.taddr + args.n_mma + col, r2);
+      ptx::tmem_wait_ld(r);
+      ptx::tmem_wait_ld(r2);
 #pragma unroll
       for (int k = 0; k < 16; ++k)
-        v[k] = 16 * __float2int_rn(__uint_as_float(r[k])) + __float2int_rn(__uint_as_float(r2[k]));
+        v[k] = 16 * __float2int_rn(__uint_as_float(r[k]) * args.acc_scale) +
+               __float2int_rn(__uint_as_float(r2[k]) * args.acc_scale);
     } else {
-      ptx::tmem_wait_ld();
+      ptx::tmem_wait_ld(r);
       if (args.fast_acc) {  // |acc| < 2^22: the exact integer from the float's encoding
 #pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = floor_scaled_biased(__uint_as_float(r[k]), 1.0f) - kMagicBits;
+        for (int k = 0; k < 16; ++k) v[k] = floor_scaled_biased(__uint_as_float(r[k]), args.acc_scale) - kMagicBits;
       } else {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = __float2int_rn(__uint_as_float(r[k]));
+        for (int k = 0; k < 16; ++k) v[k] = __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
       }
     }
-    if (!row_valid) continue;
-    const int cnt = nvalid - col < 16 ? nvalid - col : 16;
+    if (!e.valid()) continue;
+    const int cnt = e.nvalid - col < 16 ? e.nvalid - col : 16;
     if (args.acc_out) {
-      int32_t *dst = args.acc_out + m * args.K + ch0 + col;
-      if (cnt == 16 && vec_ok) {
+      int32_t *dst = args.acc_out + static_cast<long long>(e.m) * args.K + e.ch0 + col;
+      if (cnt == 16 && vec8_ok) {  // whole 32-byte sectors
+#pragma unroll
+        for (int k = 0; k < 16; k += 8)
+          ptx::st_global_v8(dst + k, v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4], v[k + 5], v[k + 6], v[k + 7]);
+      } else if (cnt == 16 && vec_ok) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           reinterpret_cast<int4 *>(dst)[k] = make_int4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
@@ -885,73 +895,42 @@ __device__ __forceinline__ void epilogue_row_general(const ConvArgs &args, uint3
         if (k < cnt) pk.put(static_cast<uint32_t>(clamp_int(v[k] >> args.shift, lo, hi)) & omask, L, lw);
     }
   }
-  if (args.packed_out && row_valid) pk.flush();
+  if (args.packed_out && e.valid()) pk.flush();
 }
 
-__device__ __forceinline__ void epilogue_row(const ConvArgs &args, uint32_t taddr, bool row_valid, long long m,
-                                             int nb, uint32_t *estage) {
+__device__ __forceinline__ void epilogue_row(const ConvArgs &args, const EpiRow &e, uint32_t *estage) {
   const bool fast = args.packed_out && !args.acc_out && !args.split && args.fast_req;
   if (fast && args.out_lane_w == args.out_bits && (!args.out_word64 || (args.out_bits & (args.out_bits - 1)) == 0)) {
     switch (args.out_bits * 2 + (args.out_signed ? 1 : 0)) {
-      case 2: epilogue_row_spec<1, false>(args, taddr, row_valid, m, nb); return;
-      case 3: epilogue_row_spec<1, true>(args, taddr, row_valid, m, nb); return;
-      case 4: epilogue_row_spec<2, false>(args, taddr, row_valid, m, nb); return;
-      case 5: epilogue_row_spec<2, true>(args, taddr, row_valid, m, nb); return;
-      case 6:
-        if (estage)
-          epilogue_row_period_staged<3, false>(args, taddr, row_valid, m, nb, estage);
-        else
-          epilogue_row_period<3, false>(args, taddr, row_valid, m, nb);
-        return;
-      case 7:
-        if (estage)
-          epilogue_row_period_staged<3, true>(args, taddr, row_valid, m, nb, estage);
-        else
-          epilogue_row_period<3, true>(args, taddr, row_valid, m, nb);
-        return;
-      case 8: epilogue_row_spec<4, false>(args, taddr, row_valid, m, nb); return;
-      case 9: epilogue_row_spec<4, true>(args, taddr, row_valid, m, nb); return;
-      case 10:
-        if (estage)
-          epilogue_row_period_staged<5, false>(args, taddr, row_valid, m, nb, estage);
-        else
-          epilogue_row_period<5, false>(args, taddr, row_valid, m, nb);
-        return;
-      case 11:
-        if (estage)
-          epilogue_row_period_staged<5, true>(args, taddr, row_valid, m, nb, estage);
-        else
-          epilogue_row_period<5, true>(args, taddr, row_valid, m, nb);
-        return;
-      case 12:
-        if (estage)
-          epilogue_row_period_staged<6, false>(args, taddr, row_valid, m, nb, estage);
-        else
-          epilogue_row_period<6, false>(args, taddr, row_valid, m, nb);
-        return;
-      case 13:
-        if (estage)
-          epilogue_row_period_staged<6, true>(args, taddr, row_valid, m, nb, estage);
-        else
-          epilogue_row_period<6, true>(args, taddr, row_valid, m, nb);
-        return;
-      case 14: epilogue_row_spec<7, false>(args, taddr, row_valid, m, nb); return;
-      case 15: epilogue_row_spec<7, true>(args, taddr, row_valid, m, nb); return;
-      case 16: epilogue_row_spec<8, false>(args, taddr, row_valid, m, nb); return;
-      case 17: epilogue_row_spec<8, true>(args, taddr, row_valid, m, nb); return;
+      case 2: epilogue_row_spec<1, false>(args, e); return;
+      case 3: epilogue_row_spec<1, true>(args, e); return;
+      case 4: epilogue_row_spec<2, false>(args, e); return;
+      case 5: epilogue_row_spec<2, true>(args, e); return;
+      case 6: epilogue_row_words<3, false>(args, e, estage); return;
+      case 7: epilogue_row_words<3, true>(args, e, estage); return;
+      case 8: epilogue_row_spec<4, false>(args, e); return;
+      case 9: epilogue_row_spec<4, true>(args, e); return;
+      case 10: epilogue_row_words<5, false>(args, e, estage); return;
+      case 11: epilogue_row_words<5, true>(args, e, estage); return;
+      case 12: epilogue_row_words<6, false>(args, e, estage); return;
+      case 13: epilogue_row_words<6, true>(args, e, estage); return;
+      case 14: epilogue_row_spec<7, false>(args, e); return;
+      case 15: epilogue_row_spec<7, true>(args, e); return;
+      case 16: epilogue_row_spec<8, false>(args, e); return;
+      case 17: epilogue_row_spec<8, true>(args, e); return;
       default: break;
     }
   }
   if (args.out_word64) {
     if (fast)
-      epilogue_row_fast<uint64_t>(args, taddr, row_valid, m, nb);
+      epilogue_row_fast<uint64_t>(args, e);
     else
-      epilogue_row_general<uint64_t>(args, taddr, row_valid, m, nb);
+      epilogue_row_general<uint64_t>(args, e);
   } else {
     if (fast)
-      epilogue_row_fast<uint32_t>(args, taddr, row_valid, m, nb);
+      epilogue_row_fast<uint32_t>(args, e);
     else
-      epilogue_row_general<uint32_t>(args, taddr, row_valid, m, nb);
+      epilogue_row_general<uint32_t>(args, e);
   }
 }
 
@@ -985,14 +964,8 @@ __device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t t
                                                 uint32_t &phase, int *status, int gw, int gi) {
   constexpr int LH = 32 / OB;  // lanes per word
   constexpr int NH = 32 / LH;  // words per 32 channels
-  constexpr int32_t lo = OS ? -(1 << (OB - 1)) : 0, hi = OS ? (1 << (OB - 1)) - 1 : (1 << OB) - 1;
-  constexpr int32_t blo = kMagicBits + lo, bhi = kMagicBits + hi;
-  constexpr uint32_t omask = (1u << OB) - 1;
-  constexpr uint32_t bias_sum = [] {
-    uint32_t b = 0;
-    for (int l = 0; l < LH; ++l) b += static_cast<uint32_t>(kMagicBits) << (l * OB);
-    return b;
-  }();
+  constexpr int32_t addend = requant_addend(OB, OS), omax = (1 << OB) - 1;
+  constexpr uint32_t flip = OS ? LaneMsb<uint32_t, OB>::kValue : 0u;
   const int ch0 = nb * args.NBc;
   const int nvalid = args.K - ch0 < args.NBc ? args.K - ch0 : args.NBc;
   const int nw = (nvalid + LH - 1) / LH;  // this block's words of a row (<= pool_nw; fewer in a last, partial block)
@@ -1002,23 +975,19 @@ __device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t t
   for (int col = 0; col < nvalid; col += 32) {
     uint32_t r[32];
     ptx::tmem_ld_32x32b_x32(taddr + col, r);
-    ptx::tmem_wait_ld();
+    ptx::tmem_wait_ld(r);
     const int cnt = nvalid - col < 32 ? nvalid - col : 32;
 #pragma unroll
     for (int j = 0; j < NH; ++j) {
       uint32_t w = 0;
 #pragma unroll
-      for (int l = 0; l < LH; ++l) {
-        int32_t t = floor_scaled_biased(__uint_as_float(r[j * LH + l]), scale);
-        t = t < blo ? blo : (t > bhi ? bhi : t);
-        if (j * LH + l >= cnt) t = kMagicBits;  // lanes past the block's channels stay zero
-        if constexpr (OS)
-          w |= (static_cast<uint32_t>(t) & omask) << (l * OB);
-        else
-          w += static_cast<uint32_t>(t) << (l * OB);
-      }
+      for (int l = 0; l < LH; ++l) w += requant_lane(r[j * LH + l], scale, addend, omax) << (l * OB);
+      w ^= flip;
       const int wi = col / LH + j;
-      if (wi < nw) prow[wi] = OS ? w : w - bias_sum;
+      // lanes past the block's channels are zero
+      const int nl = cnt - j * LH;
+      if (nl < LH) w &= nl > 0 ? (1u << (nl * OB)) - 1 : 0u;
+      if (wi < nw) prow[wi] = w;
     }
   }
   ptx::tc_fence_before();
@@ -1031,7 +1000,6 @@ __device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t t
   const int Ho2 = args.Ho / 2, Wo2 = args.Wo / 2, q = args.pool_rows / 2;
   const int q_here = Ho2 - g * q < q ? Ho2 - g * q : q;
   const int total = q_here * Wo2 * nw;
-  const uint32_t flip = OS ? LaneMsb<uint32_t, OB>::kValue : 0u;
   uint32_t *out = static_cast<uint32_t *>(args.packed_out) + ch0 / LH;
   const int Wp = args.Wp;
   for (int idx = 32 * gi + static_cast<int>(threadIdx.x & 31); idx < total; idx += 32 * gw) {
@@ -1591,8 +1559,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     const int quad = warp & 3;
     const int set = (warp - kFirstEpiWarp) / 4;
     uint32_t *const estage =
-        args.e_stage ? reinterpret_cast<uint32_t *>(smem + args.off_e) + (warp - kFirstEpiWarp) * 32 * kEpiPitch
-                     : nullptr;
+        reinterpret_cast<uint32_t *>(smem + args.off_e) +
+        (warp - kFirstEpiWarp) * 32 * (args.e_flat ? args.out_wpr : kEpiPitch);  // unused without e_flat and e_stage
     const int row = quad * 32 + lane;
     constexpr int kTileStep = HV >= 2 ? 1 : 2;
     // parts of 128 rows of a tile this warp drains: set `set` takes parts
@@ -1647,7 +1615,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       for (int hh = 0; hh < kParts; ++hh) {
         const int part = HV >= 2 ? set * kParts + hh : 0;
         bool valid;
-        long long m;
+        uint32_t m;
         const int trow = part * BM + row;  // row of the tile
         if (HALO) {
           const uint32_t v = tile_first_pos(args, mt, BMT) + trow;
@@ -1656,14 +1624,14 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           const uint32_t oh = fdiv(rem, args.fd_wp);
           const uint32_t ow = rem - oh * args.fd_wp.d;
           valid = static_cast<int>(img) < args.N && static_cast<int>(oh) < args.Ho && static_cast<int>(ow) < args.Wo;
-          m = (static_cast<long long>(img) * args.Ho + oh) * args.Wo + ow;
+          m = (img * args.Ho + oh) * args.Wo + ow;
         } else {
-          m = static_cast<long long>(mt) * BMT + trow;
-          valid = m < args.M;
+          m = mt * BMT + trow;
+          valid = m < static_cast<uint64_t>(args.M);
         }
         const uint32_t taddr = tmem_base + static_cast<uint32_t>((acc_i * HV + part) * args.mma_n) +
                                (static_cast<uint32_t>(quad * 32) << 16);
-        epilogue_row(args, taddr, valid && !warm, m, nb, estage);
+        epilogue_row(args, epi_row(args, taddr, valid ? m : ~0u, nb, warm), estage);
       }
       if (warm) {
         warm = false;

@@ -406,3 +406,23 @@ def test_pack_unpack_row_runs(samd_lib, bits, spacer, word_bits):
         back = back.cpu().numpy()
         assert np.array_equal(back[:rows * inner].astype(np.int64), v.ravel()) and (back[rows * inner:] == 0x5A).all()
     assert_status_clean()
+
+
+# 3-, 5- and 6-bit packed outputs leave flat (one channel block), by rows
+# (several) or directly, in groups of 20 or 24 columns: channel counts at the
+# edges of a word, a group and a block, on the padded grid (3x3, images whose
+# rows end inside a tile) and off it (1x1, a last tile with few rows).
+@pytest.mark.parametrize("fo_bits,fo_signed", [(3, False), (3, True), (5, True), (6, False), (6, True)])
+def test_conv_packed_rows_of_words(samd_lib, fo_bits, fo_signed):
+    fo = samd.fmt(fo_bits, fo_signed)
+    for K, (H, R) in itertools.product((1, 13, 20, 24, 25, 61, 160, 200, 256, 511), [((9, 7), 3), ((13, 11), 1)]):
+        shape = samd.ConvShape(3, 16, H[0], H[1], K, R=R, S=R, pad=R // 2)
+        a_v, w_v, a_w, w_w, fa, fw = conv_case(shape, 6, False, 3, True, synth.seed_for("row", K, R, fo_bits))
+        shift = harness_shift(6, 3, fo_bits, shape.C * R * R)
+        n = samd.samd_packed_words(fo, shape.N * shape.Ho * shape.Wo, K)
+        buf = torch.full((n + 64,), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+        samd.samd_conv2d(shape.desc(), fa, a_w, fw, w_w, None, fo, buf, shift, samd.conv_workspace(shape, fa, fw))
+        got = np_words(buf, 32)
+        assert np.array_equal(got[:n], oracle_requant_pack(oracle_conv_nhwc(a_v, w_v, shape), shift, fo)), (K, R)
+        assert (got[n:] == 0x5A5A5A5A).all()
+    assert_status_clean()
