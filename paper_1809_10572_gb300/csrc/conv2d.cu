@@ -782,7 +782,7 @@ samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const 
     a.out_fast = fast ? Lo : 0;
   }
   a.shift = shift;
-  a.acc_scale = 1.0f;
+  a.acc_scale = ldexpf(1.0f, op_exp(fa.is_signed != 0, p.fp8 != 0));
   a.out_scale = ldexpf(a.acc_scale, -shift);
   a.fast_req = (!p.split && (p.bound >> shift) < (1LL << 22)) ? 1 : 0;
   a.fast_acc = (!p.split && p.bound < (1LL << 22)) ? 1 : 0;

@@ -16,6 +16,8 @@
 //        widths up to 4 bits, and signed 5-bit lanes); half the shared-memory
 //        bytes of fp16 per product, twice the tensor rate;
 //   fp16 (kind::f16, K = 16 per MMA) otherwise: every integer of [-128, 255].
+// The A operand holds its integers times a power of two (op_exp), so the
+// accumulators do too; that changes no exactness.
 // When R*S*C*max|a|*max|w| reaches 2^24 (wide weights over many taps), the
 // fp16 weights are split into two 4-bit digits w = 16*hi + lo stacked along
 // the MMA's N; the epilogue forms 16*hi + lo in int32.
@@ -82,34 +84,43 @@ __host__ __device__ constexpr int kpos_lane(int bits, int pos) {
   return pos;
 }
 
-// e4m3 widening by byte permutes (1- and 2-bit lanes, unsigned 4-bit lanes):
-// each lane of a 32-bit half-word becomes a selector nibble of prmt over a
-// table of e4m3 codes. The reduction positions of such a half-word are
-// ordered by how the nibbles are formed (identity for 4 bits; even then odd
-// lanes for 2 bits; lanes k, k+4, ... for 1 bit); A and B use the same order.
-__host__ __device__ constexpr bool prmt8(int bits, bool is_signed) {
-  return bits == 1 || bits == 2 || (bits == 4 && !is_signed);
+// A's operand elements are the lanes' own bits where that is a number: the
+// subnormal and first normal binade of a float format are linear in its
+// encoding, so the byte v (0..16) is v * 2^-9 in e4m3 and the half-word v
+// (0..2047) is v * 2^-24 in fp16. Widening an unsigned lane is then a shift
+// and a mask, without a table, a bias or a conversion. The accumulators hold
+// exact multiples of 2^-kOpExp (the same 24 bits of an integer sum, scaled by
+// a power of two) and the epilogue's scale takes the factor back. Signed
+// lanes are sign and magnitude in e4m3; in fp16 they are widened through the
+// mantissa of 1024.0 to their own value (exponent 0).
+__host__ __device__ constexpr int op_exp(bool is_signed, bool fp8) { return fp8 ? 9 : (is_signed ? 0 : 24); }
+
+// Orders of the e4m3 positions of a 32-bit half-word of 1-, 2- and 4-bit
+// lanes; A and B use the same one. By masks (unsigned lanes, signed 4-bit
+// lanes): word x >> (BITS k) keeps one lane of every byte, so position 4k + b
+// is lane b * 8 / BITS + k. By permutes (signed 1- and 2-bit lanes, whose
+// nibbles select from a table): even then odd lanes for 2 bits, lanes k,
+// k + 4, ... for 1 bit.
+__host__ __device__ constexpr bool mask8(int bits, bool is_signed) {
+  return bits == 4 || (!is_signed && (bits == 1 || bits == 2));
 }
+__host__ __device__ constexpr bool prmt8(int bits, bool is_signed) { return is_signed && (bits == 1 || bits == 2); }
+__host__ __device__ constexpr int kpos_lane_mask32(int bits, int p) { return (p % 4) * (8 / bits) + p / 4; }
 __host__ __device__ constexpr int kpos_lane_prmt32(int bits, int p) {
-  return bits == 4 ? p : (bits == 2 ? 2 * (p % 4 + 4 * ((p / 4) % 2)) + p / 8 : 4 * (p % 8) + p / 8);
+  return bits == 2 ? 2 * (p % 4 + 4 * ((p / 4) % 2)) + p / 8 : 4 * (p % 8) + p / 8;
 }
 // The lane of an activation word held by reduction position `pos` for the
 // operand type in use.
 __host__ __device__ constexpr int kpos_lane_op(int bits, bool is_signed, bool fp8, int pos) {
-  return (fp8 && prmt8(bits, is_signed)) ? (pos / (32 / bits)) * (32 / bits) + kpos_lane_prmt32(bits, pos % (32 / bits))
-                                         : kpos_lane(bits, pos);
+  if (fp8 && (mask8(bits, is_signed) || prmt8(bits, is_signed))) {
+    const int g = 32 / bits, half = pos / g, p = pos % g;
+    return half * g + (mask8(bits, is_signed) ? kpos_lane_mask32(bits, p) : kpos_lane_prmt32(bits, p));
+  }
+  return kpos_lane(bits, pos);
 }
 
-// e4m3 code of a small integer (|v| <= 16): sign, exponent biased by 7, three
-// mantissa bits.
-__host__ __device__ constexpr uint32_t e4m3_code(int v) {
-  if (v == 0) return 0u;
-  const uint32_t sign = v < 0 ? 0x80u : 0u;
-  const int a = v < 0 ? -v : v;
-  int e = 0;
-  while ((a >> (e + 1)) != 0) ++e;
-  return sign | static_cast<uint32_t>((e + 7) << 3) | static_cast<uint32_t>(((a << 3) >> e) - 8);
-}
+// e4m3 code of v * 2^-9 (|v| <= 16): sign and magnitude.
+__host__ __device__ constexpr uint32_t e4m3_code(int v) { return v < 0 ? 0x80u | static_cast<uint32_t>(-v) : static_cast<uint32_t>(v); }
 __host__ __device__ constexpr uint32_t e4m3_table4(int v0, int v1, int v2, int v3) {
   return e4m3_code(v0) | (e4m3_code(v1) << 8) | (e4m3_code(v2) << 16) | (e4m3_code(v3) << 24);
 }
@@ -202,11 +213,12 @@ __device__ __forceinline__ uint32_t hsub2_bits(uint32_t a, uint32_t b) {
   return r;
 }
 
-// two fp16 integers (|v| <= 16, exact in e4m3) -> two e4m3 bytes, low half first
-__device__ __forceinline__ uint32_t f16x2_to_e4m3x2(uint32_t h) {
-  uint16_t r;
-  asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(r) : "r"(h));
-  return r;
+// Four lane patterns of `BITS` bits, one per byte, as signed e4m3 codes:
+// negative patterns (top bit set) become their magnitude with the sign bit.
+template <int BITS>
+__device__ __forceinline__ uint32_t sign_magnitude4(uint32_t e) {
+  const uint32_t n = (e >> (BITS - 1)) & 0x01010101u;       // 1 in the bytes of negative lanes
+  return ((e ^ (n * ((1u << BITS) - 1))) + n) + n * 0x80u;  // 2^BITS - e: bytes stay below 2^7
 }
 
 // Widening of one 64-position row of the A operand (one pixel, one chunk).
@@ -237,9 +249,14 @@ struct AUnpack {
     return static_cast<uint32_t>(w >> (kpos_lane(BITS, POS) * BITS)) & LM;
   }
 
-  // A lane pattern v (offset binary when signed) becomes fp16 1024 + v by
-  // or-ing it into the mantissa of 1024.0; subtracting 1024 + OFF leaves the
-  // lane's value exactly. A zero word (padding) therefore widens to zeros.
+  // Two fp16 operand elements. Unsigned lanes: their bits. Signed lanes: a
+  // pattern v in offset binary becomes 1024 + v by or-ing it into the
+  // mantissa of 1024.0; subtracting 1024 + OFF leaves the lane's value
+  // exactly. A zero word (padding) therefore widens to zeros.
+  __device__ static __forceinline__ uint32_t half2(uint32_t t) {
+    if constexpr (SIGNED) return hsub2_bits(t | 0x64006400u, BIAS2);
+    return t;
+  }
   template <int P>
   __device__ static __forceinline__ uint32_t pair(const W (&w)[WC]) {
     constexpr int j0 = 2 * P, j1 = 2 * P + 1;
@@ -249,13 +266,12 @@ struct AUnpack {
       constexpr int q = j0 / L, pos = j0 % L, g = 32 / BITS, half = pos / g;
       constexpr int lane0 = kpos_lane(BITS, pos) - half * g;
       const uint32_t x = static_cast<uint32_t>(w[q] >> (half * 32));
-      const uint32_t t = ((x >> (lane0 * BITS)) & (LM | (LM << 16))) | 0x64006400u;
-      return hsub2_bits(t, BIAS2);
+      return half2((x >> (lane0 * BITS)) & (LM | (LM << 16)));
     } else {
       const uint32_t v0 = field<j0 % L>(w[j0 / L]);
       uint32_t v1 = OFF;
       if constexpr (j1 < KUSED) v1 = field<j1 % L>(w[j1 / L]);
-      return hsub2_bits(v0 | (v1 << 16) | 0x64006400u, BIAS2);
+      return half2(v0 | (v1 << 16));
     }
   }
 
@@ -265,28 +281,25 @@ struct AUnpack {
     ((h[P] = pair<P>(w)), ...);
   }
 
-  static constexpr bool kPrmt = FP8 && prmt8(BITS, SIGNED);
-
-  // The e4m3 bytes of the lanes of one 32-bit half-word, in reduction order
-  // (32 / BITS bytes into out[0 .. 8 / BITS)).
-  __device__ static __forceinline__ void prmt_half(uint32_t x, uint32_t *out) {
-    if constexpr (BITS == 4) {
-      // nibbles 0-7 select e(0..7); nibbles 8-15 select the sign (0) of that
-      // table and, with bit 3 flipped, e(8..15) from the other one
-      constexpr uint32_t t0 = e4m3_table4(0, 1, 2, 3), t1 = e4m3_table4(4, 5, 6, 7);
-      constexpr uint32_t t2 = e4m3_table4(8, 9, 10, 11), t3 = e4m3_table4(12, 13, 14, 15);
-      const uint32_t xx = x ^ 0x88888888u;
-      out[0] = prmt(t0, t1, x) | prmt(t2, t3, xx);
-      out[1] = prmt(t0, t1, x >> 16) | prmt(t2, t3, xx >> 16);
+  // The e4m3 bytes of the lanes of one 32-bit half-word of 1-, 2- or 4-bit
+  // lanes, in reduction order (32 / BITS bytes into out[0 .. 8 / BITS)).
+  static constexpr bool kWordwise = FP8 && (mask8(BITS, SIGNED) || prmt8(BITS, SIGNED));
+  __device__ static __forceinline__ void bytes_of_half(uint32_t x, uint32_t *out) {
+    if constexpr (mask8(BITS, SIGNED)) {
+#pragma unroll
+      for (int k = 0; k < 8 / BITS; ++k) {
+        out[k] = (x >> (BITS * k)) & (LM * 0x01010101u);
+        if constexpr (SIGNED) out[k] = sign_magnitude4<BITS>(out[k]);
+      }
     } else if constexpr (BITS == 2) {
-      constexpr uint32_t t = SIGNED ? e4m3_table4(0, 1, -2, -1) : e4m3_table4(0, 1, 2, 3);
+      constexpr uint32_t t = e4m3_table4(0, 1, -2, -1);
       const uint32_t se = x & 0x33333333u, so = (x >> 2) & 0x33333333u;
       out[0] = prmt(t, 0u, se);
       out[1] = prmt(t, 0u, se >> 16);
       out[2] = prmt(t, 0u, so);
       out[3] = prmt(t, 0u, so >> 16);
     } else {
-      constexpr uint32_t t = SIGNED ? e4m3_table4(0, -1, 0, 0) : e4m3_table4(0, 1, 0, 0);
+      constexpr uint32_t t = e4m3_table4(0, -1, 0, 0);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const uint32_t sk = (x >> k) & 0x11111111u;
@@ -296,41 +309,54 @@ struct AUnpack {
     }
   }
 
+  // Four e4m3 operand elements, positions 4 P .. 4 P + 3 in lane order (3-
+  // and 5-bit lanes).
+  template <int P>
+  __device__ static __forceinline__ uint32_t quad(const W (&w)[WC]) {
+    const uint32_t e = lane_at<4 * P>(w) | (lane_at<4 * P + 1>(w) << 8) | (lane_at<4 * P + 2>(w) << 16) |
+                       (lane_at<4 * P + 3>(w) << 24);
+    if constexpr (SIGNED) return sign_magnitude4<BITS>(e);
+    return e;
+  }
+  template <int J>
+  __device__ static __forceinline__ uint32_t lane_at(const W (&w)[WC]) {
+    if constexpr (J < KUSED)
+      return static_cast<uint32_t>(w[J / L] >> ((J % L) * BITS)) & LM;
+    else
+      return 0u;
+  }
+  template <int... P>
+  __device__ static __forceinline__ void quads(const W (&w)[WC], uint32_t (&b)[16], std::integer_sequence<int, P...>) {
+    ((b[P] = quad<P>(w)), ...);
+  }
+
   // Widen one pixel's chunk and store it as row `row` of a swizzled K-major
   // operand whose rows are OpTraits::kRowBytes apart.
   __device__ static __forceinline__ void unpack_row(W (&w)[WC], uint8_t *tile, int row) {
     using T = OpTraits<FP8>;
-    if constexpr (kPrmt) {
-      constexpr int kHalves = WB / 32, kPer = 8 / BITS;  // 32-bit words of e4m3 bytes per half-word
+    uint8_t *rp = tile + row * T::kRowBytes;
+    if constexpr (FP8) {
       uint32_t b[16];
+      if constexpr (kWordwise) {
+        constexpr int kHalves = WB / 32, kPer = 8 / BITS;  // 32-bit words of e4m3 bytes per half-word
 #pragma unroll
-      for (int q = 0; q < WC; ++q)
+        for (int q = 0; q < WC; ++q)
 #pragma unroll
-        for (int hh = 0; hh < kHalves; ++hh)
-          prmt_half(static_cast<uint32_t>(w[q] >> (32 * hh)), b + (q * kHalves + hh) * kPer);
-      uint8_t *rp = tile + row * T::kRowBytes;
+          for (int hh = 0; hh < kHalves; ++hh)
+            bytes_of_half(static_cast<uint32_t>(w[q] >> (32 * hh)), b + (q * kHalves + hh) * kPer);
+      } else {
+        quads(w, b, std::make_integer_sequence<int, 16>{});
+      }
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         *reinterpret_cast<uint4 *>(rp + (T::swz(row, c) << 4)) = make_uint4(b[4 * c], b[4 * c + 1], b[4 * c + 2], b[4 * c + 3]);
-      return;
-    }
-    if constexpr (SIGNED) {
-#pragma unroll
-      for (int q = 0; q < WC; ++q) w[q] ^= sign_mask();
-    }
-    uint32_t h[32];
-    pairs(w, h, std::make_integer_sequence<int, 32>{});
-    uint8_t *rp = tile + row * T::kRowBytes;
-    if constexpr (FP8) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        uint32_t b[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          b[k] = f16x2_to_e4m3x2(h[8 * c + 2 * k]) | (f16x2_to_e4m3x2(h[8 * c + 2 * k + 1]) << 16);
-        *reinterpret_cast<uint4 *>(rp + (T::swz(row, c) << 4)) = make_uint4(b[0], b[1], b[2], b[3]);
-      }
     } else {
+      if constexpr (SIGNED) {
+#pragma unroll
+        for (int q = 0; q < WC; ++q) w[q] ^= sign_mask();
+      }
+      uint32_t h[32];
+      pairs(w, h, std::make_integer_sequence<int, 32>{});
 #pragma unroll
       for (int c = 0; c < 8; ++c)
         *reinterpret_cast<uint4 *>(rp + (T::swz(row, c) << 4)) =
@@ -1355,40 +1381,49 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     const W *act = static_cast<const W *>(args.act);
     if constexpr (HALO) {
       const int halo_rows = args.nseg * args.seg_rows;
-      // halo row hr -> virtual offset from the tile's first position, or -1
-      auto voff = [&](int hr) -> int {
-        const int g = static_cast<int>(fdiv(static_cast<uint32_t>(hr), args.fd_seg));
-        const int q = hr - g * args.seg_rows;
-        return q < args.seg_used ? g * args.Wp + q : -1;
-      };
-      // items k = (tile i, channel chunk j), in the MMA's order
-      auto gather = [&](uint32_t tile, int j, int slot) {
+      // Input pixels of this thread's halo rows in the tile being gathered
+      // (-1: padding), found once per tile and used for every channel chunk.
+      constexpr int kRowsPerThread = kMaxHaloRows / kProdThreads;
+      int pix[kRowsPerThread];
+      auto locate = [&](uint32_t tile) {
         const uint32_t mt = tile - fdiv(tile, args.fd_gm) * args.fd_gm.d;
         const uint32_t v0 = tile_first_pos(args, mt, BMT);
-        const uint32_t dst0 = ptx::smem_addr(sG + slot * args.g_stride);
-        for (int hr = t; hr < halo_rows; hr += kProdThreads) {
-          const int off = voff(hr);
-          if (off < 0) continue;
-          const uint32_t u = v0 + static_cast<uint32_t>(off);
+#pragma unroll
+        for (int r = 0; r < kRowsPerThread; ++r) {
+          const uint32_t hr = static_cast<uint32_t>(t + r * kProdThreads);
+          const uint32_t g = fdiv(hr, args.fd_seg);  // rows past a segment's used ones are read by no tap
+          const uint32_t u = v0 + hr + g * static_cast<uint32_t>(args.Wp - args.seg_rows);
           const uint32_t img = fdiv(u, args.fd_plane);
           const uint32_t rem = u - img * args.fd_plane.d;
           const uint32_t ihp = fdiv(rem, args.fd_wp);
           const int ih = static_cast<int>(ihp) - args.pad;
           const int iw = static_cast<int>(rem - ihp * args.fd_wp.d) - args.pad;
-          const bool valid = static_cast<int>(img) < args.N && ih >= 0 && ih < args.H && iw >= 0 && iw < args.W;
-          const W *px = act + ((static_cast<long long>(img) * args.H + ih) * args.W + iw) * args.wpr + j * WC;
+          const bool valid = static_cast<int>(img) < args.N && static_cast<unsigned>(ih) < static_cast<unsigned>(args.H) &&
+                             static_cast<unsigned>(iw) < static_cast<unsigned>(args.W);
+          pix[r] = valid ? (static_cast<int>(img) * args.H + ih) * args.W + iw : -1;
+        }
+      };
+      // items k = (tile i, channel chunk j), in the MMA's order
+      auto gather = [&](int j, int slot) {
+        const uint32_t dst0 = ptx::smem_addr(sG + slot * args.g_stride);
+        const int nw = args.wpr - j * WC;  // words of the chunk; lanes past them meet zero weights
+#pragma unroll
+        for (int r = 0; r < kRowsPerThread; ++r) {
+          const int hr = t + r * kProdThreads;
+          if (hr >= halo_rows) break;
+          const bool valid = pix[r] >= 0;
+          const W *px = valid ? act + (static_cast<long long>(pix[r]) * args.wpr + j * WC) : act;
           const uint32_t dst = dst0 + hr * St::kRowBytes;
           if (args.gather_vec) {
-            stage_chunk<W, WC>(dst, reinterpret_cast<const char *>(valid ? px : act), valid ? 1u : 0u);
+            stage_chunk<W, WC>(dst, reinterpret_cast<const char *>(px), valid ? 1u : 0u);
           } else {
 #pragma unroll
             for (int q = 0; q < WC; ++q) {
-              const bool in = valid && j * WC + q < args.wpr;
-              const W *src = in ? px + q : act;
+              if (q >= nw) break;
               if constexpr (sizeof(W) == 8)
-                ptx::cp_async_8(dst + 8 * q, src, in ? 8u : 0u);
+                ptx::cp_async_8(dst + 8 * q, px + (valid ? q : 0), valid ? 8u : 0u);
               else
-                ptx::cp_async_4(dst + 4 * q, src, in ? 4u : 0u);
+                ptx::cp_async_4(dst + 4 * q, px + (valid ? q : 0), valid ? 4u : 0u);
             }
           }
         }
@@ -1409,7 +1444,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       uint32_t gtile = first_tile;  // issue side
       int gj = 0, gslot = 0;
       auto issue = [&]() {
-        if (gtile < total_tiles) gather(gtile, gj, gslot);
+        if (gtile < total_tiles) {
+          if (gj == 0) locate(gtile);
+          gather(gj, gslot);
+        }
         ptx::cp_async_commit();
         advance(gtile, gj);
         if (++gslot == D) gslot = 0;
@@ -1431,7 +1469,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         if (reused) role_wait(opempty(hb), hpar, status);
         const uint8_t *stg = sG + cslot * args.g_stride;
         for (int hr = t; hr < halo_rows; hr += kProdThreads) {
-          if (voff(hr) < 0) continue;  // a row no tap reads
           W cur[WC];
           load_staged<W, WC>(stg + hr * St::kRowBytes, cur);
           U::unpack_row(cur, sOp + hb * args.op_stride, hr);
