@@ -202,6 +202,7 @@ struct Plan {
   int hbufs;   // HALO: widened halo buffers (2 or 3)
   int e_stage; // kEpiStageBytes at off_e stage the epilogue's 3/5/6-bit packed rows
   int e_flat;  // ConvArgs::e_flat
+  int tgroup;  // weight tiles of a streamed stage (ConvArgs::tgroup)
   int pool, pool_rows, pool_nw, pool_pitch, pool_tpi;  // fused 2x2 max-pool (ConvArgs::pool)
   long long M;
   long long bound;  // R*S*C * max|a| * max|w|: no accumulator exceeds it
@@ -322,7 +323,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   const size_t kBudget = 224 * 1024;  // below the 227 KB opt-in limit minus static shared memory
   auto finish = [&](size_t op_bytes, size_t g_bytes, int op_stages) {
     p.off_b = static_cast<uint32_t>(op_bytes);
-    p.off_g = static_cast<uint32_t>(op_bytes + p.stages * bst);
+    p.off_g = static_cast<uint32_t>(op_bytes + p.stages * p.tgroup * bst);
     p.off_e = static_cast<uint32_t>(round_up(p.off_g + g_bytes, 16));
     p.off_bar = static_cast<uint32_t>(round_up(p.off_e + e_bytes, 16));
     p.smem_bytes = 1024 + p.off_bar + bar_bytes(p.stages, op_stages);  // + alignment slack of the base
@@ -353,6 +354,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
     p.hbufs = 2;
     p.b_resident = 0;
     p.stages_a = 0;
+    p.tgroup = 1;
     p.nseg = p.seg_rows = p.seg_used = p.row_step = 0;
     p.nchunks = nchunks_gather;
     p.Kpad = p.nchunks * BK;
@@ -421,8 +423,15 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
         p.b_resident = 1;
         p.stages = ntiles_b;
       } else {
-        long long st = static_cast<long long>((kBudget - fixed - bar_bytes(8, hbufs)) / bst);
-        p.stages = static_cast<int>(st > 8 ? 8 : st);
+        // a stage of one filter row's tiles where three fit (see the MMA
+        // role: VGG-16 layers of 256 and 512 channels), else of one tile
+        // (a pooled layer's packed rows come after the other regions)
+        const size_t pool_rows_bytes = pool ? round_up(static_cast<size_t>(2 * BM) * pool_pitch(p.NBc, fo) * 4, 16) : 0;
+        const size_t room = kBudget - fixed - bar_bytes(8, hbufs);
+        p.tgroup = room >= pool_rows_bytes && (room - pool_rows_bytes) / (d->S * bst) >= 3 ? d->S : 1;
+        long long st = static_cast<long long>(room / (p.tgroup * bst));
+        const int most = p.tgroup > 1 ? 3 : 8;
+        p.stages = static_cast<int>(st > most ? most : st);
       }
       p.op_stride = static_cast<uint32_t>(halo_bytes);
       p.g_stride = static_cast<uint32_t>(stage_g);
@@ -577,7 +586,7 @@ bool layout_ok(const Plan &p) {
   const size_t op_bytes = NO * p.op_stride;
   const size_t bars = (2 * static_cast<size_t>(p.stages) + 2 * NO + 7) * 8 + 4;
   return p.stages >= 1 && NO >= 2 && op_bytes <= p.off_b &&
-         p.off_b + static_cast<size_t>(p.stages) * p.b_bytes <= p.off_g && p.off_g + static_cast<size_t>(p.halo ? p.gdepth : 2) * p.g_stride <= p.off_e &&
+         p.off_b + static_cast<size_t>(p.stages) * p.tgroup * p.b_bytes <= p.off_g && p.tgroup >= 1 && (p.tgroup == 1 || (p.halo && p.taps % p.tgroup == 0 && !p.b_resident)) && p.off_g + static_cast<size_t>(p.halo ? p.gdepth : 2) * p.g_stride <= p.off_e &&
          p.off_e <= p.off_bar && 1023 + p.off_bar + bars <= p.smem_bytes && p.op_stride % 1024 == 0 &&
          p.off_b % 1024 == 0 && p.b_bytes % 1024 == 0 && p.off_bar % 8 == 0 && 2 * p.hv * p.mma_n <= 512 &&
          (p.hv == 1 || p.hv == 2 || (p.hv == 4 && p.halo && p.fp8 && p.mma_n <= 64)) && (!p.halo || (p.gdepth >= 2 && p.gdepth <= 4 && (p.hbufs == 2 || p.hbufs == 3))) &&
@@ -817,6 +826,7 @@ samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const 
   a.off_e = p.off_e;
   a.e_stage = p.e_stage;
   a.e_flat = p.e_flat;
+  a.tgroup = p.tgroup;
   a.pool = p.pool;
   a.pool_rows = p.pool ? p.pool_rows : 0;
   a.pool_nw = p.pool ? p.pool_nw : 0;

@@ -147,7 +147,8 @@ struct ConvArgs {
   int n_mma;        // NBc rounded up to 16
   int mma_n;        // MMA N: n_mma, or 2 * n_mma with split weight digits
   int split;        // 1: accumulator columns [0, n_mma) hold hi digits, [n_mma, 2 n_mma) lo digits
-  int stages;       // weight tiles in flight (or resident)
+  int stages;       // weight stages in flight (or resident tiles)
+  int tgroup;       // weight tiles of a stage: a filter row's (HALO, streamed weights) or 1
   int stages_a;     // GATHER: A tiles in flight
   int b_resident;   // 1: all weight tiles of the layer stay in shared memory
   long long grid_m; // 128-position tiles along the output
@@ -1058,74 +1059,30 @@ __device__ __forceinline__ void epilogue_pool_dispatch(const ConvArgs &args, uin
 #undef SAMD_POOL_TILE
 }
 
-// One MMA.
-template <bool FP8>
-__device__ __forceinline__ void mma_op(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  if constexpr (FP8)
-    ptx::mma_f8(d, a, b, idesc, acc);
-  else
-    ptx::mma_f16(d, a, b, idesc, acc);
-}
-
-// For a tile of HV parts of 128 rows (HV = 1, 2, 4), each k-step issues one
-// MMA per part: part h accumulates into d + h * dn from A rows 128 h on
-// (a + h * ah).
-template <bool FP8, int HV>
-__device__ __forceinline__ void mma_kstep(uint32_t d, uint32_t dn, uint64_t a, uint64_t ah, uint64_t b, uint32_t idesc,
-                                          uint32_t acc) {
-  mma_op<FP8>(d, a, b, idesc, acc);
-  if constexpr (HV >= 2) mma_op<FP8>(d + dn, a + ah, b, idesc, acc);
-  if constexpr (HV == 4) {
-    mma_op<FP8>(d + 2 * dn, a + 2 * ah, b, idesc, acc);
-    mma_op<FP8>(d + 3 * dn, a + 3 * ah, b, idesc, acc);
-  }
-}
-
-// Issues `ksteps` (1..4) k-steps of one operand row as straight-line code.
-template <bool FP8, int HV>
-__device__ __forceinline__ void mma_ksteps(int ksteps, uint32_t d, uint32_t dn, uint64_t a, uint64_t ah, uint64_t b,
-                                           uint32_t idesc, uint32_t acc) {
-  switch (ksteps) {
-    case 4:
-      mma_kstep<FP8, HV>(d, dn, a, ah, b, idesc, acc);
-      mma_kstep<FP8, HV>(d, dn, a + 2, ah, b + 2, idesc, 1u);
-      mma_kstep<FP8, HV>(d, dn, a + 4, ah, b + 4, idesc, 1u);
-      mma_kstep<FP8, HV>(d, dn, a + 6, ah, b + 6, idesc, 1u);
-      break;
-    case 3:
-      mma_kstep<FP8, HV>(d, dn, a, ah, b, idesc, acc);
-      mma_kstep<FP8, HV>(d, dn, a + 2, ah, b + 2, idesc, 1u);
-      mma_kstep<FP8, HV>(d, dn, a + 4, ah, b + 4, idesc, 1u);
-      break;
-    case 2:
-      mma_kstep<FP8, HV>(d, dn, a, ah, b, idesc, acc);
-      mma_kstep<FP8, HV>(d, dn, a + 2, ah, b + 2, idesc, 1u);
-      break;
-    default:
-      mma_kstep<FP8, HV>(d, dn, a, ah, b, idesc, acc);
-      break;
-  }
-}
-
-// Issues the MMAs of all `taps` taps of one operand stage with resident
-// weights: tap t reads weight tile t (b advances by b_step16) and the A
-// operand one row further on, skipping a_skip16 at the end of each filter
-// row (HALO); straight-line issue keeps the tensor core fed. Descriptors
-// advance in 16-byte units of their start-address field.
-template <bool FP8, int HV>
-__device__ __forceinline__ void issue_taps(uint32_t d, uint32_t dn, uint64_t a, uint64_t ah, uint64_t b, uint32_t idesc,
-                                           int ksteps, int taps, int S, uint32_t a_row16, uint32_t a_skip16,
-                                           uint32_t b_step16, uint32_t acc) {
-  int s = 0;
-  for (int t = 0; t < taps; ++t) {
-    mma_ksteps<FP8, HV>(ksteps, d, dn, a, ah, b, idesc, acc);
-    acc = 1;
-    b += b_step16;
-    a += a_row16;
-    if (++s == S) {
-      s = 0;
-      a += a_skip16;
+// Issues the MMAs of `n` consecutive taps of a filter row, KS k-steps each
+// and one MMA per 128-row part of the tile (HV = 1, 2, 4): part h accumulates
+// into d + h * dn from A rows 128 h on (a + h * ah). Tap t reads weight tile
+// t (b advances by b_step16) and the A operand one row further on. Descriptors
+// advance in 16-byte units of their start-address field. Run by the whole
+// warp on uniform values; the leader lane issues.
+template <bool FP8, int HV, int KS>
+__device__ __forceinline__ void issue_row(uint32_t leader, uint32_t d, uint32_t dn, uint64_t a, uint64_t ah, uint64_t b,
+                                          uint32_t idesc, int n, uint32_t a_row16, uint32_t b_step16, uint32_t acc) {
+  for (int t = 0; t < n; ++t) {
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+#pragma unroll
+      for (int h = 0; h < HV; ++h) {
+        const uint32_t accumulate = ks == 0 ? acc : 1u;
+        if constexpr (FP8)
+          ptx::mma_f8(leader, d + h * dn, a + h * ah + 2 * ks, b + 2 * ks, idesc, accumulate);
+        else
+          ptx::mma_f16(leader, d + h * dn, a + h * ah + 2 * ks, b + 2 * ks, idesc, accumulate);
+      }
     }
+    acc = 1;
+    a += a_row16;
+    b += b_step16;
   }
 }
 
@@ -1175,7 +1132,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
 
-  const int STB = args.stages;  // weight tiles in flight (or resident)
+  const int STB = args.stages;  // weight stages in flight (or resident tiles)
   const bool resident = args.b_resident != 0;
   const uint32_t b_bytes = args.b_bytes;
   uint8_t *sOp = smem;  // HALO: hbufs halo buffers; GATHER: stages_a A tiles
@@ -1252,13 +1209,15 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         uint32_t par = 1;       // parity of the previous round's release
         for (uint32_t tile = first_tile; tile < total_tiles; tile += tile_step) {
           const int row0 = static_cast<int>(fdiv(tile, args.fd_gm)) * args.mma_n;
-          for (int c = 0; c < nchunks; ++c) {
+          for (int c = 0; c < nchunks; c += args.tgroup) {
             if (loaded == STB)
               role_wait(empty_b(s), par, status);
             else
               ++loaded;
-            ptx::mbar_arrive_expect_tx(full_b(s), b_bytes);
-            ptx::tma_load_2d(ptx::smem_addr(sB + s * b_bytes), &tmap_b, c * BK, row0, full_b(s));
+            ptx::mbar_arrive_expect_tx(full_b(s), args.tgroup * b_bytes);
+            const uint32_t dst = ptx::smem_addr(sB) + s * args.tgroup * b_bytes;
+            for (int g = 0; g < args.tgroup; ++g)
+              ptx::tma_load_2d(dst + g * b_bytes, &tmap_b, (c + g) * BK, row0, full_b(s));
             if (++s == STB) {
               s = 0;
               par ^= 1;
@@ -1277,19 +1236,26 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     }
   } else if (warp == 1) {
     // ---- MMA issue ----
-    // The whole warp runs this loop on warp-uniform values and one elected
-    // lane (always the same one: all lanes are converged) issues each
-    // tcgen05.mma and tcgen05.commit. Running the loop in one thread alone
-    // turns every descriptor into a per-thread value that has to be moved to
-    // the uniform datapath before each MMA, which costs more than the MMA.
+    // The whole warp runs this loop on warp-uniform values; each tcgen05.mma
+    // and tcgen05.commit is predicated on one lane (the same one throughout,
+    // whose operations a commit tracks). Running the loop in one thread, or
+    // the issue behind a branch on that lane, turns every descriptor into a
+    // per-thread value that has to be moved to the uniform datapath before
+    // each MMA, which costs more than the MMA.
+    const uint32_t leader = ptx::elect_one() ? 1u : 0u;
     const uint32_t idesc = ptx::idesc_f16_f32(BM, args.mma_n);
     auto wait = [&](uint32_t bar, uint32_t parity) { role_wait(bar, parity, status); };
     // Ring positions advance by increments (no division in this loop).
     int sb = 0, so = 0;
     uint32_t bpar = 0, opar = 0;
-    const uint32_t sB_addr = ptx::smem_addr(sB), sOp_addr = ptx::smem_addr(sOp);
+    const uint32_t sOp_addr = ptx::smem_addr(sOp);
     const int nops = HALO ? args.nck : nchunks;  // operand stages per tile
-    const int taps_here = HALO ? args.taps : 1;
+    // filter rows and taps a row of one operand stage, and how far the A
+    // operand moves on behind a row of taps
+    const int frows = HALO ? args.R : 1, ftaps = HALO ? args.S : 1;
+    const int tgroup = args.tgroup;
+    const uint32_t b_step16 = b_bytes >> 4, b_stage16 = static_cast<uint32_t>(tgroup) * b_step16;
+    const uint64_t bdesc0 = T::desc(ptx::smem_addr(sB));
     constexpr uint32_t a_row16 = T::kRowBytes / 16;  // one operand row in descriptor units
     constexpr uint64_t a_half16 = static_cast<uint64_t>(BM) * a_row16;  // from one 128-row part's A rows to the next
     const uint32_t dn = static_cast<uint32_t>(args.mma_n);          // the second half's accumulator columns
@@ -1326,49 +1292,73 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         // (TMA, or stores fenced with fence.proxy.async before the producers'
         // arrive), which the mbarrier wait already orders.
         const uint64_t a0 = T::desc(sOp_addr + so * args.op_stride);
-        if (resident) {
-          const uint64_t b0 = T::desc(sB_addr + (HALO ? j * taps_here : j) * b_bytes);
-          if (ptx::elect_one())
-            issue_taps<FP8, HV>(tmem_d, dn, a0, a_half16, b0, idesc, ksteps, taps_here, args.S, a_row16, a_skip16,
-                                b_bytes >> 4, acc);
-          __syncwarp();
-          acc = 1;
-        } else {
-          uint64_t adesc = a0;
-          int ts = 0;
-          for (int t = 0; t < taps_here; ++t) {
-            wait(full_b(sb), bpar);
-            const uint64_t bdesc = T::desc(sB_addr + sb * b_bytes);
-            if (ptx::elect_one()) {
-              mma_ksteps<FP8, HV>(ksteps, tmem_d, dn, adesc, a_half16, bdesc, idesc, acc);
-              ptx::mma_commit(empty_b(sb));
-            }
-            __syncwarp();
-            acc = 1;
-            if (++sb == STB) {
-              sb = 0;
-              bpar ^= 1;
-            }
-            if (HALO) {
-              adesc += a_row16;  // next halo row
-              if (++ts == args.S) {
-                ts = 0;
-                adesc += a_skip16;
+        auto run = [&](auto ksteps_c) {
+          constexpr int KS = decltype(ksteps_c)::value;
+          uint64_t a_r = a0;
+          if (resident) {
+            uint64_t b_r = bdesc0 + static_cast<uint32_t>(j * frows * ftaps) * b_step16;
+            auto all_taps = [&](uint32_t who) {
+              for (int r = 0; r < frows; ++r) {
+                issue_row<FP8, HV, KS>(who, tmem_d, dn, a_r, a_half16, b_r, idesc, ftaps, a_row16, b_step16, acc);
+                acc = 1;
+                a_r += static_cast<uint32_t>(ftaps) * a_row16 + a_skip16;
+                b_r += static_cast<uint32_t>(ftaps) * b_step16;
               }
+            };
+            // MMAs of up to 64 columns (48 cycles) are the one case where the
+            // predicate costs more than the branch: VGG-16 conv2 39.1 us with
+            // the predicate, 35.0 with the branch; conv4 (128 columns) 27.6
+            // and 30.7
+            if (args.mma_n <= 64) {
+              if (leader) all_taps(1u);
+              __syncwarp();
+              acc = 1;
+            } else {
+              all_taps(leader);
+            }
+          } else {
+            // Streamed weights: a stage holds tgroup tiles, a whole filter row
+            // where three such stages fit, so that one wait and one commit
+            // serve its MMAs and not one tap's.
+            for (int r = 0; r < frows; ++r) {
+              for (int q = 0; q < ftaps; q += tgroup) {
+                wait(full_b(sb), bpar);
+                issue_row<FP8, HV, KS>(leader, tmem_d, dn, a_r, a_half16, bdesc0 + static_cast<uint32_t>(sb) * b_stage16,
+                                       idesc, tgroup, a_row16, b_step16, acc);
+                ptx::mma_commit(leader, empty_b(sb));
+                acc = 1;
+                a_r += static_cast<uint32_t>(tgroup) * a_row16;
+                if (++sb == STB) {
+                  sb = 0;
+                  bpar ^= 1;
+                }
+              }
+              a_r += a_skip16;
             }
           }
+        };
+        if constexpr (FP8) {
+          if (ksteps == 2)
+            run(std::integral_constant<int, 2>{});
+          else
+            run(std::integral_constant<int, 1>{});
+        } else {
+          switch (ksteps) {
+            case 4: run(std::integral_constant<int, 4>{}); break;
+            case 3: run(std::integral_constant<int, 3>{}); break;
+            case 2: run(std::integral_constant<int, 2>{}); break;
+            default: run(std::integral_constant<int, 1>{}); break;
+          }
         }
-        if (ptx::elect_one()) ptx::mma_commit(opempty(so));  // the stage is free once these MMAs complete
-        __syncwarp();
+        ptx::mma_commit(leader, opempty(so));  // the stage is free once these MMAs complete
         if (++so == NO) {
           so = 0;
           opar ^= 1;
         }
       }
-      if (ptx::elect_one()) ptx::mma_commit(accfull(a));
-      __syncwarp();
+      ptx::mma_commit(leader, accfull(a));
     }
-    if (ptx::elect_one()) ptx::mma_commit(drain_bar);
+    ptx::mma_commit(leader, drain_bar);
     __syncwarp();
     if (lane == 0) {
       int quiet = 0;

@@ -426,3 +426,11 @@ def test_conv_packed_rows_of_words(samd_lib, fo_bits, fo_signed):
         assert np.array_equal(got[:n], oracle_requant_pack(oracle_conv_nhwc(a_v, w_v, shape), shift, fo)), (K, R)
         assert (got[n:] == 0x5A5A5A5A).all()
     assert_status_clean()
+
+
+# Streamed weights (one filter row of tiles a stage, or one tile): more
+# weights than shared memory holds, filters of 3 and 5 columns, e4m3 and fp16.
+@pytest.mark.parametrize("ba,bw,R", [(4, 4, 3), (2, 4, 5), (6, 2, 3), (8, 8, 3)])
+def test_conv_streamed_weights(samd_lib, ba, bw, R):
+    shape = samd.ConvShape(2, 200, 9, 8, 264, R=R, S=R, pad=R // 2)
+    run_conv_check(shape, ba, False, bw, True, fo_t=(ba, False, 0, 32), seed=synth.seed_for("str", ba, bw, R))
