@@ -232,6 +232,11 @@ std::atomic<int> g_min_tiles_per_cta{4};
 samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, Plan &p, bool pool = false,
                       bool two_sided = false);
 
+// Most channels of a block, and the channels of a block: a whole number of
+// output words of Lo lanes.
+int block_limit(int split) { return split ? 128 : 256; }
+int block_channels(int K, int limit, int Lo) { return K <= limit ? K : limit / Lo * Lo; }
+
 // Words between two staged rows of a pooled tile: the row's words of its
 // channel block, made odd (outputs of 1, 2, 4 or 8 bits in 32-bit words).
 int pool_pitch(int NBc, samd_fmt fo) {
@@ -282,13 +287,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   // of 128 for layers with few output positions, which doubles their CTAs,
   // measured slower: every block gathers and widens the whole A operand
   // again, and those layers are bound by that work.)
-  const int limit = p.split ? 128 : 256;
-  if (d->K <= limit) {
-    p.NBc = d->K;
-  } else {
-    const int Lo = fo.bits ? lanes_per_word(fo) : 1;
-    p.NBc = (limit / Lo) * Lo;
-  }
+  p.NBc = block_channels(d->K, block_limit(p.split), fo.bits ? lanes_per_word(fo) : 1);
   p.n_mma = (p.NBc + 15) / 16 * 16;
   p.mma_n = p.split ? 2 * p.n_mma : p.n_mma;
   p.nblocks = (d->K + p.NBc - 1) / p.NBc;
@@ -631,18 +630,23 @@ SymbolAddr g_status_addr, g_scratch_addr;
 }  // namespace conv
 
 size_t conv2d_workspace_size(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw) {
-  // the channel blocking depends on the output format only above 128/256
-  // channels: report the largest size over every output format
+  // The size depends on the output format only through the channel blocking,
+  // and on that only above one block's channels: a block is a whole number of
+  // output words of Lo lanes. The largest size over every output format takes
+  // one plan and the Lo that occur (3 to 64 of them; a plan for each of the
+  // 144 formats took most of a small convolution call).
   conv::Plan p;
   if (conv::make_plan(d, fa, fw, conv::none_fmt(), p) != SAMD_OK) return 0;
+  const int limit = conv::block_limit(p.split);
+  if (d->K <= limit) return p.ws_bytes;
+  const size_t row = static_cast<size_t>(p.Kpad) * (p.fp8 ? 1 : 2);
   size_t best = p.ws_bytes;
   for (int wb : {32, 64})
-    for (int bits = 1; bits <= 8; ++bits)
-      for (int sp = 0; sp + bits <= 16 && sp <= 8; ++sp) {
-        samd_fmt fo{static_cast<uint8_t>(bits), 0, static_cast<uint8_t>(sp), static_cast<uint8_t>(wb)};
-        conv::Plan q;
-        if (conv::make_plan(d, fa, fw, fo, q) == SAMD_OK && q.ws_bytes > best) best = q.ws_bytes;
-      }
+    for (int lane = 1; lane <= 16; ++lane) {
+      const int NBc = conv::block_channels(d->K, limit, wb / lane);
+      const size_t rows = static_cast<size_t>((d->K + NBc - 1) / NBc) * ((NBc + 15) / 16 * 16) * (p.split ? 2 : 1);
+      if (rows * row > best) best = rows * row;
+    }
   return best;
 }
 
@@ -664,12 +668,11 @@ samd_status conv2d_check(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw) {
   return conv::make_plan(d, fa, fw, conv::none_fmt(), p);
 }
 
-samd_status conv2d_prepare(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const void *wt, samd_fmt fo,
-                           void *prepared, size_t prepared_bytes, cudaStream_t s) {
-  using namespace conv;
-  Plan p;
-  samd_status st = make_plan(d, fa, fw, fo, p);
-  if (st != SAMD_OK) return st;
+namespace conv {
+namespace {
+// samd_conv2d_prepare with its plan.
+samd_status prepare_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const void *wt,
+                            void *prepared, size_t prepared_bytes, cudaStream_t s) {
   if (prepared_bytes < p.ws_bytes) return SAMD_ESHAPE;
   WPrepArgs wa;
   wa.K = d->K;
@@ -711,17 +714,10 @@ samd_status conv2d_prepare(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, co
   return cudaGetLastError() == cudaSuccess ? SAMD_OK : SAMD_ECUDA;
 }
 
-samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const void *act, const void *prepared,
-                       size_t prepared_bytes, int32_t *acc_out, samd_fmt fo, void *packed_out, int shift,
-                       cudaStream_t s, void *pooled_out) {
-  using namespace conv;
-  Plan p;
-  // pooled_out: the 2x2 max-pool of the packed output is the only output
-  const bool pool = pooled_out != nullptr;
-  if (pool && (acc_out || packed_out)) return SAMD_EINVAL;
-  if (pool) packed_out = pooled_out;
-  samd_status st = make_plan(d, fa, fw, fo, p, pool);
-  if (st != SAMD_OK) return st;
+// samd_conv2d_prepared (or, with a pooled plan, its fused pool) with its plan.
+samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, const void *act, const void *prepared,
+                        size_t prepared_bytes, int32_t *acc_out, samd_fmt fo, void *packed_out, int shift,
+                        cudaStream_t s) {
   if (prepared_bytes < p.ws_bytes) return SAMD_ESHAPE;
   if (p.M == 0) return SAMD_OK;
   if (!layout_ok(p)) return SAMD_EUNSUP;
@@ -869,13 +865,40 @@ samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const 
   return e == cudaSuccess ? SAMD_OK : SAMD_ECUDA;
 }
 
+}  // namespace
+}  // namespace conv
+
+samd_status conv2d_prepare(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const void *wt, samd_fmt fo,
+                           void *prepared, size_t prepared_bytes, cudaStream_t s) {
+  conv::Plan p;
+  const samd_status st = conv::make_plan(d, fa, fw, fo, p);
+  return st != SAMD_OK ? st : conv::prepare_planned(p, d, fa, fw, wt, prepared, prepared_bytes, s);
+}
+
+samd_status conv2d_run(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const void *act, const void *prepared,
+                       size_t prepared_bytes, int32_t *acc_out, samd_fmt fo, void *packed_out, int shift,
+                       cudaStream_t s, void *pooled_out) {
+  // pooled_out: the 2x2 max-pool of the packed output is the only output
+  const bool pool = pooled_out != nullptr;
+  if (pool && (acc_out || packed_out)) return SAMD_EINVAL;
+  if (pool) packed_out = pooled_out;
+  conv::Plan p;
+  const samd_status st = conv::make_plan(d, fa, fw, fo, p, pool);
+  if (st != SAMD_OK) return st;
+  if (pool && !conv::layout_ok(p)) return SAMD_EUNSUP;
+  return conv::run_planned(p, d, fa, act, prepared, prepared_bytes, acc_out, fo, packed_out, shift, s);
+}
+
 samd_status conv2d_nhwc(const samd_conv_desc *d, samd_fmt fa, const void *act, samd_fmt fw, const void *wt,
                         int32_t *acc_out, samd_fmt fo, void *packed_out, int shift, void *workspace,
                         size_t workspace_bytes, cudaStream_t s) {
   const samd_fmt fplan = packed_out ? fo : conv::none_fmt();
-  samd_status st = conv2d_prepare(d, fa, fw, wt, fplan, workspace, workspace_bytes, s);
+  conv::Plan p;
+  samd_status st = conv::make_plan(d, fa, fw, fplan, p);
   if (st != SAMD_OK) return st;
-  return conv2d_run(d, fa, fw, act, workspace, workspace_bytes, acc_out, fplan, packed_out, shift, s);
+  st = conv::prepare_planned(p, d, fa, fw, wt, workspace, workspace_bytes, s);
+  if (st != SAMD_OK) return st;
+  return conv::run_planned(p, d, fa, act, workspace, workspace_bytes, acc_out, fplan, packed_out, shift, s);
 }
 
 samd_status conv2d_noalloc(const samd_conv_desc *d, samd_fmt fa, const void *act, samd_fmt fw, const void *wt,
