@@ -187,6 +187,7 @@ struct ConvArgs {
   uint32_t off_b, b_bytes, off_g, g_stride, off_e, off_bar;
   int e_stage;  // 1: kEpiStageBytes at off_e stage 32 words of each 3/5/6-bit packed row (epilogue_row_words)
   int e_flat;   // 1: 32 whole rows per epilogue warp at off_e instead (one channel block)
+  int early;    // 1: the next kernel of the stream may be set up while this one drains
   // Fused 2x2 max-pool (pool = 1; halo layers): tile mt is pool_rows output
   // rows (pool_rows / 2 row pairs) of one image from an even row on, at
   // virtual position img * Hv * Wp + g * pool_rows * Wp (img = mt / tiles
@@ -1193,6 +1194,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     if (lane == 0) {
       // ---- weight tiles ----
       ptx::prefetch_tmap(&tmap_b);
+      ptx::grid_dependency_wait();  // the prepared weights
       int quiet = 0;  // the waits below end only when the copies land (or time out)
       if (resident) {
         for (int c = 0; c < nchunks; ++c) {
@@ -1369,6 +1371,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     // ---- operand producers ----
     const int t = threadIdx.x - 64;  // 0 .. kProdThreads - 1
     const W *act = static_cast<const W *>(args.act);
+    ptx::grid_dependency_wait();  // the activations
     if constexpr (HALO) {
       const int halo_rows = args.nseg * args.seg_rows;
       // Input pixels of this thread's halo rows in the tile being gathered
@@ -1578,6 +1581,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       }
       ptx::cp_async_wait<0>();
     }
+    // what is left of this CTA is its last MMAs and rows: the next kernel of
+    // the stream may be set up where there is room
+    if (args.early) ptx::grid_dependents_launch();
   } else {
     // ---- epilogue ----
     // One-half tiles: warp set `set` drains accumulator `set`, i.e. the CTA's
@@ -1608,6 +1614,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         // pooled by all eight epilogue warps, one-half tiles by the four of
         // the set that drains them (alternate tiles, own buffer and barrier)
         pooled = true;
+        ptx::grid_dependency_wait();
         constexpr int gw = HV == 2 ? kEpiWarps : kEpiWarps / 2;
         const int gi = HV == 2 ? warp - kFirstEpiWarp : warp - kFirstEpiWarp - 4 * set;
         uint32_t *const pbuf = reinterpret_cast<uint32_t *>(smem + args.off_e) + (HV == 2 ? 0 : set * BM * args.pool_pitch);
@@ -1662,6 +1669,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       }
       if (warm) {
         warm = false;
+        ptx::grid_dependency_wait();  // earlier readers of the outputs
         continue;
       }
       ptx::tc_fence_before();
@@ -1716,8 +1724,22 @@ cudaError_t launch_conv(const CUtensorMap &tmap, const ConvArgs &args, bool halo
   }
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void *>(kern), smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kThreads, smem, s>>>(tmap, args);
-  return cudaGetLastError();
+  // Launched as a programmatic dependent of the kernel before it in the
+  // stream: barriers, tensor memory and the epilogue's code are set up while
+  // that one drains; every role waits (grid_dependency_wait) before it reads
+  // or writes global memory.
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, kern, tmap, args);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Launchers, one per (operand type, activation word width, lane width), each

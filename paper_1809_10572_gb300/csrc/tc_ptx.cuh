@@ -104,6 +104,15 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int *st
   }
 }
 
+// ---- programmatic dependent launch -----------------------------------------
+
+// Waits until the kernels this launch depends on have completed and their
+// writes are visible (at once if it was launched without the attribute).
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// This CTA no longer minds the next kernel of the stream being set up (its
+// own grid_dependency_wait still waits for this grid to complete).
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- cp.async (global -> shared, zero fill when src_bytes < size) ----------
 
 __device__ __forceinline__ void cp_async_4(uint32_t dst, const void *src, uint32_t src_bytes) {
