@@ -106,6 +106,7 @@ struct WPrepArgs {
   int bits_a, signed_a, fp8, La, WC, wpr_a, words_total;  // reduction order set by the activation format
   int Kpad, n_mma, mma_n, NBc, split;
   int halo, taps;  // halo: reduction order (chunk, tap, position); else (tap-major words, position)
+  int nchw, R, S;  // nchw: weight rows are (k, c, r) of S lanes; else (k, r, s) of C lanes
   long long rows_total;
 };
 
@@ -150,9 +151,14 @@ __global__ void __launch_bounds__(256) wprep_kernel(const WW *__restrict__ wt, v
       if (kw < a.words_total) {
         const int ch = wi * a.La + kpos_lane_op(a.bits_a, a.signed_a != 0, a.fp8 != 0, pos);
         if (ch < a.C) {
-          const long long wrow = static_cast<long long>(k) * a.RS + tap;
-          const WW word = wt[wrow * a.wpr_w + ch / a.Lw];
-          const uint32_t p = static_cast<uint32_t>(word >> ((ch % a.Lw) * a.lane_w_w)) & mask;
+          long long wrow = static_cast<long long>(k) * a.RS + tap;
+          int lane = ch;
+          if (a.nchw) {
+            wrow = (static_cast<long long>(k) * a.C + ch) * a.R + tap / a.S;
+            lane = tap % a.S;
+          }
+          const WW word = wt[wrow * a.wpr_w + lane / a.Lw];
+          const uint32_t p = static_cast<uint32_t>(word >> ((lane % a.Lw) * a.lane_w_w)) & mask;
           v = lane_value(p, a.bits_w, a.signed_w);
           if (plane == 0) v >>= 4;       // floor(v / 16)
           else if (plane == 1) v &= 15;  // v - 16 * floor(v / 16)
@@ -595,6 +601,13 @@ bool layout_ok(const Plan &p) {
                       p.off_e + static_cast<size_t>(2 * BM) * p.pool_pitch * 4 <= p.off_bar));
 }
 
+// The kernel's index math runs in 32 bits.
+bool indexes_ok(const Plan &p, const samd_conv_desc *d) {
+  return static_cast<long long>(d->N) * p.Hv * p.Wp + (p.nseg + 1) * static_cast<long long>(p.Wp) + kMaxHaloRows +
+                 2 * BM < (1LL << 31) &&
+         p.M < (1LL << 31) && p.grid_m * p.nblocks < (1LL << 31);
+}
+
 // Device address of a __device__ symbol in the current context, looked up
 // once per context (the symbol's host-side name is not a device address; a
 // context made after a device reset loads the module again, at a new address).
@@ -673,7 +686,7 @@ namespace conv {
 namespace {
 // samd_conv2d_prepare with its plan.
 samd_status prepare_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, const void *wt,
-                            void *prepared, size_t prepared_bytes, cudaStream_t s) {
+                            void *prepared, size_t prepared_bytes, cudaStream_t s, bool nchw = false) {
   if (prepared_bytes < p.ws_bytes) return SAMD_ESHAPE;
   WPrepArgs wa;
   wa.K = d->K;
@@ -683,7 +696,10 @@ samd_status prepare_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa,
   wa.signed_w = fw.is_signed;
   wa.lane_w_w = fw.bits + fw.spacer;
   wa.Lw = lanes_per_word(fw);
-  wa.wpr_w = static_cast<int>(words_per_row(fw, d->C));
+  wa.nchw = nchw;
+  wa.R = d->R;
+  wa.S = d->S;
+  wa.wpr_w = static_cast<int>(words_per_row(fw, nchw ? d->S : d->C));
   wa.bits_a = fa.bits;
   wa.signed_a = fa.is_signed;
   wa.fp8 = p.fp8;
@@ -718,7 +734,7 @@ samd_status prepare_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa,
 // samd_conv2d_prepared (or, with a pooled plan, its fused pool) with its plan.
 samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, const void *act, const void *prepared,
                         size_t prepared_bytes, int32_t *acc_out, samd_fmt fo, void *packed_out, int shift,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool nchw = false, uint8_t *q8_out = nullptr) {
   if (prepared_bytes < p.ws_bytes) return SAMD_ESHAPE;
   if (p.M == 0) return SAMD_OK;
   if (!layout_ok(p)) return SAMD_EUNSUP;
@@ -746,6 +762,8 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.act = act;
   a.acc_out = acc_out;
   a.packed_out = packed_out;
+  a.nchw = nchw;
+  a.q8_out = q8_out;
   a.status = static_cast<int *>(status_ptr);
   a.N = d->N;
   a.C = d->C;
@@ -787,6 +805,10 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
                                                         : (Lo == 8 || Lo == 16 || Lo == 32));
     a.out_fast = fast ? Lo : 0;
   }
+  if (q8_out) {
+    a.out_bits = fo.bits;
+    a.out_signed = fo.is_signed;
+  }
   a.shift = shift;
   a.acc_scale = ldexpf(1.0f, op_exp(fa.is_signed != 0, p.fp8 != 0));
   a.out_scale = ldexpf(a.acc_scale, -shift);
@@ -802,16 +824,13 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.full = p.full;
   a.hv = p.hv;
   a.taps = p.taps;
-  // the kernel's index math runs in 32 bits
-  if (static_cast<long long>(d->N) * p.Hv * p.Wp + (p.nseg + 1) * static_cast<long long>(p.Wp) + kMaxHaloRows + 2 * BM >=
-          (1LL << 31) ||
-      p.M >= (1LL << 31) || p.grid_m * p.nblocks >= (1LL << 31))
-    return SAMD_EUNSUP;
+  if (!indexes_ok(p, d)) return SAMD_EUNSUP;
   a.fd_plane = make_fastdiv(static_cast<uint32_t>(p.Hv * p.Wp));
   a.fd_wp = make_fastdiv(static_cast<uint32_t>(p.Wp));
   a.fd_seg = make_fastdiv(static_cast<uint32_t>(p.seg_rows > 0 ? p.seg_rows : 1));
   a.fd_wo = make_fastdiv(static_cast<uint32_t>(p.Wo));
   a.fd_ho = make_fastdiv(static_cast<uint32_t>(p.Ho));
+  a.fd_howo = make_fastdiv(static_cast<uint32_t>(p.Ho) * static_cast<uint32_t>(p.Wo));
   a.fd_gm = make_fastdiv(static_cast<uint32_t>(p.grid_m));
   a.op_stride = p.op_stride;
   a.off_b = p.off_b;
@@ -906,6 +925,115 @@ samd_status conv2d_nhwc(const samd_conv_desc *d, samd_fmt fa, const void *act, s
   st = conv::prepare_planned(p, d, fa, fw, wt, workspace, workspace_bytes, s);
   if (st != SAMD_OK) return st;
   return conv::run_planned(p, d, fa, act, workspace, workspace_bytes, acc_out, fplan, packed_out, shift, s);
+}
+
+namespace conv {
+namespace {
+
+// ---- NCHW layers on the tensor cores ------------------------------------------
+//
+// Activations packed along W become pixels packed along C: a block takes the
+// lanes of 32 neighbouring pixels of a row from the words of up to kRepackWords
+// output words' channels, one byte per lane in shared memory, and builds the
+// pixels' words from there. Both sides are L2-sized for the layers that come
+// this way; the byte reads of a word run down a column that the 32 lanes of a
+// warp share a bank row of.
+constexpr int kRepackWords = 8;
+
+struct RepackArgs {
+  int C, H, W, bits, L, wpr_in, wpr_out, wtiles, ctiles;
+  long long tiles;  // (image row) x (32 pixels) x (channel group)
+  FastDiv fd_L;
+};
+
+template <typename WA>
+__global__ void __launch_bounds__(256) nchw_repack_kernel(const WA *__restrict__ in, WA *__restrict__ out,
+                                                          const RepackArgs a) {
+  __shared__ uint8_t lanes[kRepackWords * 64 * 33];  // [channel][pixel], 33 bytes apart
+  const uint32_t mask = (1u << a.bits) - 1;
+  const int px = threadIdx.x & 31, part = threadIdx.x >> 5;
+  for (long long t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+    const int ct = static_cast<int>(t % a.ctiles);
+    const long long rest = t / a.ctiles;
+    const int w0 = static_cast<int>(rest % a.wtiles) * 32;
+    const long long nh = rest / a.wtiles;  // n * H + h
+    const long long n = nh / a.H;
+    const int h = static_cast<int>(nh - n * a.H);
+    const int c0 = ct * kRepackWords * a.L;
+    const int nc = a.C - c0 < kRepackWords * a.L ? a.C - c0 : kRepackWords * a.L;
+    const int w = w0 + px;
+    const uint32_t wi = fdiv(static_cast<uint32_t>(w), a.fd_L);
+    const int sh = (w - static_cast<int>(wi) * a.L) * a.bits;
+    if (w < a.W)
+      for (int c = part; c < nc; c += 8) {
+        const WA word = in[((n * a.C + c0 + c) * a.H + h) * a.wpr_in + wi];
+        lanes[c * 33 + px] = static_cast<uint8_t>(static_cast<uint32_t>(word >> sh) & mask);
+      }
+    __syncthreads();
+    const int q = ct * kRepackWords + part;  // this thread's word of pixel w
+    if (w < a.W && q < a.wpr_out) {
+      const int first = part * a.L;
+      const int cnt = nc - first < a.L ? nc - first : a.L;
+      WA word = 0;
+      for (int i = 0; i < cnt; ++i) word |= static_cast<WA>(lanes[(first + i) * 33 + px]) << (i * a.bits);
+      out[((n * a.H + h) * a.W + w) * a.wpr_out + q] = word;
+    }
+    __syncthreads();
+  }
+}
+
+template <typename WA>
+cudaError_t launch_repack(const samd_conv_desc *d, samd_fmt fa, const void *act, void *out, cudaStream_t s) {
+  RepackArgs a;
+  a.C = d->C;
+  a.H = d->H;
+  a.W = d->W;
+  a.bits = fa.bits;
+  a.L = lanes_per_word(fa);
+  a.wpr_in = static_cast<int>(words_per_row(fa, d->W));
+  a.wpr_out = static_cast<int>(words_per_row(fa, d->C));
+  a.wtiles = (d->W + 31) / 32;
+  a.ctiles = (a.wpr_out + kRepackWords - 1) / kRepackWords;
+  a.tiles = static_cast<long long>(d->N) * d->H * a.wtiles * a.ctiles;
+  a.fd_L = make_fastdiv(static_cast<uint32_t>(a.L));
+  const int grid = resident_grid<nchw_repack_kernel<WA>>(a.tiles * 256, 256);
+  nchw_repack_kernel<WA><<<grid, 256, 0, s>>>(static_cast<const WA *>(act), static_cast<WA *>(out), a);
+  return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace conv
+
+// An NCHW layer whose sums the tensor cores hold exactly and whose repacked
+// activations, widened weights and requantized bytes fit the caller's
+// workspace (sized for the wide-multiply engine) runs as the NHWC kernel
+// between two changes of layout: repacked activations in, NCHW outputs out
+// (the int32 sums to acc_out, and, where packed rows are wanted (fo.bits != 0),
+// the requantized lanes one per byte to *q8 in the workspace, for the caller
+// to pack). *taken tells whether it did; otherwise nothing was launched.
+// 8 x 64 x 56 x 56, u4 x s4, 64 outputs, 3x3: 356 us by wide multiplies, 41 us
+// this way (a call from Python, bound by its four launches).
+samd_status conv2d_nchw_tc(const samd_conv_desc *d, samd_fmt fa, const void *act, samd_fmt fw, const void *wt,
+                           int32_t *acc_out, samd_fmt fo, int shift, void *workspace, size_t workspace_bytes,
+                           cudaStream_t s, bool *taken, const int8_t **q8) {
+  using namespace conv;
+  *taken = false;
+  Plan p;
+  if (make_plan(d, fa, fw, none_fmt(), p) != SAMD_OK || !layout_ok(p) || !indexes_ok(p, d) || p.M == 0) return SAMD_OK;
+  const size_t act_bytes = round_up(static_cast<size_t>(d->N) * d->H * d->W * p.wpr * (fa.word_bits / 8), 256);
+  const size_t wt_bytes = round_up(p.ws_bytes, 256);
+  const size_t q_bytes = fo.bits ? static_cast<size_t>(p.M) * d->K : 0;
+  if (act_bytes + wt_bytes + q_bytes > workspace_bytes) return SAMD_OK;
+  *taken = true;
+  uint8_t *const px = static_cast<uint8_t *>(workspace), *const wp = px + act_bytes;
+  uint8_t *const bytes = fo.bits ? wp + wt_bytes : nullptr;
+  *q8 = reinterpret_cast<const int8_t *>(bytes);
+  const cudaError_t e =
+      fa.word_bits == 32 ? launch_repack<uint32_t>(d, fa, act, px, s) : launch_repack<uint64_t>(d, fa, act, px, s);
+  if (e != cudaSuccess) return SAMD_ECUDA;
+  samd_status st = prepare_planned(p, d, fa, fw, wt, wp, p.ws_bytes, s, true);
+  if (st != SAMD_OK) return st;
+  return run_planned(p, d, fa, px, wp, p.ws_bytes, acc_out, fo, nullptr, shift, s, true, bytes);
 }
 
 samd_status conv2d_noalloc(const samd_conv_desc *d, samd_fmt fa, const void *act, samd_fmt fw, const void *wt,

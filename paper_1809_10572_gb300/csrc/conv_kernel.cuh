@@ -138,6 +138,10 @@ struct ConvArgs {
   const void *act;
   int32_t *acc_out;
   void *packed_out;
+  // NCHW outputs (nchw = 1): acc_out is [N][K][Ho][Wo], and q8_out (or null)
+  // receives the requantized lane patterns one per byte in the same order
+  int nchw;
+  uint8_t *q8_out;
   int *status;  // sticky SAMD_ETIMEOUT record of this device
   int N, C, H, W, K, R, S, stride, pad, Ho, Wo;
   long long M;
@@ -181,6 +185,7 @@ struct ConvArgs {
   FastDiv fd_plane, fd_wp;  // / (Hv * Wp), / Wp
   FastDiv fd_seg;           // / seg_rows
   FastDiv fd_wo, fd_ho;     // output pixel index -> (n, oh, ow)
+  FastDiv fd_howo;          // output pixel index -> (n, pixel of the image)
   FastDiv fd_gm;            // tile -> (channel block, position tile)
   // shared memory carve-up (bytes from the 1024-byte-aligned base)
   uint32_t op_stride;  // one halo buffer or one A tile
@@ -926,7 +931,45 @@ __device__ __forceinline__ void epilogue_row_general(const ConvArgs &args, const
   if (args.packed_out && e.valid()) pk.flush();
 }
 
+// NCHW outputs: the 32 rows of a warp are neighbouring pixels, so for one
+// channel their int32 sums, or their requantized bytes, are neighbours in
+// memory and each store covers whole sectors.
+__device__ __forceinline__ void epilogue_row_nchw(const ConvArgs &args, const EpiRow &e) {
+  const int lo = lane_lo(args.out_bits, args.out_signed), hi = lane_hi(args.out_bits, args.out_signed);
+  const uint32_t omask = (1u << args.out_bits) - 1;
+  const uint32_t howo = args.fd_howo.d;
+  const uint32_t img = e.valid() ? fdiv(e.m, args.fd_howo) : 0u;
+  const size_t base = (static_cast<size_t>(img) * args.K + e.ch0) * howo + (e.m - img * howo);
+  for (int col = 0; col < e.nvalid; col += 16) {
+    uint32_t r[16];
+    int v[16];
+    ptx::tmem_ld_32x32b_x16(e.taddr + col, r);
+    ptx::tmem_wait_ld(r);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
+    if (args.split) {  // acc = 16 * hi + lo
+      ptx::tmem_ld_32x32b_x16(e.taddr + args.n_mma + col, r);
+      ptx::tmem_wait_ld(r);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = 16 * v[k] + __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
+    }
+    if (!e.valid()) continue;
+    const int cnt = e.nvalid - col < 16 ? e.nvalid - col : 16;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      if (k >= cnt) break;
+      const size_t at = base + static_cast<size_t>(col + k) * howo;
+      if (args.acc_out) args.acc_out[at] = v[k];
+      if (args.q8_out) args.q8_out[at] = static_cast<uint8_t>(static_cast<uint32_t>(clamp_int(v[k] >> args.shift, lo, hi)) & omask);
+    }
+  }
+}
+
 __device__ __forceinline__ void epilogue_row(const ConvArgs &args, const EpiRow &e, uint32_t *estage) {
+  if (args.nchw) {
+    epilogue_row_nchw(args, e);
+    return;
+  }
   const bool fast = args.packed_out && !args.acc_out && !args.split && args.fast_req;
   if (fast && args.out_lane_w == args.out_bits && (!args.out_word64 || (args.out_bits & (args.out_bits - 1)) == 0)) {
     switch (args.out_bits * 2 + (args.out_signed ? 1 : 0)) {

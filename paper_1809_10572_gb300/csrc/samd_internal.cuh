@@ -213,6 +213,10 @@ samd_status conv2d_noalloc(const samd_conv_desc *d, samd_fmt fa, const void *act
                                 int32_t *acc_out, samd_fmt fo, void *packed_out, int shift, cudaStream_t s);
 // NCHW packed along W: the wide-multiply engine of widemul.cu
 samd_status conv2d_nchw_check(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, size_t *ws_bytes);
+// the tensor-core route of an NCHW layer (conv2d.cu), where it applies
+samd_status conv2d_nchw_tc(const samd_conv_desc *d, samd_fmt fa, const void *act, samd_fmt fw, const void *wt,
+                           int32_t *acc_out, samd_fmt fo, int shift, void *workspace, size_t workspace_bytes,
+                           cudaStream_t s, bool *taken, const int8_t **q8);
 samd_status conv2d_nchw(const samd_conv_desc *d, samd_fmt fa, const void *act, samd_fmt fw, const void *wt,
                         int32_t *acc_out, samd_fmt fo, void *packed_out, int shift, void *workspace,
                         size_t workspace_bytes, cudaStream_t s);

@@ -119,3 +119,33 @@ def test_nchw_limits(samd_lib):
         samd.samd_conv2d_prepare(samd.ConvShape(1, 8, 8, 8, 4).desc(samd.SAMD_NCHW), fa, fw, dummy, None, dummy)
     assert e.value.status == samd.SAMD_EUNSUP
     assert not dummy.any()
+
+
+# Layers whose repacked operands fit the workspace run on the tensor cores
+# (enough input channels for their outputs), the others by wide multiplies:
+# both sides of that line, ragged widths and channel counts, every kind of
+# operand (e4m3, fp16, split digits), both word widths, extreme values.
+@pytest.mark.parametrize("word_bits", (32, 64))
+@pytest.mark.parametrize("ba,sa,bw,sw", [(4, False, 4, True), (3, True, 2, True), (1, False, 1, True), (6, False, 2, True),
+                                         (7, True, 5, True), (8, False, 6, True)])
+def test_nchw_both_routes(samd_lib, ba, sa, bw, sw, word_bits):
+    for shape in (samd.ConvShape(2, 40, 5, 33, 24, R=1, S=1, pad=0), samd.ConvShape(1, 70, 6, 31, 17, R=1, S=2, pad=1),
+                  samd.ConvShape(2, 24, 9, 64, 20, R=3, S=1, pad=0), samd.ConvShape(2, 3, 9, 33, 70, R=1, S=2, pad=0),
+                  samd.ConvShape(1, 2, 7, 65, 40, R=2, S=1, pad=1)):
+        fa, fw = samd.fmt(ba, sa, 0, word_bits), samd.fmt(bw, sw, 0, word_bits)
+        if samd.samd_conv2d_operand_bits(shape.desc(samd.SAMD_NCHW), fa, fw) == 0:
+            continue
+        fo = samd.fmt(5, sa, 0, word_bits)
+        seed = synth.seed_for("nchw2", shape, ba, sa, bw, sw)
+        check(shape, ba, sa, bw, sw, seed, fo=fo, shift=3, word_bits=word_bits)
+        amin, wmin = (-(1 << (ba - 1)) if sa else (1 << ba) - 1), -(1 << (bw - 1))
+        check(shape, ba, sa, bw, sw, seed, fo=fo, shift=2, word_bits=word_bits,
+              act_gen=lambda s, v=amin: np.where(np.arange(np.prod(s)).reshape(s) % 3 == 0, 0, v),
+              wt_gen=lambda s, v=wmin: np.full(s, v, np.int64))
+
+
+# Sums of 2^24 and more are beyond the tensor cores' exact range.
+def test_nchw_large_sums(samd_lib):
+    shape = samd.ConvShape(1, 2100, 3, 9, 2, R=2, S=2, pad=0)
+    check(shape, 8, False, 4, True, 5, act_gen=lambda s: np.full(s, 255, np.int64),
+          wt_gen=lambda s: np.where(np.arange(np.prod(s)).reshape(s) % 2 == 0, -8, -7))
