@@ -429,13 +429,15 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
         p.b_resident = 1;
         p.stages = ntiles_b;
       } else {
-        // a stage of one filter row's tiles where three fit (see the MMA
-        // role: VGG-16 layers of 256 and 512 channels), else of one tile
-        // (a pooled layer's packed rows come after the other regions)
+        // a stage of one filter row's tiles where three fit (two beside a
+        // pooled layer's packed rows, which come after the other regions),
+        // else of one tile. The two-sided plans, which decide what the fused
+        // pool takes, count single tiles.
         const size_t pool_rows_bytes = pool ? round_up(static_cast<size_t>(2 * BM) * pool_pitch(p.NBc, fo) * 4, 16) : 0;
-        const size_t room = kBudget - fixed - bar_bytes(8, hbufs);
-        p.tgroup = room >= pool_rows_bytes && (room - pool_rows_bytes) / (d->S * bst) >= 3 ? d->S : 1;
-        long long st = static_cast<long long>(room / (p.tgroup * bst));
+        const size_t all = kBudget - fixed - bar_bytes(8, hbufs);
+        const size_t room = all > pool_rows_bytes ? all - pool_rows_bytes : 0;
+        p.tgroup = !two_sided && room / (d->S * bst) >= (pool ? 2 : 3) ? d->S : 1;
+        const long long st = static_cast<long long>((p.tgroup > 1 ? room : all) / (p.tgroup * bst));
         const int most = p.tgroup > 1 ? 3 : 8;
         p.stages = static_cast<int>(st > most ? most : st);
       }
@@ -605,7 +607,7 @@ bool layout_ok(const Plan &p) {
 bool indexes_ok(const Plan &p, const samd_conv_desc *d) {
   return static_cast<long long>(d->N) * p.Hv * p.Wp + (p.nseg + 1) * static_cast<long long>(p.Wp) + kMaxHaloRows +
                  2 * BM < (1LL << 31) &&
-         p.M < (1LL << 31) && p.grid_m * p.nblocks < (1LL << 31);
+         p.M < (1LL << 31) && (p.grid_m + 1) * p.nblocks < (1LL << 31);
 }
 
 // Device address of a __device__ symbol in the current context, looked up
@@ -750,7 +752,17 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   const int esize = p.fp8 ? 1 : 2;
   cuuint64_t gdim[2] = {static_cast<cuuint64_t>(p.Kpad), static_cast<cuuint64_t>(rows_total)};
   cuuint64_t gstride[1] = {static_cast<cuuint64_t>(p.Kpad) * esize};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(BK), static_cast<cuuint32_t>(p.mma_n)};
+  // Pairs of CTAs share the streamed weights of e4m3 halo layers of more than
+  // 128 columns, which pull them through L2 at its bandwidth (VGG-16 conv6:
+  // 240 MB in 27.0 us; 24.0 shared, conv9 31.0 -> 27.8, conv11 16.4 -> 15.5).
+  // fp16 layers (8-bit, 256 channels: 17.7 and 17.9 us), gather layers (131.7
+  // and 132.9 for the ResNet-50 28x28 block) and 128 columns (conv4 with its
+  // pool 30.3 and 31.9) do not gain. A pair's tiles lie in one channel block,
+  // so the position tiles are made even in number; the extra one holds no
+  // output.
+  const bool pair = p.fp8 && p.halo && !p.b_resident && p.mma_n > 128 && p.grid_m >= 2;
+  const long long grid_m = pair ? (p.grid_m + 1) / 2 * 2 : p.grid_m;
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(BK), static_cast<cuuint32_t>(pair ? p.mma_n / 2 : p.mma_n)};
   cuuint32_t estride[2] = {1, 1};
   CUresult cr = enc(&tmap, p.fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
                     const_cast<void *>(prepared), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -786,7 +798,8 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.stages = p.stages;
   a.stages_a = p.stages_a;
   a.b_resident = p.b_resident;
-  a.grid_m = p.grid_m;
+  a.grid_m = grid_m;
+  a.pair = pair;
   a.nblocks = p.nblocks;
   a.gather_vec = p.gather_vec;
   a.gather_win = p.gather_win;
@@ -831,7 +844,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.fd_wo = make_fastdiv(static_cast<uint32_t>(p.Wo));
   a.fd_ho = make_fastdiv(static_cast<uint32_t>(p.Ho));
   a.fd_howo = make_fastdiv(static_cast<uint32_t>(p.Ho) * static_cast<uint32_t>(p.Wo));
-  a.fd_gm = make_fastdiv(static_cast<uint32_t>(p.grid_m));
+  a.fd_gm = make_fastdiv(static_cast<uint32_t>(grid_m));
   a.op_stride = p.op_stride;
   a.off_b = p.off_b;
   a.b_bytes = p.b_bytes;
@@ -848,6 +861,8 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.pool_nw = p.pool ? p.pool_nw : 0;
   a.pool_pitch = p.pool ? p.pool_pitch : 0;
   a.fd_tpi = make_fastdiv(static_cast<uint32_t>(p.pool ? p.pool_tpi : 1));
+  a.fd_pnw = make_fastdiv(static_cast<uint32_t>(p.pool ? p.pool_nw : 1));
+  a.fd_wo2 = make_fastdiv(static_cast<uint32_t>(p.pool ? p.Wo / 2 : 1));
   a.off_bar = p.off_bar;
   // A small layer gives each CTA at least T reference tiles of work (T from
   // samd_conv2d_set_min_tiles_per_cta; a reference tile is 128 positions of
@@ -856,7 +871,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   // on other streams. A tile of this layer weighs hv * nchunks * mma_n of
   // those 9 * 64, so layers with long reductions or many output channels
   // spread over more SMs.
-  const long long total_tiles = p.grid_m * p.nblocks;
+  const long long total_tiles = grid_m * p.nblocks;
   const long long ref_work = static_cast<long long>(g_min_tiles_per_cta.load(std::memory_order_relaxed)) * 9 * 64;
   long long tile_work = static_cast<long long>(p.hv) * p.nchunks * p.mma_n;
   // A gather tile with a short reduction (1x1 layers over few channels) is
@@ -867,6 +882,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   if (min_tiles < 1) min_tiles = 1;
   long long ctas = (total_tiles + min_tiles - 1) / min_tiles;
   if (ctas > sm_count()) ctas = sm_count();
+  if (pair) ctas = (ctas + 1) / 2 * 2 <= sm_count() ? (ctas + 1) / 2 * 2 : ctas / 2 * 2;
   dim3 grid(static_cast<unsigned>(ctas));
   // The next kernel of the stream may hold SMs while it waits for this one
   // to drain (one layer after another: ResNet-50 7x7 block 98.3 -> 92.4 us),

@@ -152,6 +152,7 @@ struct ConvArgs {
   int mma_n;        // MMA N: n_mma, or 2 * n_mma with split weight digits
   int split;        // 1: accumulator columns [0, n_mma) hold hi digits, [n_mma, 2 n_mma) lo digits
   int stages;       // weight stages in flight (or resident tiles)
+  int pair;         // 1: clusters of two CTAs share their streamed weights (each loads half of every tile for both)
   int tgroup;       // weight tiles of a stage: a filter row's (HALO, streamed weights) or 1
   int stages_a;     // GATHER: A tiles in flight
   int b_resident;   // 1: all weight tiles of the layer stay in shared memory
@@ -201,7 +202,8 @@ struct ConvArgs {
   // words of the channel block per row) and write only the lane-wise maxima
   // of the 2x2 windows, rows of (N, Ho / 2, Wo / 2) pixels, to packed_out.
   int pool, pool_rows, pool_nw, pool_pitch;
-  FastDiv fd_tpi;  // tiles per image
+  FastDiv fd_tpi;          // tiles per image
+  FastDiv fd_pnw, fd_wo2;  // / pool_nw, / (Wo / 2)
 };
 
 // First position, in the padded virtual grid N x Hv x Wp, of tile mt of a
@@ -598,6 +600,19 @@ __device__ __forceinline__ constexpr int32_t requant_addend(int bits, bool is_si
   return (is_signed ? 1 << (bits - 1) : 0) - kMagicBits;
 }
 
+// Requantizes columns FIRST .. FIRST + 15 of a 32-column group into the
+// group's words of 32 / OB offset patterns.
+template <int OB, bool OS, int FIRST, int NH>
+__device__ __forceinline__ void pack_16(const uint32_t (&r)[16], uint32_t (&h)[NH], float scale) {
+  constexpr int LH = 32 / OB;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int c = FIRST + k;
+    const uint32_t v = requant_lane(r[k], scale, requant_addend(OB, OS), (1 << OB) - 1) << ((c % LH) * OB);
+    h[c / LH] = c % LH == 0 ? v : h[c / LH] + v;
+  }
+}
+
 // What the epilogue of a row works on: rows are output pixels (m; ~0 for a
 // row outside the output, which only skips the stores), nvalid the channels
 // of this block from ch0 on. The first, store-free pass asks for one column
@@ -673,7 +688,6 @@ __device__ __forceinline__ void epilogue_row_spec(const ConvArgs &args, const Ep
   constexpr int LH = 32 / OB;  // lanes per 32-bit half-word (a divisor of 32: OB = 1, 2, 4, 7, 8)
   constexpr int NH = 32 / LH;  // half-words per 32-channel group
   static_assert(32 % LH == 0, "whole half-words per 32-channel group");
-  constexpr int32_t addend = requant_addend(OB, OS), omax = (1 << OB) - 1;
   constexpr uint32_t flip = OS ? LaneMsb<uint32_t, OB>::kValue : 0u;
   const float scale = args.out_scale;
   // 32-bit half-words of this row: output channel c sits in half-word c / LH
@@ -696,19 +710,11 @@ __device__ __forceinline__ void epilogue_row_spec(const ConvArgs &args, const Ep
   for (int col = 0; col < e.nvalid; col += 32) {
     const int cnt = e.nvalid - col < 32 ? e.nvalid - col : 32;
     uint32_t h[NH];
-    auto half = [&](const uint32_t (&r)[16], auto first) {  // columns first .. first + 15 of the group
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int c = decltype(first)::value + k;
-        const uint32_t v = requant_lane(r[k], scale, addend, omax) << ((c % LH) * OB);
-        h[c / LH] = c % LH == 0 ? v : h[c / LH] + v;
-      }
-    };
     load(col + 16, rb);
-    half(ra, std::integral_constant<int, 0>{});
+    pack_16<OB, OS, 0>(ra, h, scale);
     ptx::tmem_wait_ld(rb);
     load(col + 32, ra);
-    half(rb, std::integral_constant<int, 16>{});
+    pack_16<OB, OS, 16>(rb, h, scale);
 #pragma unroll
     for (int j = 0; j < NH; ++j) h[j] ^= flip;
     ptx::tmem_wait_ld(ra);
@@ -1035,7 +1041,6 @@ __device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t t
                                                 uint32_t &phase, int *status, int gw, int gi) {
   constexpr int LH = 32 / OB;  // lanes per word
   constexpr int NH = 32 / LH;  // words per 32 channels
-  constexpr int32_t addend = requant_addend(OB, OS), omax = (1 << OB) - 1;
   constexpr uint32_t flip = OS ? LaneMsb<uint32_t, OB>::kValue : 0u;
   const int ch0 = nb * args.NBc;
   const int nvalid = args.K - ch0 < args.NBc ? args.K - ch0 : args.NBc;
@@ -1043,23 +1048,31 @@ __device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t t
   const int pitch = args.pool_pitch;
   const float scale = args.out_scale;
   uint32_t *prow = pbuf + trow * pitch;
+  // 16 columns are packed while the next 16 are on their way
+  uint32_t ra[16], rb[16];
+  auto load = [&](int col, uint32_t (&r)[16]) {
+    ptx::tmem_ld_32x32b_x16(taddr + (col < args.n_mma ? col : 0), r);
+  };
+  load(0, ra);
+  ptx::tmem_wait_ld(ra);
   for (int col = 0; col < nvalid; col += 32) {
-    uint32_t r[32];
-    ptx::tmem_ld_32x32b_x32(taddr + col, r);
-    ptx::tmem_wait_ld(r);
     const int cnt = nvalid - col < 32 ? nvalid - col : 32;
+    uint32_t h[NH];
+    load(col + 16, rb);
+    pack_16<OB, OS, 0>(ra, h, scale);
+    ptx::tmem_wait_ld(rb);
+    load(col + 32, ra);
+    pack_16<OB, OS, 16>(rb, h, scale);
 #pragma unroll
     for (int j = 0; j < NH; ++j) {
-      uint32_t w = 0;
-#pragma unroll
-      for (int l = 0; l < LH; ++l) w += requant_lane(r[j * LH + l], scale, addend, omax) << (l * OB);
-      w ^= flip;
+      uint32_t w = h[j] ^ flip;
       const int wi = col / LH + j;
       // lanes past the block's channels are zero
       const int nl = cnt - j * LH;
       if (nl < LH) w &= nl > 0 ? (1u << (nl * OB)) - 1 : 0u;
       if (wi < nw) prow[wi] = w;
     }
+    ptx::tmem_wait_ld(ra);
   }
   ptx::tc_fence_before();
   __syncwarp();
@@ -1069,13 +1082,16 @@ __device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t t
   const uint32_t img = fdiv(mt, args.fd_tpi);
   const int g = static_cast<int>(mt - img * args.fd_tpi.d);
   const int Ho2 = args.Ho / 2, Wo2 = args.Wo / 2, q = args.pool_rows / 2;
-  const int q_here = Ho2 - g * q < q ? Ho2 - g * q : q;
-  const int total = q_here * Wo2 * nw;
+  int q_here = Ho2 - g * q < q ? Ho2 - g * q : q;
+  if (img >= static_cast<uint32_t>(args.N)) q_here = 0;  // the tile that makes the tiles' number even
+  const int total = q_here * Wo2 * args.pool_nw;
   uint32_t *out = static_cast<uint32_t *>(args.packed_out) + ch0 / LH;
   const int Wp = args.Wp;
+#pragma unroll 2
   for (int idx = 32 * gi + static_cast<int>(threadIdx.x & 31); idx < total; idx += 32 * gw) {
-    const int pix = idx / nw, w = idx - (idx / nw) * nw;
-    const int i = pix / Wo2, j = pix - (pix / Wo2) * Wo2;
+    const int pix = static_cast<int>(fdiv(static_cast<uint32_t>(idx), args.fd_pnw)), w = idx - pix * args.pool_nw;
+    if (w >= nw) continue;  // a last block of fewer words
+    const int i = static_cast<int>(fdiv(static_cast<uint32_t>(pix), args.fd_wo2)), j = pix - i * Wo2;
     const uint32_t *b0 = pbuf + (2 * i * Wp + 2 * j) * pitch + w;
     const uint32_t top = swar_lane_max<uint32_t, OB>(b0[0], b0[pitch], flip);
     const uint32_t bot = swar_lane_max<uint32_t, OB>(b0[Wp * pitch], b0[(Wp + 1) * pitch], flip);
@@ -1208,7 +1224,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   if (threadIdx.x == 32) {
     for (int s = 0; s < STB; ++s) {
       ptx::mbar_init(full_b(s), 1);
-      ptx::mbar_init(empty_b(s), 1);
+      ptx::mbar_init(empty_b(s), args.pair ? 2 : 1);  // the MMAs of every CTA that the stage's loads reach
     }
     for (int s = 0; s < NO; ++s) {
       ptx::mbar_init(opfull(s), (HALO || HV == 2) ? kProdWarps : kProdWarps / 2);
@@ -1226,6 +1242,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
+  if (args.pair) ptx::cluster_sync();  // the other CTA's barriers are set up
   const uint32_t tmem_base = *tmem_holder;
 
   // fewer than 2^31 tiles, and a CTA's last step stays below 2^31 + gridDim.x (checked on the host)
@@ -1250,6 +1267,11 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         // Ring position and round parity advance by increments (a 64-bit
         // division by the runtime ring size costs this thread about as much
         // as the rest of the step).
+        // The CTAs of a pair work on neighbouring position tiles of one
+        // channel block at the same time: each loads its half of every weight
+        // tile's rows into both, once both have consumed the stage.
+        const uint32_t half_row = args.pair ? ptx::cluster_rank() * (args.mma_n / 2) : 0u;
+        const uint32_t half_off = half_row * T::kRowBytes;
         int s = 0, loaded = 0;  // loaded: tiles issued so far, counted up to the ring's size
         uint32_t par = 1;       // parity of the previous round's release
         for (uint32_t tile = first_tile; tile < total_tiles; tile += tile_step) {
@@ -1261,8 +1283,13 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
               ++loaded;
             ptx::mbar_arrive_expect_tx(full_b(s), args.tgroup * b_bytes);
             const uint32_t dst = ptx::smem_addr(sB) + s * args.tgroup * b_bytes;
-            for (int g = 0; g < args.tgroup; ++g)
-              ptx::tma_load_2d(dst + g * b_bytes, &tmap_b, (c + g) * BK, row0, full_b(s));
+            for (int g = 0; g < args.tgroup; ++g) {
+              if (args.pair)
+                ptx::tma_load_2d_multicast(dst + g * b_bytes + half_off, &tmap_b, (c + g) * BK, row0 + half_row,
+                                           full_b(s), 3);
+              else
+                ptx::tma_load_2d(dst + g * b_bytes, &tmap_b, (c + g) * BK, row0, full_b(s));
+            }
             if (++s == STB) {
               s = 0;
               par ^= 1;
@@ -1276,6 +1303,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           int q = loaded == STB ? s + k : k;
           if (q >= STB) q -= STB;
           ptx::mbar_wait_bounded(full_b(q), q < s ? par ^ 1u : par, &quiet, kWaitLimitNs / 10);
+          // and, for a pair, both CTAs' arrivals on this one's barriers have come
+          if (args.pair) ptx::mbar_wait_bounded(empty_b(q), q < s ? par ^ 1u : par, &quiet, kWaitLimitNs);
         }
       }
     }
@@ -1370,7 +1399,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
                 wait(full_b(sb), bpar);
                 issue_row<FP8, HV, KS>(leader, tmem_d, dn, a_r, a_half16, bdesc0 + static_cast<uint32_t>(sb) * b_stage16,
                                        idesc, tgroup, a_row16, b_step16, acc);
-                ptx::mma_commit(leader, empty_b(sb));
+                if (args.pair)
+                  ptx::mma_commit_multicast(leader, empty_b(sb), 3);
+                else
+                  ptx::mma_commit(leader, empty_b(sb));
                 acc = 1;
                 a_r += static_cast<uint32_t>(tgroup) * a_row16;
                 if (++sb == STB) {
@@ -1730,6 +1762,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, args.tmem_cols);
   }
+  if (args.pair) {  // neither CTA exits while the other's loads and arrivals may still reach it
+    __syncwarp();
+    ptx::cluster_sync();
+  }
 }
 
 // cudaFuncSetAttribute once per (kernel, device); defined in conv2d.cu.
@@ -1771,7 +1807,7 @@ cudaError_t launch_conv(const CUtensorMap &tmap, const ConvArgs &args, bool halo
   // stream: barriers, tensor memory and the epilogue's code are set up while
   // that one drains; every role waits (grid_dependency_wait) before it reads
   // or writes global memory.
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
@@ -1781,6 +1817,12 @@ cudaError_t launch_conv(const CUtensorMap &tmap, const ConvArgs &args, bool halo
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (args.pair) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
   e = cudaLaunchKernelEx(&cfg, kern, tmap, args);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
