@@ -434,3 +434,25 @@ def test_conv_packed_rows_of_words(samd_lib, fo_bits, fo_signed):
 def test_conv_streamed_weights(samd_lib, ba, bw, R):
     shape = samd.ConvShape(2, 200, 9, 8, 264, R=R, S=R, pad=R // 2)
     run_conv_check(shape, ba, False, bw, True, fo_t=(ba, False, 0, 32), seed=synth.seed_for("str", ba, bw, R))
+
+
+# Unpack of 1-, 2- and 4-bit lanes stores 32 bytes at a time where the output
+# is aligned to that, and less elsewhere: both alignments, one quad of words
+# more or less than a step takes, guard bytes.
+@pytest.mark.parametrize("word_bits", (32, 64))
+@pytest.mark.parametrize("signed", SIGNS)
+@pytest.mark.parametrize("bits", (1, 2, 4))
+def test_unpack_whole_words_by_alignment(samd_lib, bits, signed, word_bits):
+    f = samd.fmt(bits, signed, 0, word_bits)
+    for words in (128, 128 * 2 + 1, 128 * 2500 + 77):
+        n = words * (32 // bits) + 5
+        v, b = values_and_bytes(synth.seed_for("ua", bits, signed, n), (n,), bits, signed)
+        packed = gpu_pack(b, f, 1, n)
+        for off in (0, 16):
+            buf = torch.full((n + 64,), 0x5A, dtype=torch.int8, device="cuda")
+            assert buf.data_ptr() % 32 == 0
+            samd.samd_unpack(f, packed, buf[off:], 1, n)
+            got = buf.cpu().numpy()
+            assert np.array_equal(got[off:off + n].astype(np.int64), v), (words, off)
+            assert (got[:off] == 0x5A).all() and (got[off + n:] == 0x5A).all()
+    assert_status_clean()
