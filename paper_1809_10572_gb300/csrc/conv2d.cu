@@ -239,6 +239,13 @@ std::atomic<int> g_min_tiles_per_cta{kDefaultMinTiles};
 samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, Plan &p, bool pool = false,
                       bool two_sided = false);
 
+// Whether parts of packed rows (NBc channels of a block) are worth staging:
+// 3-, 5- and 6-bit lanes in 32-bit words, at least 96 (5 bits) or 160 channels.
+bool staged_rows(samd_fmt fo, int NBc) {
+  return (fo.bits == 3 || fo.bits == 5 || fo.bits == 6) && fo.spacer == 0 && fo.word_bits == 32 &&
+         NBc >= (fo.bits == 5 ? 96 : 160);
+}
+
 // Most channels of a block, and the channels of a block: a whole number of
 // output words of Lo lanes.
 int block_limit(int split) { return split ? 128 : 256; }
@@ -458,7 +465,11 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
         p.b_resident = 1;
         p.stages = p.nchunks;
       } else {
-        long long st = static_cast<long long>((kBudget - fixed - bar_bytes(8, sta)) / bst);
+        // rows of several channel blocks leave through the epilogue's stage
+        // where two weight tiles still fit beside it
+        const size_t e_want = p.nblocks > 1 && staged_rows(fo, p.NBc) ? kEpiStageBytes : 0;
+        const size_t room = kBudget - fixed - bar_bytes(8, sta);
+        const long long st = static_cast<long long>((room >= e_want + 2 * bst ? room - e_want : room) / bst);
         p.stages = static_cast<int>(st > 8 ? 8 : st);
       }
       p.op_stride = static_cast<uint32_t>(tile_bytes);
@@ -534,7 +545,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
         p = whole;
       }
     }
-    if (!p.e_flat && p.NBc >= (fo.bits == 5 ? 96 : 160) && fits(kEpiStageBytes)) {
+    if (!p.e_flat && staged_rows(fo, p.NBc) && fits(kEpiStageBytes)) {
       p.e_stage = 1;
       reserve(kEpiStageBytes);
     }

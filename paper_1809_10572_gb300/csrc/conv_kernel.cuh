@@ -806,6 +806,14 @@ __device__ __forceinline__ void epilogue_row_words(const ConvArgs &args, const E
   const bool flat = args.e_flat != 0, by_rows = args.e_stage != 0;
   uint32_t *const mine = flat ? stg + __popc(vmask & ((1u << lane) - 1)) * nwords : stg + lane * kEpiPitch;
   auto load = [&](int c0, uint32_t (&r)[kCols]) {
+    if (c0 + kCols <= args.n_mma) {  // a whole group: two loads (each takes the warp about 27 cycles)
+      ptx::tmem_ld_32x32b_x16(e.taddr + c0, r);
+      if constexpr (kCols == 20)
+        ptx::tmem_ld_32x32b_x4(e.taddr + c0 + 16, r + 16);
+      else
+        ptx::tmem_ld_32x32b_x8(e.taddr + c0 + 16, r + 16);
+      return;
+    }
 #pragma unroll
     for (int q = 0; q < kCols; q += kPiece) {
       const int col = c0 + q < args.n_mma ? c0 + q : 0;  // past the last column: any, not stored
@@ -815,23 +823,30 @@ __device__ __forceinline__ void epilogue_row_words(const ConvArgs &args, const E
         ptx::tmem_ld_32x32b_x8(e.taddr + col, r + q);
     }
   };
+  // rows of a multiple of four words are staged 16 bytes at a time (13 such
+  // pieces a row of 256 6-bit channels: an odd number, so no bank conflicts)
+  const bool vec4 = kWords == 4 && flat && (nwords & 3) == 0;
+  uint32_t *const to = flat ? mine : own;
   auto group = [&](int c0, int w0, const uint32_t (&r)[kCols]) {
+    uint32_t w[kWords];
 #pragma unroll
     for (int j = 0; j < kWords; ++j) {
-      uint32_t w = 0;
+      w[j] = 0;
 #pragma unroll
-      for (int l = 0; l < L; ++l) w += requant_lane(r[j * L + l], scale, addend, omax) << (l * OB);
-      w ^= flip;
-      const int wi = w0 + j;
-      if (wi == nwords - 1) w &= last_mask;  // the row's last, partial word
-      if (wi < nwords) {
-        if (flat) {
-          if (e.valid()) mine[wi] = w;
-        } else if (by_rows) {
-          mine[wi & 31] = w;
-        } else if (e.valid()) {
-          own[wi] = w;
-        }
+      for (int l = 0; l < L; ++l) w[j] += requant_lane(r[j * L + l], scale, addend, omax) << (l * OB);
+      w[j] ^= flip;
+      if (w0 + j == nwords - 1) w[j] &= last_mask;  // the row's last, partial word
+    }
+    if (by_rows) {
+#pragma unroll
+      for (int j = 0; j < kWords; ++j) mine[(w0 + j) & 31] = w[j];
+    } else if (e.valid()) {
+      if (vec4) {
+        if constexpr (kWords == 4) *reinterpret_cast<uint4 *>(to + w0) = make_uint4(w[0], w[1], w[2], w[3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < kWords; ++j)
+          if (w0 + j < nwords) to[w0 + j] = w[j];
       }
     }
     if (by_rows && (((w0 + kWords) & 31) == 0 || c0 + kCols >= e.nvalid)) {
@@ -868,6 +883,7 @@ __device__ __forceinline__ void epilogue_row_words(const ConvArgs &args, const E
     int i = 0;
     if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
       i = total & ~3;
+#pragma unroll 4
       for (int k = 4 * lane; k < i; k += 128)
         *reinterpret_cast<uint4 *>(dst + k) = *reinterpret_cast<const uint4 *>(stg + k);
     }
