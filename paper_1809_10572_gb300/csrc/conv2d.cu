@@ -239,6 +239,7 @@ size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // s2, batch 64: 58.8 -> 32.9 us; 14x14 (1.15), 512 channels, u4 x s4, batch
 // 16: 35.1 -> 22.4 us.
 constexpr double kMaxHaloWaste = 1.35;
+constexpr size_t kBudget = 224 * 1024;  // shared memory: below the 227 KB opt-in limit minus static shared memory
 constexpr int kHaloGatherDepth = 2;  // packed staging slots of the halo producers (2..4)
 // minimum 128-pixel tiles per CTA of a launch (samd_conv2d_set_min_tiles_per_cta)
 constexpr int kDefaultMinTiles = 4;
@@ -344,7 +345,6 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   auto bar_bytes = [](int stages, int op_stages) {
     return round_up(static_cast<size_t>(2 * stages + 2 * op_stages + 7) * 8 + 4, 16);
   };
-  const size_t kBudget = 224 * 1024;  // below the 227 KB opt-in limit minus static shared memory
   auto finish = [&](size_t op_bytes, size_t g_bytes, int op_stages) {
     p.off_b = static_cast<uint32_t>(op_bytes);
     p.off_g = static_cast<uint32_t>(op_bytes + p.stages * p.tgroup * bst);
@@ -367,6 +367,13 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   p.Hv = d->H + (d->pad < d->R && !two_sided ? d->pad : 2 * d->pad);
   p.Wp = d->W + (d->pad < d->S && !two_sided ? d->pad : 2 * d->pad);
   const int nchunks_gather = p.nchunks;
+  // Streamed weights leave room for the epilogue's stage, where two (halo:
+  // three) stages of them still fit beside it: int32 rows that are not whole
+  // sectors leave through it, and a gather layer's packed rows of several
+  // channel blocks (a halo layer loses more by the weight stages that it
+  // costs: 7x7, 512 channels, u6 x s2 30.5 -> 31.8 us).
+  const size_t e_want =
+      !two_sided && !pool && ((p.nblocks > 1 && staged_rows(fo, p.NBc)) || d->K % 8 != 0) ? round_up(kEpiStageBytes, 16) : 0;
   // One configuration: operand mode (halo or gather) and tile halves hv.
   // Returns false if it does not fit, or if `need_resident` and the weights
   // would not stay resident.
@@ -453,9 +460,10 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
         // pool takes, count single tiles.
         const size_t pool_rows_bytes = pool ? round_up(static_cast<size_t>(2 * BM) * pool_pitch(p.NBc, fo) * 4, 16) : 0;
         const size_t all = kBudget - fixed - bar_bytes(8, hbufs);
-        const size_t room = all > pool_rows_bytes ? all - pool_rows_bytes : 0;
+        const size_t kept = pool_rows_bytes + (d->K % 8 != 0 && all >= e_want + 3 * bst ? e_want : 0);
+        const size_t room = all > kept ? all - kept : 0;
         p.tgroup = !two_sided && room / (d->S * bst) >= (pool ? 2 : 3) ? d->S : 1;
-        const long long st = static_cast<long long>((p.tgroup > 1 ? room : all) / (p.tgroup * bst));
+        const long long st = static_cast<long long>((p.tgroup > 1 || !pool ? room : all) / (p.tgroup * bst));
         const int most = p.tgroup > 1 ? 3 : 8;
         p.stages = static_cast<int>(st > most ? most : st);
       }
@@ -476,9 +484,6 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
         p.b_resident = 1;
         p.stages = p.nchunks;
       } else {
-        // rows of several channel blocks leave through the epilogue's stage
-        // where two weight tiles still fit beside it
-        const size_t e_want = p.nblocks > 1 && staged_rows(fo, p.NBc) ? kEpiStageBytes : 0;
         const size_t room = kBudget - fixed - bar_bytes(8, sta);
         const long long st = static_cast<long long>((room >= e_want + 2 * bst ? room - e_want : room) / bst);
         p.stages = static_cast<int>(st > 8 ? 8 : st);
@@ -893,7 +898,22 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.fd_tpi = make_fastdiv(static_cast<uint32_t>(p.pool ? p.pool_tpi : 1));
   a.fd_pnw = make_fastdiv(static_cast<uint32_t>(p.pool ? p.pool_nw : 1));
   a.fd_wo2 = make_fastdiv(static_cast<uint32_t>(p.pool ? p.Wo / 2 : 1));
-  a.off_bar = p.off_bar;
+  // The epilogue warps' stages: packed rows as planned, and int32 rows that
+  // are not whole 32-byte sectors, where the buffer fits.
+  a.e_words = p.e_flat ? 32 * static_cast<int>(words_per_row(fo, d->K)) : (p.e_stage ? 32 * kEpiPitch : 0);
+  a.acc_stage = 0;
+  size_t off_bar = p.off_bar, smem_bytes = p.smem_bytes;
+  if (acc_out && !nchw && (d->K % 8 != 0 || (reinterpret_cast<uintptr_t>(acc_out) & 31) != 0)) {
+    const int words = a.e_words > 32 * kEpiPitch ? a.e_words : 32 * kEpiPitch;
+    const size_t bar = round_up(p.off_e + static_cast<size_t>(kEpiWarps) * words * 4, 16);
+    if (p.smem_bytes - p.off_bar + bar <= kBudget) {
+      a.acc_stage = 1;
+      a.e_words = words;
+      smem_bytes = p.smem_bytes - p.off_bar + bar;
+      off_bar = bar;
+    }
+  }
+  a.off_bar = static_cast<uint32_t>(off_bar);
   // A small layer gives each CTA at least T reference tiles of work (T from
   // samd_conv2d_set_min_tiles_per_cta; a reference tile is 128 positions of
   // a 3x3 convolution over 64 input and 64 output channels: 9 operand rows of
@@ -933,7 +953,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   const int wi = fa.word_bits == 64 ? 1 : 0;
   if (p.fp8 && fa.bits > 5) return SAMD_EUNSUP;  // not reached: e4m3 only for |a| <= 16
   const LaunchFn fn = p.fp8 ? kF8[wi][fa.bits - 1] : kF16[wi][fa.bits - 1];
-  const cudaError_t e = fn(fa.is_signed != 0, tmap, a, p.halo != 0, grid, p.smem_bytes, s);
+  const cudaError_t e = fn(fa.is_signed != 0, tmap, a, p.halo != 0, grid, smem_bytes, s);
   return e == cudaSuccess ? SAMD_OK : SAMD_ECUDA;
 }
 

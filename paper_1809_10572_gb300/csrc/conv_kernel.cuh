@@ -193,6 +193,8 @@ struct ConvArgs {
   uint32_t off_b, b_bytes, off_g, g_stride, off_e, off_bar;
   int e_stage;  // 1: kEpiStageBytes at off_e stage 32 words of each 3/5/6-bit packed row (epilogue_row_words)
   int e_flat;   // 1: 32 whole rows per epilogue warp at off_e instead (one channel block)
+  int acc_stage;  // 1: int32 rows are staged too, 32 words of each (epilogue_row_acc)
+  int e_words;    // words of an epilogue warp's stage
   int early;    // 1: the next kernel of the stream may be set up while this one drains
   // Fused 2x2 max-pool (pool = 1; halo layers): tile mt is pool_rows output
   // rows (pool_rows / 2 row pairs) of one image from an even row on, at
@@ -892,65 +894,94 @@ __device__ __forceinline__ void epilogue_row_words(const ConvArgs &args, const E
   }
 }
 
-// Every other case, 16 columns at a time: split digits (acc = 16 hi + lo),
-// int32 outputs, accumulators too large for the fma path.
+// The exact integers of 16 accumulator columns (split digits: 16 hi + lo).
+__device__ __forceinline__ void exact_16(const ConvArgs &args, uint32_t taddr, int (&v)[16]) {
+  uint32_t r[16];
+  ptx::tmem_ld_32x32b_x16(taddr, r);
+  ptx::tmem_wait_ld(r);
+  if (args.split) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = 16 * __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
+    ptx::tmem_ld_32x32b_x16(taddr + args.n_mma, r);
+    ptx::tmem_wait_ld(r);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] += __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
+  } else if (args.fast_acc) {  // |acc| < 2^22: the exact integer from the float's encoding
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = floor_scaled_biased(__uint_as_float(r[k]), args.acc_scale) - kMagicBits;
+  } else {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
+  }
+}
+
+// int32 outputs: whole sectors of a thread's own row where rows are whole
+// sectors; otherwise 32 columns of the warp's rows are staged (acc_stage) and
+// written row by row, 32 consecutive words a store, or, without room for
+// that, one word at a time. 29 x 51 x 140 positions of 262 channels (217 MB),
+// with 3-bit packed rows: 451 us one word at a time, 242 this way.
+__device__ __forceinline__ void epilogue_row_acc(const ConvArgs &args, const EpiRow &e, uint32_t *stg) {
+  const bool vec_ok = args.K % 4 == 0 && e.ch0 % 4 == 0;
+  const bool vec8_ok = args.K % 8 == 0 && e.ch0 % 8 == 0 && (reinterpret_cast<uintptr_t>(args.acc_out) & 31) == 0;
+  const int lane = threadIdx.x & 31;
+  int32_t *const row = args.acc_out + (static_cast<size_t>(e.m) * args.K + e.ch0);
+  for (int col = 0; col < e.nvalid; col += 16) {
+    int v[16];
+    exact_16(args, e.taddr + col, v);
+    const int cnt = e.nvalid - col < 16 ? e.nvalid - col : 16;
+    if (args.acc_stage) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) stg[lane * kEpiPitch + (col & 16) + k] = static_cast<uint32_t>(v[k]);
+      if ((col & 16) == 0 && col + 16 < e.nvalid) continue;
+      __syncwarp();
+      const int c = (col & ~31) + lane;
+      const bool has = c < e.nvalid;
+#pragma unroll 4
+      for (int rr = 0; rr < 32; ++rr) {
+        const uint32_t mr = __shfl_sync(0xffffffffu, e.m, rr);
+        if (has && mr != ~0u)
+          args.acc_out[static_cast<size_t>(mr) * args.K + e.ch0 + c] = static_cast<int32_t>(stg[rr * kEpiPitch + lane]);
+      }
+      __syncwarp();
+      continue;
+    }
+    if (!e.valid()) continue;
+    int32_t *dst = row + col;
+    if (cnt == 16 && vec8_ok) {
+#pragma unroll
+      for (int k = 0; k < 16; k += 8)
+        ptx::st_global_v8(dst + k, v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4], v[k + 5], v[k + 6], v[k + 7]);
+    } else if (cnt == 16 && vec_ok) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        reinterpret_cast<int4 *>(dst)[k] = make_int4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (k < cnt) dst[k] = v[k];
+    }
+  }
+}
+
+// Packed rows that the fast forms do not take (split digits, |acc| / 2^shift
+// of 2^22 and more), 16 columns at a time.
 template <typename WO>
 __device__ __forceinline__ void epilogue_row_general(const ConvArgs &args, const EpiRow &e) {
-  const bool vec_ok = (args.K % 4 == 0) && (e.ch0 % 4 == 0);
-  const bool vec8_ok = (args.K % 8 == 0) && (e.ch0 % 8 == 0) && (reinterpret_cast<uintptr_t>(args.acc_out) & 31) == 0;
   const int lo = lane_lo(args.out_bits, args.out_signed), hi = lane_hi(args.out_bits, args.out_signed);
   const uint32_t omask = (1u << args.out_bits) - 1;
   const int L = args.out_L, lw = args.out_lane_w;
   RowPacker<WO> pk;
-  pk.dst = static_cast<WO *>(args.packed_out) + (static_cast<long long>(e.m) * args.out_wpr + e.ch0 / (L > 0 ? L : 1));
+  pk.dst = static_cast<WO *>(args.packed_out) + (static_cast<long long>(e.m) * args.out_wpr + e.ch0 / L);
   for (int col = 0; col < e.nvalid; col += 16) {
-    uint32_t r[16];
     int v[16];
-    ptx::tmem_ld_32x32b_x16(e.taddr + col, r);
-    if (args.split) {  // acc = 16 * hi + lo
-      uint32_t r2[16];
-      ptx::tmem_ld_32x32b_x16(e.taddr + args.n_mma + col, r2);
-      ptx::tmem_wait_ld(r);
-      ptx::tmem_wait_ld(r2);
-#pragma unroll
-      for (int k = 0; k < 16; ++k)
-        v[k] = 16 * __float2int_rn(__uint_as_float(r[k]) * args.acc_scale) +
-               __float2int_rn(__uint_as_float(r2[k]) * args.acc_scale);
-    } else {
-      ptx::tmem_wait_ld(r);
-      if (args.fast_acc) {  // |acc| < 2^22: the exact integer from the float's encoding
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = floor_scaled_biased(__uint_as_float(r[k]), args.acc_scale) - kMagicBits;
-      } else {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
-      }
-    }
+    exact_16(args, e.taddr + col, v);
     if (!e.valid()) continue;
     const int cnt = e.nvalid - col < 16 ? e.nvalid - col : 16;
-    if (args.acc_out) {
-      int32_t *dst = args.acc_out + static_cast<long long>(e.m) * args.K + e.ch0 + col;
-      if (cnt == 16 && vec8_ok) {  // whole 32-byte sectors
 #pragma unroll
-        for (int k = 0; k < 16; k += 8)
-          ptx::st_global_v8(dst + k, v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4], v[k + 5], v[k + 6], v[k + 7]);
-      } else if (cnt == 16 && vec_ok) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          reinterpret_cast<int4 *>(dst)[k] = make_int4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if (k < cnt) dst[k] = v[k];
-      }
-    }
-    if (args.packed_out) {
-#pragma unroll
-      for (int k = 0; k < 16; ++k)
-        if (k < cnt) pk.put(static_cast<uint32_t>(clamp_int(v[k] >> args.shift, lo, hi)) & omask, L, lw);
-    }
+    for (int k = 0; k < 16; ++k)
+      if (k < cnt) pk.put(static_cast<uint32_t>(clamp_int(v[k] >> args.shift, lo, hi)) & omask, L, lw);
   }
-  if (args.packed_out && e.valid()) pk.flush();
+  if (e.valid()) pk.flush();
 }
 
 // NCHW outputs: the 32 rows of a warp are neighbouring pixels, so for one
@@ -963,18 +994,8 @@ __device__ __forceinline__ void epilogue_row_nchw(const ConvArgs &args, const Ep
   const uint32_t img = e.valid() ? fdiv(e.m, args.fd_howo) : 0u;
   const size_t base = (static_cast<size_t>(img) * args.K + e.ch0) * howo + (e.m - img * howo);
   for (int col = 0; col < e.nvalid; col += 16) {
-    uint32_t r[16];
     int v[16];
-    ptx::tmem_ld_32x32b_x16(e.taddr + col, r);
-    ptx::tmem_wait_ld(r);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) v[k] = __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
-    if (args.split) {  // acc = 16 * hi + lo
-      ptx::tmem_ld_32x32b_x16(e.taddr + args.n_mma + col, r);
-      ptx::tmem_wait_ld(r);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = 16 * v[k] + __float2int_rn(__uint_as_float(r[k]) * args.acc_scale);
-    }
+    exact_16(args, e.taddr + col, v);
     if (!e.valid()) continue;
     const int cnt = e.nvalid - col < 16 ? e.nvalid - col : 16;
 #pragma unroll
@@ -992,7 +1013,11 @@ __device__ __forceinline__ void epilogue_row(const ConvArgs &args, const EpiRow 
     epilogue_row_nchw(args, e);
     return;
   }
-  const bool fast = args.packed_out && !args.acc_out && !args.split && args.fast_req;
+  // int32 sums and packed rows are two passes over the accumulator (reading it
+  // again costs less than packing by the general form)
+  if (args.acc_out) epilogue_row_acc(args, e, estage);
+  if (!args.packed_out) return;
+  const bool fast = !args.split && args.fast_req;
   if (fast && args.out_lane_w == args.out_bits && (!args.out_word64 || (args.out_bits & (args.out_bits - 1)) == 0)) {
     switch (args.out_bits * 2 + (args.out_signed ? 1 : 0)) {
       case 2: epilogue_row_spec<1, false>(args, e); return;
@@ -1683,8 +1708,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     const int quad = warp & 3;
     const int set = (warp - kFirstEpiWarp) / 4;
     uint32_t *const estage =
-        reinterpret_cast<uint32_t *>(smem + args.off_e) +
-        (warp - kFirstEpiWarp) * 32 * (args.e_flat ? args.out_wpr : kEpiPitch);  // unused without e_flat and e_stage
+        reinterpret_cast<uint32_t *>(smem + args.off_e) + (warp - kFirstEpiWarp) * args.e_words;
     const int row = quad * 32 + lane;
     constexpr int kTileStep = HV >= 2 ? 1 : 2;
     // parts of 128 rows of a tile this warp drains: set `set` takes parts

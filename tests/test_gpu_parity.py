@@ -456,3 +456,27 @@ def test_unpack_whole_words_by_alignment(samd_lib, bits, signed, word_bits):
             assert np.array_equal(got[off:off + n].astype(np.int64), v), (words, off)
             assert (got[:off] == 0x5A).all() and (got[off + n:] == 0x5A).all()
     assert_status_clean()
+
+
+# int32 rows that are not whole sectors are staged 32 channels at a time beside
+# the packed ones: channel counts at the edges of 16, 32 and a block, with and
+# without packed rows, on the grid and off it, split digits; guard words.
+@pytest.mark.parametrize("ba,bw,fo_bits", [(4, 3, 4), (6, 2, 6), (8, 8, 0), (3, 4, 3)])
+def test_conv_int32_rows(samd_lib, ba, bw, fo_bits):
+    for K, (HW, R) in itertools.product((1, 15, 17, 31, 33, 64, 100, 262, 300), [((9, 7), 3), ((13, 11), 1)]):
+        C = 300 if ba == 8 else 24
+        shape = samd.ConvShape(2, C, HW[0], HW[1], K, R=R, S=R, pad=R // 2)
+        a_v, w_v, a_w, w_w, fa, fw = conv_case(shape, ba, False, bw, True, synth.seed_for("i32", K, R, ba))
+        fo = samd.fmt(fo_bits, False) if fo_bits else None
+        shift = harness_shift(ba, bw, fo_bits or 8, C * R * R)
+        m = shape.N * shape.Ho * shape.Wo
+        acc = torch.full((m * K + 64,), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+        packed = samd.empty_words(fo, m, K) if fo else None
+        samd.samd_conv2d(shape.desc(), fa, a_w, fw, w_w, acc, fo, packed, shift, samd.conv_workspace(shape, fa, fw))
+        want = oracle_conv_nhwc(a_v, w_v, shape)
+        got = acc.cpu().numpy()
+        assert np.array_equal(got[:m * K].astype(np.int64), want.ravel()), (K, R)
+        assert (got[m * K:] == 0x5A5A5A5A).all()
+        if fo:
+            assert np.array_equal(np_words(packed, 32), oracle_requant_pack(want, shift, fo)), (K, R)
+    assert_status_clean()
