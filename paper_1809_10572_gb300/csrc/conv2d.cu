@@ -634,7 +634,7 @@ bool layout_ok(const Plan &p) {
 bool indexes_ok(const Plan &p, const samd_conv_desc *d) {
   return static_cast<long long>(d->N) * p.Hv * p.Wp + (p.nseg + 1) * static_cast<long long>(p.Wp) + kMaxHaloRows +
                  2 * BM < (1LL << 31) &&
-         p.M < (1LL << 31) && (p.grid_m + 1) * p.nblocks < (1LL << 31);
+         p.M < (1LL << 31) && p.grid_m * p.nblocks < (1LL << 31);
 }
 
 // Device address of a __device__ symbol in the current context, looked up
@@ -787,17 +787,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   const int esize = p.fp8 ? 1 : 2;
   cuuint64_t gdim[2] = {static_cast<cuuint64_t>(p.Kpad), static_cast<cuuint64_t>(rows_total)};
   cuuint64_t gstride[1] = {static_cast<cuuint64_t>(p.Kpad) * esize};
-  // Pairs of CTAs share the streamed weights of e4m3 halo layers of more than
-  // 128 columns, which pull them through L2 at its bandwidth (VGG-16 conv6:
-  // 240 MB in 27.0 us; 24.0 shared, conv9 31.0 -> 27.8, conv11 16.4 -> 15.5).
-  // fp16 layers (8-bit, 256 channels: 17.7 and 17.9 us), gather layers (131.7
-  // and 132.9 for the ResNet-50 28x28 block) and 128 columns (conv4 with its
-  // pool 30.3 and 31.9) do not gain. A pair's tiles lie in one channel block,
-  // so the position tiles are made even in number; the extra one holds no
-  // output.
-  const bool pair = p.fp8 && p.halo && !p.b_resident && p.mma_n > 128 && p.grid_m >= 2;
-  const long long grid_m = pair ? (p.grid_m + 1) / 2 * 2 : p.grid_m;
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(BK), static_cast<cuuint32_t>(pair ? p.mma_n / 2 : p.mma_n)};
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(BK), static_cast<cuuint32_t>(p.mma_n)};
   cuuint32_t estride[2] = {1, 1};
   CUresult cr = enc(&tmap, p.fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
                     const_cast<void *>(prepared), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -833,8 +823,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.stages = p.stages;
   a.stages_a = p.stages_a;
   a.b_resident = p.b_resident;
-  a.grid_m = grid_m;
-  a.pair = pair;
+  a.grid_m = p.grid_m;
   a.nblocks = p.nblocks;
   a.gather_vec = p.gather_vec;
   a.gather_win = p.gather_win;
@@ -879,7 +868,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.fd_wo = make_fastdiv(static_cast<uint32_t>(p.Wo));
   a.fd_ho = make_fastdiv(static_cast<uint32_t>(p.Ho));
   a.fd_howo = make_fastdiv(static_cast<uint32_t>(p.Ho) * static_cast<uint32_t>(p.Wo));
-  a.fd_gm = make_fastdiv(static_cast<uint32_t>(grid_m));
+  a.fd_gm = make_fastdiv(static_cast<uint32_t>(p.grid_m));
   a.op_stride = p.op_stride;
   a.off_b = p.off_b;
   a.b_bytes = p.b_bytes;
@@ -921,7 +910,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   // on other streams. A tile of this layer weighs hv * nchunks * mma_n of
   // those 9 * 64, so layers with long reductions or many output channels
   // spread over more SMs.
-  const long long total_tiles = grid_m * p.nblocks;
+  const long long total_tiles = p.grid_m * p.nblocks;
   const long long ref_work = static_cast<long long>(g_min_tiles_per_cta.load(std::memory_order_relaxed)) * 9 * 64;
   long long tile_work = static_cast<long long>(p.hv) * p.nchunks * p.mma_n;
   // A gather tile with a short reduction (1x1 layers over few channels) is
@@ -932,7 +921,6 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   if (min_tiles < 1) min_tiles = 1;
   long long ctas = (total_tiles + min_tiles - 1) / min_tiles;
   if (ctas > sm_count()) ctas = sm_count();
-  if (pair) ctas = (ctas + 1) / 2 * 2 <= sm_count() ? (ctas + 1) / 2 * 2 : ctas / 2 * 2;
   dim3 grid(static_cast<unsigned>(ctas));
   // The next kernel of the stream may hold SMs while it waits for this one
   // to drain (one layer after another: ResNet-50 7x7 block 98.3 -> 92.4 us),

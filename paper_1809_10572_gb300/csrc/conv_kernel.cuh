@@ -152,7 +152,6 @@ struct ConvArgs {
   int mma_n;        // MMA N: n_mma, or 2 * n_mma with split weight digits
   int split;        // 1: accumulator columns [0, n_mma) hold hi digits, [n_mma, 2 n_mma) lo digits
   int stages;       // weight stages in flight (or resident tiles)
-  int pair;         // 1: clusters of two CTAs share their streamed weights (each loads half of every tile for both)
   int tgroup;       // weight tiles of a stage: a filter row's (HALO, streamed weights) or 1
   int stages_a;     // GATHER: A tiles in flight
   int b_resident;   // 1: all weight tiles of the layer stay in shared memory
@@ -1123,8 +1122,7 @@ __device__ __noinline__ void epilogue_pool_tile(const ConvArgs &args, uint32_t t
   const uint32_t img = fdiv(mt, args.fd_tpi);
   const int g = static_cast<int>(mt - img * args.fd_tpi.d);
   const int Ho2 = args.Ho / 2, Wo2 = args.Wo / 2, q = args.pool_rows / 2;
-  int q_here = Ho2 - g * q < q ? Ho2 - g * q : q;
-  if (img >= static_cast<uint32_t>(args.N)) q_here = 0;  // the tile that makes the tiles' number even
+  const int q_here = Ho2 - g * q < q ? Ho2 - g * q : q;
   const int total = q_here * Wo2 * args.pool_nw;
   uint32_t *out = static_cast<uint32_t *>(args.packed_out) + ch0 / LH;
   const int Wp = args.Wp;
@@ -1265,7 +1263,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   if (threadIdx.x == 32) {
     for (int s = 0; s < STB; ++s) {
       ptx::mbar_init(full_b(s), 1);
-      ptx::mbar_init(empty_b(s), args.pair ? 2 : 1);  // the MMAs of every CTA that the stage's loads reach
+      ptx::mbar_init(empty_b(s), 1);
     }
     for (int s = 0; s < NO; ++s) {
       ptx::mbar_init(opfull(s), (HALO || HV == 2) ? kProdWarps : kProdWarps / 2);
@@ -1283,7 +1281,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  if (args.pair) ptx::cluster_sync();  // the other CTA's barriers are set up
   const uint32_t tmem_base = *tmem_holder;
 
   // fewer than 2^31 tiles, and a CTA's last step stays below 2^31 + gridDim.x (checked on the host)
@@ -1308,11 +1305,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         // Ring position and round parity advance by increments (a 64-bit
         // division by the runtime ring size costs this thread about as much
         // as the rest of the step).
-        // The CTAs of a pair work on neighbouring position tiles of one
-        // channel block at the same time: each loads its half of every weight
-        // tile's rows into both, once both have consumed the stage.
-        const uint32_t half_row = args.pair ? ptx::cluster_rank() * (args.mma_n / 2) : 0u;
-        const uint32_t half_off = half_row * T::kRowBytes;
         int s = 0, loaded = 0;  // loaded: tiles issued so far, counted up to the ring's size
         uint32_t par = 1;       // parity of the previous round's release
         for (uint32_t tile = first_tile; tile < total_tiles; tile += tile_step) {
@@ -1324,13 +1316,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
               ++loaded;
             ptx::mbar_arrive_expect_tx(full_b(s), args.tgroup * b_bytes);
             const uint32_t dst = ptx::smem_addr(sB) + s * args.tgroup * b_bytes;
-            for (int g = 0; g < args.tgroup; ++g) {
-              if (args.pair)
-                ptx::tma_load_2d_multicast(dst + g * b_bytes + half_off, &tmap_b, (c + g) * BK, row0 + half_row,
-                                           full_b(s), 3);
-              else
-                ptx::tma_load_2d(dst + g * b_bytes, &tmap_b, (c + g) * BK, row0, full_b(s));
-            }
+            for (int g = 0; g < args.tgroup; ++g)
+              ptx::tma_load_2d(dst + g * b_bytes, &tmap_b, (c + g) * BK, row0, full_b(s));
             if (++s == STB) {
               s = 0;
               par ^= 1;
@@ -1344,8 +1331,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           int q = loaded == STB ? s + k : k;
           if (q >= STB) q -= STB;
           ptx::mbar_wait_bounded(full_b(q), q < s ? par ^ 1u : par, &quiet, kWaitLimitNs / 10);
-          // and, for a pair, both CTAs' arrivals on this one's barriers have come
-          if (args.pair) ptx::mbar_wait_bounded(empty_b(q), q < s ? par ^ 1u : par, &quiet, kWaitLimitNs);
         }
       }
     }
@@ -1440,10 +1425,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
                 wait(full_b(sb), bpar);
                 issue_row<FP8, HV, KS>(leader, tmem_d, dn, a_r, a_half16, bdesc0 + static_cast<uint32_t>(sb) * b_stage16,
                                        idesc, tgroup, a_row16, b_step16, acc);
-                if (args.pair)
-                  ptx::mma_commit_multicast(leader, empty_b(sb), 3);
-                else
-                  ptx::mma_commit(leader, empty_b(sb));
+                ptx::mma_commit(leader, empty_b(sb));
                 acc = 1;
                 a_r += static_cast<uint32_t>(tgroup) * a_row16;
                 if (++sb == STB) {
@@ -1802,10 +1784,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, args.tmem_cols);
   }
-  if (args.pair) {  // neither CTA exits while the other's loads and arrivals may still reach it
-    __syncwarp();
-    ptx::cluster_sync();
-  }
 }
 
 // cudaFuncSetAttribute once per (kernel, device); defined in conv2d.cu.
@@ -1847,7 +1825,7 @@ cudaError_t launch_conv(const CUtensorMap &tmap, const ConvArgs &args, bool halo
   // stream: barriers, tensor memory and the epilogue's code are set up while
   // that one drains; every role waits (grid_dependency_wait) before it reads
   // or writes global memory.
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
@@ -1857,12 +1835,6 @@ cudaError_t launch_conv(const CUtensorMap &tmap, const ConvArgs &args, bool halo
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (args.pair) {
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.numAttrs = 2;
-  }
   e = cudaLaunchKernelEx(&cfg, kern, tmap, args);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

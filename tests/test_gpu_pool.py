@@ -122,11 +122,11 @@ def test_fused_pool_vgg16_layers_full_batch(samd_lib, name):
     assert_status_clean()
 
 
-# Layers whose streamed weights two CTAs share (e4m3, more than 128 columns): an
-# odd number of tiles, so that one of a pair holds no output, one channel
-# block and two, pooled and not, more tiles than CTAs.
+# Layers of more than 128 columns with streamed weights (e4m3): an odd number
+# of tiles and an even one, one channel block and two, pooled and not, more
+# tiles than CTAs.
 @pytest.mark.parametrize("shape", [samd.ConvShape(1, 160, 28, 28, 256), samd.ConvShape(3, 160, 28, 28, 264),
                                    samd.ConvShape(28, 72, 28, 28, 250)],
                          ids=lambda v: f"{v.N}x{v.C}x{v.H}x{v.W}-K{v.K}")
-def test_pooled_and_plain_layers_of_shared_weights(samd_lib, shape):
+def test_pooled_and_plain_layers_of_streamed_weights(samd_lib, shape):
     run_pool_case(shape, 4, False, 4, True, samd.fmt(4, False), synth.seed_for("pair", shape))

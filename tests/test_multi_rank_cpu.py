@@ -64,3 +64,14 @@ def test_reference_arm_under_torchrun_prints_once():
     line = json.loads(lines[0])
     assert line["impl"] == "reference" and line["n_gpus"] == 2 and line["value"] > 0
     assert line["cpu_baseline"]["kind"] == "oracle" and line["e2e"]["h2d_bytes_per_step"] == 0
+
+
+def test_library_sources_use_no_cluster_multicast():
+    """Every rank of a run on several GPUs loads this library, and copies with
+    cluster multicast are for code that runs on one GPU alone."""
+    csrc = os.path.join(ROOT, "paper_1809_10572_gb300", "csrc")
+    names = sorted(os.listdir(csrc))
+    assert "tc_ptx.cuh" in names
+    for name in names:
+        with open(os.path.join(csrc, name)) as f:
+            assert "multicast" not in f.read(), name
