@@ -636,7 +636,12 @@ __device__ __forceinline__ EpiRow epi_row(const ConvArgs &args, uint32_t taddr, 
 
 // Epilogue of one accumulator row of a channel block: fp32 accumulators ->
 // exact integers -> optional int32 store, optional requantize-and-pack.
-// Called by whole warps (tcgen05.ld is collective).
+// Called by whole warps. tcgen05.ld is collective, and lanes make or skip
+// their stores by their own row: a __syncwarp before the next load converges
+// the warp (nothing else would guarantee it), or, in the loops that it would
+// slow down (epilogue_row_words: ResNet-50 56x56 block 123 -> 128 us;
+// epilogue_row_acc), the stores are predicated and the warp never branches
+// apart.
 //
 // Formats with spacers or 64-bit words of 3, 5, 6 or 7 bits: packed output
 // only, no split digits, |acc| / 2^shift < 2^22.
@@ -650,6 +655,7 @@ __device__ __forceinline__ void epilogue_row_fast(const ConvArgs &args, const Ep
   WO *const row = static_cast<WO *>(args.packed_out) + (static_cast<long long>(e.m) * args.out_wpr + e.ch0 / L);
   pk.dst = row;
   for (int col = 0; col < e.nvalid; col += 32) {
+    __syncwarp();
     uint32_t y[32];
     ptx::tmem_ld_32x32b_x32(e.taddr + col, y);
     ptx::tmem_wait_ld(y);
@@ -706,9 +712,11 @@ __device__ __forceinline__ void epilogue_row_spec(const ConvArgs &args, const Ep
   auto load = [&](int col, uint32_t (&r)[16]) {
     ptx::tmem_ld_32x32b_x16(e.taddr + (col < args.n_mma ? col : 0), r);
   };
+  __syncwarp();
   load(0, ra);
   ptx::tmem_wait_ld(ra);
   for (int col = 0; col < e.nvalid; col += 32) {
+    __syncwarp();
     const int cnt = e.nvalid - col < 32 ? e.nvalid - col : 32;
     uint32_t h[NH];
     load(col + 16, rb);
@@ -841,14 +849,11 @@ __device__ __forceinline__ void epilogue_row_words(const ConvArgs &args, const E
     if (by_rows) {
 #pragma unroll
       for (int j = 0; j < kWords; ++j) mine[(w0 + j) & 31] = w[j];
-    } else if (e.valid()) {
-      if (vec4) {
-        if constexpr (kWords == 4) *reinterpret_cast<uint4 *>(to + w0) = make_uint4(w[0], w[1], w[2], w[3]);
-      } else {
+    } else if (vec4) {
+      if constexpr (kWords == 4) ptx::st_v4_if(e.valid(), to + w0, w[0], w[1], w[2], w[3]);
+    } else {
 #pragma unroll
-        for (int j = 0; j < kWords; ++j)
-          if (w0 + j < nwords) to[w0 + j] = w[j];
-      }
+      for (int j = 0; j < kWords; ++j) ptx::st_if(e.valid() && w0 + j < nwords, to + w0 + j, w[j]);
     }
     if (by_rows && (((w0 + kWords) & 31) == 0 || c0 + kCols >= e.nvalid)) {
       __syncwarp();
@@ -923,7 +928,7 @@ __device__ __forceinline__ void epilogue_row_acc(const ConvArgs &args, const Epi
   const bool vec_ok = args.K % 4 == 0 && e.ch0 % 4 == 0;
   const bool vec8_ok = args.K % 8 == 0 && e.ch0 % 8 == 0 && (reinterpret_cast<uintptr_t>(args.acc_out) & 31) == 0;
   const int lane = threadIdx.x & 31;
-  int32_t *const row = args.acc_out + (static_cast<size_t>(e.m) * args.K + e.ch0);
+  uint32_t *const row = reinterpret_cast<uint32_t *>(args.acc_out) + (static_cast<size_t>(e.m) * args.K + e.ch0);
   for (int col = 0; col < e.nvalid; col += 16) {
     int v[16];
     exact_16(args, e.taddr + col, v);
@@ -944,20 +949,17 @@ __device__ __forceinline__ void epilogue_row_acc(const ConvArgs &args, const Epi
       __syncwarp();
       continue;
     }
-    if (!e.valid()) continue;
-    int32_t *dst = row + col;
+    uint32_t *dst = row + col;
     if (cnt == 16 && vec8_ok) {
 #pragma unroll
       for (int k = 0; k < 16; k += 8)
-        ptx::st_global_v8(dst + k, v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4], v[k + 5], v[k + 6], v[k + 7]);
+        ptx::st_global_v8_if(e.valid(), dst + k, v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4], v[k + 5], v[k + 6], v[k + 7]);
     } else if (cnt == 16 && vec_ok) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        reinterpret_cast<int4 *>(dst)[k] = make_int4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+      for (int k = 0; k < 16; k += 4) ptx::st_v4_if(e.valid(), dst + k, v[k], v[k + 1], v[k + 2], v[k + 3]);
     } else {
 #pragma unroll
-      for (int k = 0; k < 16; ++k)
-        if (k < cnt) dst[k] = v[k];
+      for (int k = 0; k < 16; ++k) ptx::st_if(e.valid() && k < cnt, dst + k, v[k]);
     }
   }
 }
@@ -973,6 +975,7 @@ __device__ __forceinline__ void epilogue_row_general(const ConvArgs &args, const
   pk.dst = static_cast<WO *>(args.packed_out) + (static_cast<long long>(e.m) * args.out_wpr + e.ch0 / L);
   for (int col = 0; col < e.nvalid; col += 16) {
     int v[16];
+    __syncwarp();
     exact_16(args, e.taddr + col, v);
     if (!e.valid()) continue;
     const int cnt = e.nvalid - col < 16 ? e.nvalid - col : 16;
@@ -994,6 +997,7 @@ __device__ __forceinline__ void epilogue_row_nchw(const ConvArgs &args, const Ep
   const size_t base = (static_cast<size_t>(img) * args.K + e.ch0) * howo + (e.m - img * howo);
   for (int col = 0; col < e.nvalid; col += 16) {
     int v[16];
+    __syncwarp();
     exact_16(args, e.taddr + col, v);
     if (!e.valid()) continue;
     const int cnt = e.nvalid - col < 16 ? e.nvalid - col : 16;
@@ -1008,6 +1012,7 @@ __device__ __forceinline__ void epilogue_row_nchw(const ConvArgs &args, const Ep
 }
 
 __device__ __forceinline__ void epilogue_row(const ConvArgs &args, const EpiRow &e, uint32_t *estage) {
+  __syncwarp();  // the stores of the part before
   if (args.nchw) {
     epilogue_row_nchw(args, e);
     return;
@@ -1051,9 +1056,18 @@ __device__ __forceinline__ void epilogue_row(const ConvArgs &args, const EpiRow 
   }
 }
 
-// A role's wait on one of the kernel's barriers, by whole warps.
+// A role's wait on one of the kernel's barriers, by whole warps or one lane:
+// every lane polls for itself.
 __device__ __forceinline__ void role_wait(uint32_t bar, uint32_t parity, int *status) {
   ptx::mbar_wait(bar, parity, status, static_cast<int>(SAMD_ETIMEOUT), kWaitLimitNs);
+}
+
+// The epilogue warps' wait: converged again behind it, as the collective
+// tcgen05.ld needs (the MMA and producer warps have a __syncwarp, or nothing
+// collective, behind theirs).
+__device__ __forceinline__ void epi_wait(uint32_t bar, uint32_t parity, int *status) {
+  role_wait(bar, parity, status);
+  __syncwarp();
 }
 
 // The epilogue warps' meeting point of a pooled tile: every warp of the
@@ -1062,9 +1076,8 @@ __device__ __forceinline__ void role_wait(uint32_t bar, uint32_t parity, int *st
 __device__ __forceinline__ void epi_group_sync(uint32_t bar, uint32_t &phase, int *status) {
   __syncwarp();
   if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(bar);
-  role_wait(bar, phase & 1u, status);
+  epi_wait(bar, phase & 1u, status);
   ++phase;
-  __syncwarp();
 }
 
 // Epilogue of one pooled tile for output lanes of OB = 1, 2, 4 or 8 bits
@@ -1722,7 +1735,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         for (uint32_t tile = first_tile + (HV == 2 ? 0 : set) * tile_step; tile < total_tiles;
              tile += kStep * tile_step, ip += kStep) {
           const int acc_i = HV == 2 ? static_cast<int>(ip & 1) : set;
-          role_wait(accfull(acc_i), (ip >> 1) & 1u, status);
+          epi_wait(accfull(acc_i), (ip >> 1) & 1u, status);
           ptx::tc_fence_after();
           const uint32_t nbu = fdiv(tile, args.fd_gm);
           const uint32_t mt = tile - nbu * args.fd_gm.d;
@@ -1736,7 +1749,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     for (uint32_t tile = first_tile + (HV >= 2 ? 0 : set) * tile_step; !pooled && tile < total_tiles;) {
       const int acc_i = HV >= 2 ? static_cast<int>(i & 1) : set;  // accumulator of this tile
       if (!warm) {
-        role_wait(accfull(acc_i), (i >> 1) & 1u, status);
+        epi_wait(accfull(acc_i), (i >> 1) & 1u, status);
         ptx::tc_fence_after();
       }
       const uint32_t nbu = fdiv(tile, args.fd_gm);

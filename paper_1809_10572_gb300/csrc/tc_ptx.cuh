@@ -143,6 +143,36 @@ __device__ __forceinline__ void st_global_v8(void *dst, uint32_t v0, uint32_t v1
                : "memory");
 }
 
+// Stores (generic addresses) that a lane makes only with `on` set, by a
+// predicate and not a branch: the warp stays converged.
+__device__ __forceinline__ void st_if(bool on, uint32_t *p, uint32_t v) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.u32 q, %0, 0;\n\t"
+      "@q st.b32 [%1], %2;\n\t}" ::"r"(static_cast<uint32_t>(on)),
+      "l"(p), "r"(v)
+      : "memory");
+}
+__device__ __forceinline__ void st_v4_if(bool on, uint32_t *p, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.u32 q, %0, 0;\n\t"
+      "@q st.v4.b32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(static_cast<uint32_t>(on)),
+      "l"(p), "r"(v0), "r"(v1), "r"(v2), "r"(v3)
+      : "memory");
+}
+
+// (dst in global memory, 32-byte aligned)
+__device__ __forceinline__ void st_global_v8_if(bool on, void *dst, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3,
+                                                uint32_t v4, uint32_t v5, uint32_t v6, uint32_t v7) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.u32 q, %0, 0;\n\t"
+      "@q st.global.v8.b32 [%1], {%2, %3, %4, %5, %6, %7, %8, %9};\n\t}" ::"r"(static_cast<uint32_t>(on)),
+      "l"(dst), "r"(v0), "r"(v1), "r"(v2), "r"(v3), "r"(v4), "r"(v5), "r"(v6), "r"(v7)
+      : "memory");
+}
+
 // ---- TMA -------------------------------------------------------------------
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int x, int y, uint32_t bar) {
