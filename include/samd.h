@@ -168,7 +168,9 @@ typedef struct {
  * other streams run beside it.
  * Other limits (SAMD_EUNSUP): spacer 0 for fa and fw; R, S <= 16.
  * A kernel that gives up on a bounded wait leaves its outputs undefined and
- * records SAMD_ETIMEOUT for samd_device_status.
+ * records SAMD_ETIMEOUT for samd_device_status. Until that is reset, later
+ * convolutions on the device may give up as well, on any wait longer than
+ * about 20 us.
  */
 SAMD_API samd_status samd_conv2d(const samd_conv_desc *desc, samd_fmt fa, const void *act, samd_fmt fw, const void *wt,
                         int32_t *acc_out, samd_fmt fo, void *packed_out, int shift, void *workspace,
@@ -283,11 +285,11 @@ SAMD_API samd_status samd_device_status(int *status, int reset, samd_stream_t st
 
 /*
  * samd_selftest_wait_timeout: exercises the failure path of the bounded waits
- * without faulting the GPU. Launches one block on `stream` whose thread waits
- * on an mbarrier phase that nothing completes; after limit_ns nanoseconds
- * (1000 .. 2e9, else SAMD_EINVAL) the wait gives up and records
- * SAMD_ETIMEOUT in the sticky status read by samd_device_status, as a
- * convolution role that gives up does. The context stays usable. Asynchronous.
+ * without faulting the GPU. Launches one block on `stream` whose warp waits,
+ * by the convolution roles' own wait, on an mbarrier phase that nothing
+ * completes; after limit_ns nanoseconds (1000 .. 2e9, else SAMD_EINVAL) the
+ * wait gives up and records SAMD_ETIMEOUT in the sticky status read by
+ * samd_device_status. The context stays usable. Asynchronous.
  */
 SAMD_API samd_status samd_selftest_wait_timeout(uint64_t limit_ns, samd_stream_t stream);
 

@@ -1056,27 +1056,31 @@ __device__ __forceinline__ void epilogue_row(const ConvArgs &args, const EpiRow 
   }
 }
 
-// A role's wait on one of the kernel's barriers, by whole warps or one lane:
-// every lane polls for itself.
-__device__ __forceinline__ void role_wait(uint32_t bar, uint32_t parity, int *status) {
-  ptx::mbar_wait(bar, parity, status, static_cast<int>(SAMD_ETIMEOUT), kWaitLimitNs);
+// A role's wait on one of the kernel's barriers. A role whose wait gives up
+// (false) stops: the loader and the epilogue at once, the MMA warp and the
+// producers at the end of a tile or a few items, filling and releasing every
+// stage in step until there (with undefined values). The others' waits then
+// give up in turn, within one poll of the failure's being recorded, and the
+// kernel ends with what was in flight drained.
+__device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, int *status, uint64_t limit_ns = kWaitLimitNs) {
+  return ptx::mbar_wait(bar, parity, status, static_cast<int>(SAMD_ETIMEOUT), limit_ns);
 }
 
-// The epilogue warps' wait: converged again behind it, as the collective
-// tcgen05.ld needs (the MMA and producer warps have a __syncwarp, or nothing
-// collective, behind theirs).
-__device__ __forceinline__ void epi_wait(uint32_t bar, uint32_t parity, int *status) {
-  role_wait(bar, parity, status);
-  __syncwarp();
+// The same by a whole warp, every lane polling for itself: one answer for all,
+// and the warp is converged again behind it (the collective tcgen05.ld needs
+// that).
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, int *status, uint64_t limit_ns = kWaitLimitNs) {
+  return __all_sync(0xffffffffu, role_wait(bar, parity, status, limit_ns));
 }
 
 // The epilogue warps' meeting point of a pooled tile: every warp of the
 // tile's group arrives on `bar` once its part of the step is done, then
-// waits, bounded, for the phase.
+// waits, bounded, for the phase. (One that gives up goes on to the end of its
+// tile: what it reads and writes there is in bounds, and undefined.)
 __device__ __forceinline__ void epi_group_sync(uint32_t bar, uint32_t &phase, int *status) {
   __syncwarp();
   if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(bar);
-  epi_wait(bar, phase & 1u, status);
+  (void)warp_wait(bar, phase & 1u, status);
   ++phase;
 }
 
@@ -1232,7 +1236,8 @@ __device__ __forceinline__ void issue_row(uint32_t leader, uint32_t d, uint32_t 
 //               first, store-free pass over the first tile fetches the
 //               epilogue's code early. Pooled tiles (ConvArgs::pool) are
 //               drained, requantized and pooled by the warps of a group.
-// Every wait is bounded; one that gives up records SAMD_ETIMEOUT (role_wait).
+// Every wait is bounded; a role whose wait gives up records SAMD_ETIMEOUT and
+// stops (role_wait).
 template <typename W, int BITS, bool SIGNED, bool HALO, bool FP8, bool FULL, int HV>
 __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                                            const ConvArgs args) {
@@ -1320,13 +1325,19 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         // as the rest of the step).
         int s = 0, loaded = 0;  // loaded: tiles issued so far, counted up to the ring's size
         uint32_t par = 1;       // parity of the previous round's release
-        for (uint32_t tile = first_tile; tile < total_tiles; tile += tile_step) {
+        // A stage is armed again when its copies have landed and the MMAs have
+        // released it. (Those waited for the copies too, unless that wait gave
+        // up; a barrier armed twice in one phase would be lost.)
+        bool ok = true;
+        for (uint32_t tile = first_tile; ok && tile < total_tiles; tile += tile_step) {
           const int row0 = static_cast<int>(fdiv(tile, args.fd_gm)) * args.mma_n;
           for (int c = 0; c < nchunks; c += args.tgroup) {
-            if (loaded == STB)
-              role_wait(empty_b(s), par, status);
-            else
+            if (loaded == STB) {
+              ok = role_wait(full_b(s), par, status) && role_wait(empty_b(s), par, status);
+              if (!ok) break;
+            } else {
               ++loaded;
+            }
             ptx::mbar_arrive_expect_tx(full_b(s), args.tgroup * b_bytes);
             const uint32_t dst = ptx::smem_addr(sB) + s * args.tgroup * b_bytes;
             for (int g = 0; g < args.tgroup; ++g)
@@ -1357,7 +1368,13 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     // each MMA, which costs more than the MMA.
     const uint32_t leader = ptx::elect_one() ? 1u : 0u;
     const uint32_t idesc = ptx::idesc_f16_f32(BM, args.mma_n);
-    auto wait = [&](uint32_t bar, uint32_t parity) { role_wait(bar, parity, status); };
+    // A wait that gives up ends the loop behind its tile: an exit at the wait,
+    // or a leader that depends on it, costs the loop its uniform registers
+    // (sweep step 122 -> 139 us).
+    bool gave_up = false;
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+      if (!role_wait(bar, parity, status)) gave_up = true;
+    };
     // Ring positions advance by increments (no division in this loop).
     int sb = 0, so = 0;
     uint32_t bpar = 0, opar = 0;
@@ -1470,6 +1487,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         }
       }
       ptx::mma_commit(leader, accfull(a));
+      if (__any_sync(0xffffffffu, gave_up)) break;
     }
     ptx::mma_commit(leader, drain_bar);
     __syncwarp();
@@ -1483,6 +1501,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     const int t = threadIdx.x - 64;  // 0 .. kProdThreads - 1
     const W *act = static_cast<const W *>(args.act);
     ptx::grid_dependency_wait();  // the activations
+    bool gave_up = false;  // looked at behind a tile, or a few items: a vote on every item costs time
     if constexpr (HALO) {
       const int halo_rows = args.nseg * args.seg_rows;
       // Input pixels of this thread's halo rows in the tile being gathered
@@ -1570,7 +1589,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
           ptx::cp_async_wait<2>();
         else
           ptx::cp_async_wait<1>();  // item k of this thread's rows has landed
-        if (reused) role_wait(opempty(hb), hpar, status);
+        if (reused && !role_wait(opempty(hb), hpar, status)) gave_up = true;
         const uint8_t *stg = sG + cslot * args.g_stride;
         for (int hr = t; hr < halo_rows; hr += kProdThreads) {
           W cur[WC];
@@ -1581,6 +1600,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(opfull(hb));
         advance(ctile, cj);
+        if (cj == 0 && __any_sync(0xffffffffu, gave_up)) break;
         if (++cslot == D) cslot = 0;
         if (++hb == NO) {
           hb = 0;
@@ -1676,13 +1696,16 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         } else {
           load_staged<W, WC>(srow, cur);
         }
-        if (reused) role_wait(opempty(sa), apar, status);
+        if (reused && !role_wait(opempty(sa), apar, status)) gave_up = true;
         U::unpack_row(cur, sOp + sa * args.op_stride, row);
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(opfull(sa));
         issue_next(slot);  // refill the slot just read
-        if (++slot == kGatherDepth) slot = 0;
+        if (++slot == kGatherDepth) {
+          slot = 0;
+          if (__any_sync(0xffffffffu, gave_up)) break;
+        }
         sa += kItemStep;
         if (sa >= NO) {
           sa -= NO;
@@ -1735,7 +1758,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
         for (uint32_t tile = first_tile + (HV == 2 ? 0 : set) * tile_step; tile < total_tiles;
              tile += kStep * tile_step, ip += kStep) {
           const int acc_i = HV == 2 ? static_cast<int>(ip & 1) : set;
-          epi_wait(accfull(acc_i), (ip >> 1) & 1u, status);
+          if (!warp_wait(accfull(acc_i), (ip >> 1) & 1u, status)) break;
           ptx::tc_fence_after();
           const uint32_t nbu = fdiv(tile, args.fd_gm);
           const uint32_t mt = tile - nbu * args.fd_gm.d;
@@ -1749,7 +1772,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     for (uint32_t tile = first_tile + (HV >= 2 ? 0 : set) * tile_step; !pooled && tile < total_tiles;) {
       const int acc_i = HV >= 2 ? static_cast<int>(i & 1) : set;  // accumulator of this tile
       if (!warm) {
-        epi_wait(accfull(acc_i), (i >> 1) & 1u, status);
+        if (!warp_wait(accfull(acc_i), (i >> 1) & 1u, status)) break;
         ptx::tc_fence_after();
       }
       const uint32_t nbu = fdiv(tile, args.fd_gm);

@@ -85,23 +85,21 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   }
 }
 
-// The kernel roles' wait, executed by whole warps (every lane polls): a wait
-// that gives up records `code` in *status and returns like any other, so that
-// the callers' control flow does not depend on the outcome and stays uniform
-// (the compiler keeps ring positions and descriptors in uniform registers).
-// The loops of a failed launch run on to their end without waiting longer
-// than one poll; their results are undefined, as the status says.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int *status, int code, uint64_t limit_ns) {
+// The kernel roles' wait: one that runs out records `code` in *status. False
+// if it ran out or another wait's failure was recorded meanwhile (or by an
+// earlier launch and not reset); the caller then issues nothing more.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int *status, int code, uint64_t limit_ns) {
   if (__builtin_expect(!mbar_try_wait(bar, parity), 0)) {
     const uint64_t t0 = global_timer_ns();
     while (!mbar_try_wait_hint(bar, parity, 20000u)) {
-      if (*static_cast<volatile int *>(status) != 0) break;
+      if (*static_cast<volatile int *>(status) != 0) return false;
       if (global_timer_ns() - t0 > limit_ns) {
         atomicOr(status, code);
-        break;
+        return false;
       }
     }
   }
+  return true;
 }
 
 // ---- programmatic dependent launch -----------------------------------------

@@ -279,6 +279,46 @@ def test_bounded_wait_timeout_is_recorded_and_the_context_survives(samd_lib):
     assert e.value.status == samd.SAMD_EINVAL
 
 
+# A role whose wait gives up stops, and with it the launch: with a failure on
+# record every wait of more than a poll (20 us) gives up, and these layers'
+# first tiles take longer. The launch ends by itself, writes nothing outside
+# its output and not all of that, and after a reset the same call gives the
+# words that it gave before. Several tiles a CTA; streamed weights by the halo
+# and the gather form, one and two channel blocks, and pooled.
+@pytest.mark.parametrize("shape,ba,bw,pool", [(samd.ConvShape(128, 2048, 14, 14, 512), 4, 4, False),
+                                              (samd.ConvShape(64, 1024, 28, 28, 1000, stride=2), 6, 2, False),
+                                              (samd.ConvShape(64, 2048, 28, 28, 256), 4, 4, True)],
+                         ids=lambda v: f"{v.N}x{v.C}x{v.H}x{v.W}-K{v.K}" if isinstance(v, samd.ConvShape) else None)
+def test_a_launch_whose_waits_give_up_ends_and_the_next_is_exact(samd_lib, shape, ba, bw, pool):
+    assert samd.samd_device_status() == samd.SAMD_OK
+    fa, fw = samd.fmt(ba, False), samd.fmt(bw, True)
+    a_w = samd.pack(synth.to_bytes_t(synth.lanes_t(31, (shape.N * shape.H * shape.W, shape.C), ba, False, device="cuda")), fa)
+    w_w = samd.pack(synth.to_bytes_t(synth.lanes_t(32, (shape.K * shape.R * shape.S, shape.C), bw, True, device="cuda")), fw)
+    fo, shift = (samd.fmt(4, True), 14) if pool else (samd.fmt(8, True), 11)  # sums of about -70000, or -145000
+    conv = samd.PreparedConv(w_w, shape, fa, fw, fo)
+    rows = shape.N * (shape.Ho // 2) * (shape.Wo // 2) if pool else shape.N * shape.Ho * shape.Wo
+    n = samd.samd_packed_words(fo, rows, shape.K)
+
+    def run():
+        buf = torch.full((n + 64,), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+        if pool:
+            conv.pool2x2(a_w, buf[:n], shift)
+        else:
+            conv(a_w, None, buf[:n], shift)
+        torch.cuda.synchronize()
+        assert bool((buf[n:] == 0x5A5A5A5A).all())
+        return buf[:n]
+
+    want = run()
+    assert samd.samd_device_status() == samd.SAMD_OK
+    samd.samd_selftest_wait_timeout(100_000)
+    got = run()
+    assert samd.samd_device_status(reset=True) == samd.SAMD_ETIMEOUT
+    assert bool((got == 0x5A5A5A5A).any())
+    assert torch.equal(run(), want)
+    assert samd.samd_device_status() == samd.SAMD_OK
+
+
 # 1x1 layers whose packed pixel rows are not 16-byte multiples take the
 # gather through 16-byte windows: rows at every 4-byte offset, the last chunk
 # of a pixel running past its words, stride 2, 64-bit words, and the last
