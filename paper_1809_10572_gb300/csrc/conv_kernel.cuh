@@ -1390,6 +1390,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     constexpr uint64_t a_half16 = static_cast<uint64_t>(BM) * a_row16;  // from one 128-row part's A rows to the next
     const uint32_t dn = static_cast<uint32_t>(args.mma_n);          // the second half's accumulator columns
     const uint32_t a_skip16 = HALO ? static_cast<uint32_t>(args.row_step - args.S) * a_row16 : 0u;
+    // The first wait's limit counts from here on, not from the launch: the
+    // kernel before this one may run on long after it let this one in.
+    ptx::grid_dependency_wait();
     if (resident)  // resident weights: wait for all of them once
       for (int c = 0; c < nchunks; ++c) wait(full_b(c), 0);
     uint32_t i = 0;
@@ -1860,7 +1863,7 @@ cudaError_t launch_conv(const CUtensorMap &tmap, const ConvArgs &args, bool halo
   // Launched as a programmatic dependent of the kernel before it in the
   // stream: barriers, tensor memory and the epilogue's code are set up while
   // that one drains; every role waits (grid_dependency_wait) before it reads
-  // or writes global memory.
+  // or writes global memory, or waits for another role.
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
