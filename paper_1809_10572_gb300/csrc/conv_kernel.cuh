@@ -656,8 +656,11 @@ __device__ __forceinline__ void epilogue_row_fast(const ConvArgs &args, const Ep
   pk.dst = row;
   for (int col = 0; col < e.nvalid; col += 32) {
     __syncwarp();
+    // the block's MMA columns are a multiple of 16; past them, which may be
+    // past this CTA's tensor memory, the first ones are read again
     uint32_t y[32];
-    ptx::tmem_ld_32x32b_x32(e.taddr + col, y);
+    ptx::tmem_ld_32x32b_x16(e.taddr + col, y);
+    ptx::tmem_ld_32x32b_x16(e.taddr + (col + 16 < args.n_mma ? col + 16 : 0), y + 16);
     ptx::tmem_wait_ld(y);
     const int cnt = e.nvalid - col < 32 ? e.nvalid - col : 32;
 #pragma unroll

@@ -372,6 +372,26 @@ def test_conv_packed_only_outputs_partial_groups(samd_lib, fo_bits, fo_signed):
     assert_status_clean()
 
 
+# At most 16 output channels: two accumulators of the fewest tensor-memory
+# columns, by the form that packs any format (spacers, 64-bit words of 3, 5, 6
+# and 7 bits), in tiles of two and of four parts, several a CTA.
+@pytest.mark.parametrize("fo_t", [(3, True, 0, 64), (5, False, 0, 64), (6, True, 0, 64), (7, False, 0, 64), (4, False, 1, 32),
+                                  (2, True, 3, 64)])
+@pytest.mark.parametrize("K", (1, 5, 16))
+def test_conv_packed_few_channels(samd_lib, K, fo_t):
+    for shape in (samd.ConvShape(4, 16, 40, 41, K), samd.ConvShape(4, 48, 33, 30, K, R=1, S=1, pad=0),
+                  samd.ConvShape(2, 3, 400, 401, K)):
+        a_v, w_v, a_w, w_w, fa, fw = conv_case(shape, 4, False, 3, True, synth.seed_for("few", shape, fo_t[0]))
+        fo = samd.fmt(*fo_t)
+        shift = harness_shift(4, 3, fo.bits, shape.C * shape.R * shape.S)
+        n = samd.samd_packed_words(fo, shape.N * shape.Ho * shape.Wo, K)
+        buf = torch.full((n + 64,), 0x5A5A5A5A, dtype=samd.word_dtype(fo), device="cuda")
+        samd.samd_conv2d(shape.desc(), fa, a_w, fw, w_w, None, fo, buf, shift, samd.conv_workspace(shape, fa, fw))
+        assert np.array_equal(np_words(buf[:n], fo.word_bits), oracle_requant_pack(oracle_conv_nhwc(a_v, w_v, shape), shift, fo))
+        assert bool((buf[n:] == 0x5A5A5A5A).all())
+    assert_status_clean()
+
+
 # 64-bit output words of 1-, 2-, 4- and 8-bit lanes are written as 32-bit
 # halves: a last word whose channels end in its low half must still be whole.
 @pytest.mark.parametrize("fo_bits,K", [(1, 16), (1, 70), (2, 16), (2, 40), (4, 24), (4, 290), (8, 20), (8, 33)])
