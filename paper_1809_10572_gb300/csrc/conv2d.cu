@@ -1058,9 +1058,28 @@ cudaError_t launch_repack(const samd_conv_desc *d, samd_fmt fa, const void *act,
 }  // namespace
 }  // namespace conv
 
-// An NCHW layer whose sums the tensor cores hold exactly and whose repacked
-// activations, widened weights and requantized bytes fit the caller's
-// workspace (sized for the wide-multiply engine) runs as the NHWC kernel
+// The parts of the workspace of an NCHW layer on the tensor cores.
+struct NchwBuffers {
+  size_t act, wt, bytes;
+};
+
+// Whether the tensor cores take an NCHW layer: they hold its sums exactly
+// (below 2^24, or in two weight digits), and its repacked activations, widened
+// weights and requantized bytes (fo.bits != 0) fit the workspace, which is
+// sized for the wide-multiply engine. That leaves the engine the layers of few
+// input channels against the output's, and sums of 2^24 and more with weights
+// of up to 4 bits.
+bool nchw_on_tensor_cores(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fmt fo, size_t workspace_bytes,
+                          conv::Plan &p, NchwBuffers &b) {
+  using namespace conv;
+  if (make_plan(d, fa, fw, none_fmt(), p) != SAMD_OK || !layout_ok(p) || !indexes_ok(p, d) || p.M == 0) return false;
+  b.act = round_up(static_cast<size_t>(d->N) * d->H * d->W * p.wpr * (fa.word_bits / 8), 256);
+  b.wt = round_up(p.ws_bytes, 256);
+  b.bytes = fo.bits ? static_cast<size_t>(p.M) * d->K : 0;
+  return b.act + b.wt + b.bytes <= workspace_bytes;
+}
+
+// A layer that nchw_on_tensor_cores takes runs as the NHWC kernel
 // between two changes of layout: repacked activations in, NCHW outputs out
 // (the int32 sums to acc_out, and, where packed rows are wanted (fo.bits != 0),
 // the requantized lanes one per byte to *q8 in the workspace, for the caller
@@ -1073,14 +1092,11 @@ samd_status conv2d_nchw_tc(const samd_conv_desc *d, samd_fmt fa, const void *act
   using namespace conv;
   *taken = false;
   Plan p;
-  if (make_plan(d, fa, fw, none_fmt(), p) != SAMD_OK || !layout_ok(p) || !indexes_ok(p, d) || p.M == 0) return SAMD_OK;
-  const size_t act_bytes = round_up(static_cast<size_t>(d->N) * d->H * d->W * p.wpr * (fa.word_bits / 8), 256);
-  const size_t wt_bytes = round_up(p.ws_bytes, 256);
-  const size_t q_bytes = fo.bits ? static_cast<size_t>(p.M) * d->K : 0;
-  if (act_bytes + wt_bytes + q_bytes > workspace_bytes) return SAMD_OK;
+  NchwBuffers b;
+  if (!nchw_on_tensor_cores(d, fa, fw, fo, workspace_bytes, p, b)) return SAMD_OK;
   *taken = true;
-  uint8_t *const px = static_cast<uint8_t *>(workspace), *const wp = px + act_bytes;
-  uint8_t *const bytes = fo.bits ? wp + wt_bytes : nullptr;
+  uint8_t *const px = static_cast<uint8_t *>(workspace), *const wp = px + b.act;
+  uint8_t *const bytes = fo.bits ? wp + b.wt : nullptr;
   *q8 = reinterpret_cast<const int8_t *>(bytes);
   const cudaError_t e =
       fa.word_bits == 32 ? launch_repack<uint32_t>(d, fa, act, px, s) : launch_repack<uint64_t>(d, fa, act, px, s);

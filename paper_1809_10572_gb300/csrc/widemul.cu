@@ -10,9 +10,10 @@
 //
 // This runs on the CUDA cores (64 x 64 -> 128-bit multiplies, which the GPU
 // builds from 32-bit multiply-adds); it is the paper's engine, and the path of
-// the NCHW layers that the tensor cores cannot take (conv2d_nchw_tc): sums
-// of 2^24 and more, and layers whose operands in the NHWC form do not fit the
-// workspace, which is this engine's.
+// the NCHW layers that the tensor cores do not take (nchw_on_tensor_cores in
+// conv2d.cu): sums of 2^24 and more with weights of up to 4 bits, and layers
+// whose operands in the NHWC form do not fit the workspace, which is this
+// engine's.
 //
 // Plan (host): bound = R*S*C*max|a|*max|w| (no partial or final sum exceeds
 // it), F = bits(bound) + 1, nx = floor(64 / F) input positions per word,
@@ -245,9 +246,7 @@ samd_status conv2d_nchw(const samd_conv_desc *d, samd_fmt fa, const void *act, s
   if (packed_out && static_cast<size_t>(g.Wo) * kWarps > 48 * 1024) return SAMD_EUNSUP;  // row buffers
   const long long rows = static_cast<long long>(d->N) * d->K * g.Ho;
   if (rows == 0) return SAMD_OK;
-  // the tensor cores where they hold the sums exactly and the workspace their
-  // operands; the multiplies below take the rest (sums of 2^24 and more, few
-  // input channels against the output's)
+  // the tensor cores where they take the layer; the multiplies below do the rest
   bool taken = false;
   const int8_t *q8 = nullptr;
   st = conv2d_nchw_tc(d, fa, act, fw, wt, acc_out, packed_out ? fo : samd_fmt{0, 0, 0, 0}, shift, workspace,

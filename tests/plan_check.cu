@@ -5,26 +5,9 @@
 // launchers are replaced by stubs (nothing is launched).
 #include "../paper_1809_10572_gb300/csrc/conv2d.cu"
 
-#define SAMD_STUB(name)                                                                                      \
-  namespace samd {                                                                                           \
-  namespace conv {                                                                                           \
-  cudaError_t name(bool, const CUtensorMap &, const ConvArgs &, bool, dim3, size_t, cudaStream_t) {          \
-    return cudaErrorInvalidValue;                                                                            \
-  }                                                                                                          \
-  }                                                                                                          \
-  }
-SAMD_STUB(launch_conv_f16_w32_b1) SAMD_STUB(launch_conv_f16_w32_b2) SAMD_STUB(launch_conv_f16_w32_b3)
-SAMD_STUB(launch_conv_f16_w32_b4) SAMD_STUB(launch_conv_f16_w32_b5) SAMD_STUB(launch_conv_f16_w32_b6)
-SAMD_STUB(launch_conv_f16_w32_b7) SAMD_STUB(launch_conv_f16_w32_b8) SAMD_STUB(launch_conv_f16_w64_b1)
-SAMD_STUB(launch_conv_f16_w64_b2) SAMD_STUB(launch_conv_f16_w64_b3) SAMD_STUB(launch_conv_f16_w64_b4)
-SAMD_STUB(launch_conv_f16_w64_b5) SAMD_STUB(launch_conv_f16_w64_b6) SAMD_STUB(launch_conv_f16_w64_b7)
-SAMD_STUB(launch_conv_f16_w64_b8) SAMD_STUB(launch_conv_f8_w32_b1) SAMD_STUB(launch_conv_f8_w32_b2)
-SAMD_STUB(launch_conv_f8_w32_b3) SAMD_STUB(launch_conv_f8_w32_b4) SAMD_STUB(launch_conv_f8_w32_b5)
-SAMD_STUB(launch_conv_f8_w64_b1) SAMD_STUB(launch_conv_f8_w64_b2) SAMD_STUB(launch_conv_f8_w64_b3)
-SAMD_STUB(launch_conv_f8_w64_b4) SAMD_STUB(launch_conv_f8_w64_b5)
+#include "conv_stubs.cuh"
 
 namespace samd {
-int sm_count() { return 152; }  // defined in samd_api.cu, not linked here
 // the NCHW path lives in widemul.cu, not linked here
 samd_status conv2d_nchw_check(const samd_conv_desc *, samd_fmt, samd_fmt, samd_fmt, size_t *) { return SAMD_EUNSUP; }
 samd_status conv2d_nchw(const samd_conv_desc *, samd_fmt, const void *, samd_fmt, const void *, int32_t *, samd_fmt,

@@ -1,15 +1,18 @@
 """GPU parity of the NCHW convolution: tensors packed along the image width
 (rows of W lanes, the layout of the paper's Fig. 12 x-loop), computed by the
-paper's wide-multiply engine (section 5.1 with the Fig. 10 sign extension
-and Fig. 11 repair) on the CUDA cores. Compared with the CPU oracle's direct
-convolution element by element; the requantized output packed along W
-against the oracle's requantize + pack."""
+tensor-core kernel between two changes of layout where it takes the layer, and
+by the paper's wide-multiply engine (section 5.1 with the Fig. 10 sign
+extension and Fig. 11 repair) on the CUDA cores otherwise; the layers of
+tests/nchw_cases.py are known to take one or the other. Compared with the CPU
+oracle's direct convolution element by element; the requantized output packed
+along W against the oracle's requantize + pack."""
 import numpy as np
 import pytest
 import torch
 
+import nchw_cases
 import oracle
-from gpu_util import assert_status_clean, np_words, values_and_bytes
+from gpu_util import assert_status_clean, harness_shift, np_words, values_and_bytes
 from paper_1809_10572_gb300 import samd, synth
 
 pytestmark = pytest.mark.gpu
@@ -144,7 +147,26 @@ def test_nchw_both_routes(samd_lib, ba, sa, bw, sw, word_bits):
               wt_gen=lambda s, v=wmin: np.full(s, v, np.int64))
 
 
-# Sums of 2^24 and more are beyond the tensor cores' exact range.
+# Random lanes, and the extremes: every lane at its most negative value (the
+# largest sums, every borrow repaired), and that value next to zero and to the
+# other extreme along the row (coefficients of zero beside negative ones: the
+# double increment of section 6), on both routes.
+@pytest.mark.parametrize("route", ("ENGINE", "TENSOR"))
+def test_nchw_random_and_extreme_values_by_route(samd_lib, route):
+    for shape, ba, sa, bw, sw, wb, fo_bits in getattr(nchw_cases, route):
+        fo = samd.fmt(fo_bits, sa, 0, wb) if fo_bits else None
+        shift = harness_shift(ba, bw, fo_bits or 8, shape.C * shape.R * shape.S)
+        check(shape, ba, sa, bw, sw, synth.seed_for("route", shape, ba, bw), fo=fo, shift=shift, word_bits=wb)
+        amin, amax = (-(1 << (ba - 1)), (1 << (ba - 1)) - 1) if sa else ((1 << ba) - 1, 0)
+        wext = -(1 << (bw - 1)) if sw else (1 << bw) - 1
+        for other in {amin, 0, amax}:
+            check(shape, ba, sa, bw, sw, 0, fo=fo, shift=shift, word_bits=wb,
+                  act_gen=lambda s, o=other: np.where(np.arange(np.prod(s)).reshape(s) % 2 == 0, amin, o),
+                  wt_gen=lambda s: np.full(s, wext, np.int64))
+
+
+# Sums of 2^24 and more with 4-bit weights are beyond the tensor cores' exact
+# range (wider weights are split into two digits).
 def test_nchw_large_sums(samd_lib):
     shape = samd.ConvShape(1, 2100, 3, 9, 2, R=2, S=2, pad=0)
     check(shape, 8, False, 4, True, 5, act_gen=lambda s: np.full(s, 255, np.int64),

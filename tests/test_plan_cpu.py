@@ -8,30 +8,45 @@ import tempfile
 
 import pytest
 
+import nchw_cases
 from paper_1809_10572_gb300 import build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-def test_every_plan_fits_and_does_not_overlap():
+def run_host_program(name, stdin=""):
+    """Compiles tests/<name>.cu for the host and runs it."""
     try:
         nvcc = build.nvcc()
     except RuntimeError:
         pytest.skip("nvcc not available")
     with tempfile.TemporaryDirectory(prefix="samd_plan_") as tmp:
-        exe = os.path.join(tmp, "plan_check")
+        exe = os.path.join(tmp, name)
         cmd = [nvcc] + build.ARCH + ["-O2", "-std=c++17", "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include"),
-                                     os.path.join(ROOT, "tests", "plan_check.cu"), "-o", exe, "-lcuda"]
+                                     os.path.join(ROOT, "tests", name + ".cu"), "-o", exe, "-lcuda"]
         r = subprocess.run(cmd, capture_output=True, text=True)
         assert r.returncode == 0, r.stderr[-2000:]
-        r = subprocess.run([exe], capture_output=True, text=True, timeout=600)
-        assert r.returncode == 0, r.stdout[-2000:]
-        assert "bad 0" in r.stdout
-        # the grid reaches every planning mode
-        for mode in ("halo", "segmented", "e4m3", "resident", "two-half", "four-part", "window gather", "staging at the chosen depth",
-                     "staged epilogue"):
-            count = int(r.stdout.split(mode)[1].split()[0].strip("(),"))
-            assert count > 0, (mode, r.stdout)
+        return subprocess.run([exe], capture_output=True, text=True, timeout=600, input=stdin)
+
+
+def test_nchw_cases_take_their_routes():
+    cases = nchw_cases.ENGINE + nchw_cases.TENSOR
+    lines = [" ".join(map(str, (s.N, s.C, s.H, s.W, s.K, s.R, s.S, s.pad, ba, int(sa), bw, int(sw), wb, fo)))
+             for s, ba, sa, bw, sw, wb, fo in cases]
+    r = run_host_program("nchw_route", "\n".join(lines) + "\n")
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split() == ["engine"] * len(nchw_cases.ENGINE) + ["tensor"] * len(nchw_cases.TENSOR)
+
+
+def test_every_plan_fits_and_does_not_overlap():
+    r = run_host_program("plan_check")
+    assert r.returncode == 0, r.stdout[-2000:]
+    assert "bad 0" in r.stdout
+    # the grid reaches every planning mode
+    for mode in ("halo", "segmented", "e4m3", "resident", "two-half", "four-part", "window gather", "staging at the chosen depth",
+                 "staged epilogue"):
+        count = int(r.stdout.split(mode)[1].split()[0].strip("(),"))
+        assert count > 0, (mode, r.stdout)
 
 
 @pytest.mark.parametrize("N,H,W,R,S,pad", [(2, 3, 4, 3, 3, 1), (3, 1, 1, 3, 3, 1), (2, 5, 4, 5, 5, 2), (2, 4, 3, 3, 3, 2),
