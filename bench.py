@@ -458,11 +458,12 @@ def time_packed_ops(dev, flush):
     return res
 
 
-def time_nchw_widemul(dev):
-    """The paper's wide-multiply engine (NCHW packed along W, CUDA cores) on
-    the sweep's 3x3 C64 -> 64 56x56 layer at batch 8, for the lane widths whose
-    kernel row fits one 64-bit word: effective MAC/s, beside the tensor-core
-    path's per-layer rates."""
+def time_nchw(dev):
+    """One NCHW call (tensors packed along W, packed output) of the sweep's 3x3
+    C64 -> 64 56x56 layer at batch 8, for the lane widths that NCHW layers of
+    this shape take: effective MAC/s. These layers run on the tensor cores
+    between two changes of layout, four launches a call; the wide-multiply
+    engine is not timed here."""
     import torch
 
     from paper_1809_10572_gb300 import samd, synth
@@ -797,7 +798,7 @@ def run_samd(args, layers):
                                        "timing": "8 launches back to back over rotating buffer sets of more than "
                                                  "twice the L2 (write-back of each output inside the timed region); "
                                                  "L2 flushed first"}
-        line["nchw_widemul_mac_s"] = time_nchw_widemul(dev)
+        line["nchw_mac_s"] = time_nchw(dev)
     line["clocks"] = clk
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
         v, cores, sample = cpu_oracle_rate(layers, args.cpu_seconds)

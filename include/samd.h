@@ -143,7 +143,7 @@ typedef struct {
  *   acc[n][k][ho][wo] = sum_{c,r,s} act[n][c][ho*stride-pad+r][wo*stride-pad+s] * wt[k][c][r][s]
  * (cross-correlation; taps outside the image read zero), computed exactly
  * in int32.
- * Layout SAMD_NHWC (the one implemented): act is N*H*W rows of C elements
+ * Layout SAMD_NHWC: act is N*H*W rows of C elements
  * packed along C with format fa; wt is K*R*S rows of C elements packed
  * along C with format fw ([K][R][S][C]). Outputs, each optional (NULL to
  * skip, but not both):
@@ -151,9 +151,16 @@ typedef struct {
  *   packed_out  N*Ho*Wo rows of K elements packed along K with format fo,
  *               each element clamp_fo(floor(acc / 2^shift)) (the requantize
  *               epilogue; an unsigned fo doubles as ReLU).
+ * Layout SAMD_NCHW (stride 1; S fields of bits(R*S*C * max|a| * max|w|) + 1
+ * bits within 64, else SAMD_EUNSUP): act is N*C*H rows of W elements, wt
+ * K*C*R rows of S elements, acc_out int32 [N][K][Ho][Wo], packed_out N*K*Ho
+ * rows of Wo elements. Layers that fit the workspace run on the tensor cores
+ * between two changes of layout, the others by wide multiplies; the results
+ * are the same.
  * workspace / workspace_bytes: caller-owned device scratch of at least
  * samd_conv2d_workspace_size(...) bytes (16-byte aligned) that receives the
- * weights in the tensor-core operand layout on every call.
+ * weights in the tensor-core operand layout on every call (SAMD_NCHW: both
+ * operands).
  * Exactness: the sum runs on the tensor cores with fp32 accumulation, exact
  * while every partial sum stays below 2^24, over e4m3 operands when
  * max|a| <= 16 and max|w| <= 16 (lanes of up to 4 bits, and signed 5-bit
@@ -194,7 +201,9 @@ SAMD_API samd_status samd_conv2d_set_min_tiles_per_cta(int tiles);
 
 /* Width in bits of the tensor-core operands samd_conv2d uses for this shape
  * and these formats: 8 (e4m3), 16 (fp16), or 0 if the convolution is
- * rejected (invalid arguments or SAMD_EUNSUP). Host-only; no GPU needed. */
+ * rejected (invalid arguments or SAMD_EUNSUP). SAMD_NCHW: 64 (the words of
+ * the wide-multiply engine, whose limits such a layer has to keep) whichever
+ * way the layer then runs, or 0. Host-only; no GPU needed. */
 SAMD_API int samd_conv2d_operand_bits(const samd_conv_desc *desc, samd_fmt fa, samd_fmt fw);
 
 /*
