@@ -23,8 +23,9 @@
  *   canonical.
  * - Sizes of zero are valid and launch nothing.
  *
- * Thread safety: entry points keep no host state except a per-device cache
- * of kernel attributes, guarded by a mutex.
+ * Thread safety: entry points keep no host state except caches of device and
+ * kernel properties, guarded by mutexes, and the setting of
+ * samd_conv2d_set_min_tiles_per_cta.
  */
 #ifndef SAMD_H_
 #define SAMD_H_
@@ -114,7 +115,8 @@ typedef enum {
  * samd_elementwise: lane-wise op over n elements packed as one row
  * (rows = 1, inner = n).
  *   a, b, out  packed arrays; b is read only by ADD/SUB/MUL (NULL otherwise)
- *              and has format fa. out may alias a or b.
+ *              and has format fa. out may alias a or b, except where
+ *              REQUANT changes the lanes per word.
  *   fo         output format: must equal fa for ADD/SUB/MUL/RELU; REQUANT
  *              may change bits and signedness (same word_bits and spacer).
  *   shift      REQUANT only, 0..31 (arithmetic shift for signed inputs).
@@ -195,7 +197,10 @@ SAMD_API size_t samd_conv2d_workspace_size(const samd_conv_desc *desc, samd_fmt 
  * (process-wide, all devices, takes effect at the next launch). 1 spreads
  * every layer over all SMs (lowest latency of a single layer); larger values
  * leave SMs free for independent layers launched on other streams (higher
- * throughput when several small layers run at once). Default 4.
+ * throughput when several small layers run at once). Default 4. Values above
+ * 4 also keep a convolution from letting the next kernel of its stream onto
+ * the GPU before it has ended, which pays for layers one after another on one
+ * stream and costs layers on other streams their SMs.
  * SAMD_EINVAL for values below 1 or above 1024. */
 SAMD_API samd_status samd_conv2d_set_min_tiles_per_cta(int tiles);
 
@@ -215,7 +220,9 @@ SAMD_API int samd_conv2d_operand_bits(const samd_conv_desc *desc, samd_fmt fa, s
  * touching wt, in one kernel launch. Both calls must get the same desc, fa,
  * fw and fo; fo may be {0,0,0,0} ("no packed output") in both. The
  * prepared buffer is only read by samd_conv2d_prepared, so concurrent calls
- * may share it.
+ * may share it. Its layout belongs to the build of the library that wrote it
+ * (samd_version changes with it): keep the packed weights, not the prepared
+ * ones, across builds.
  */
 SAMD_API samd_status samd_conv2d_prepare(const samd_conv_desc *desc, samd_fmt fa, samd_fmt fw, const void *wt,
                                          samd_fmt fo, void *prepared, size_t prepared_bytes, samd_stream_t stream);

@@ -245,6 +245,6 @@ const char *samd_status_str(samd_status s) {
   return "unknown samd_status";
 }
 
-const char *samd_version(void) { return "samd-gb300 0.1 (sm_103a)"; }
+const char *samd_version(void) { return "samd-gb300 0.2 (sm_103a)"; }
 
 }  // extern "C"
