@@ -217,8 +217,9 @@ struct Plan {
   int stages_a, b_resident;
   int gdepth;  // HALO: packed staging slots (items gathered gdepth - 1 ahead of the widening)
   int hbufs;   // HALO: widened halo buffers (2 or 3)
-  int e_stage; // kEpiStageBytes at off_e stage the epilogue's 3/5/6-bit packed rows
+  int e_stage; // the epilogue's 3/5/6-bit packed rows are staged, 32 words of each
   int e_flat;  // ConvArgs::e_flat
+  int e_words; // words of an epilogue warp's stage at off_e (0: none)
   int tgroup;  // weight tiles of a streamed stage (ConvArgs::tgroup)
   int pool, pool_rows, pool_nw, pool_pitch, pool_tpi;  // fused 2x2 max-pool (ConvArgs::pool)
   long long M;
@@ -538,7 +539,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   // gives up A tiles in flight, down to two, to make room), else 32 words of
   // each row at a time when a block's row holds at least 96 (5 bits) or 160
   // channels; shorter parts of rows measured faster stored directly.
-  p.e_stage = p.e_flat = 0;
+  p.e_stage = p.e_flat = p.e_words = 0;
   if ((fo.bits == 3 || fo.bits == 5 || fo.bits == 6) && fo.spacer == 0 && fo.word_bits == 32 && !pool) {
     auto fits = [&](size_t bytes) { return p.smem_bytes + round_up(bytes, 16) <= kBudget; };
     auto reserve = [&](size_t bytes) {
@@ -546,7 +547,8 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       p.smem_bytes = 1024 + p.off_bar + bar_bytes(p.stages, p.halo ? p.hbufs : p.stages_a);
     };
     const int Lo = lanes_per_word(fo);
-    const size_t flat_bytes = static_cast<size_t>(kEpiWarps) * 32 * 4 * ((d->K + Lo - 1) / Lo);
+    const int flat_words = 32 * ((d->K + Lo - 1) / Lo);
+    const size_t flat_bytes = static_cast<size_t>(kEpiWarps) * 4 * flat_words;
     if (p.nblocks == 1) {
       const Plan whole = p;
       while (!fits(flat_bytes) && !p.halo && p.stages_a > 2) {
@@ -556,6 +558,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       }
       if (fits(flat_bytes)) {
         p.e_flat = 1;
+        p.e_words = flat_words;
         reserve(flat_bytes);
       } else {
         p = whole;
@@ -563,6 +566,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
     }
     if (!p.e_flat && staged_rows(fo, p.NBc) && fits(kEpiStageBytes)) {
       p.e_stage = 1;
+      p.e_words = 32 * kEpiPitch;
       reserve(kEpiStageBytes);
     }
   }
@@ -612,6 +616,19 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   return SAMD_OK;
 }
 
+// The epilogue warps' stage for int32 rows, 32 words of each, where it fits:
+// it shares the stage of the packed rows, and what lies behind moves on.
+bool place_acc_stage(Plan &p) {
+  const int words = p.e_words > 32 * kEpiPitch ? p.e_words : 32 * kEpiPitch;
+  const size_t off_bar = round_up(p.off_e + static_cast<size_t>(kEpiWarps) * words * 4, 16);
+  const size_t smem_bytes = p.smem_bytes - p.off_bar + off_bar;
+  if (smem_bytes > kBudget) return false;
+  p.e_words = words;
+  p.off_bar = static_cast<uint32_t>(off_bar);
+  p.smem_bytes = smem_bytes;
+  return true;
+}
+
 samd_fmt none_fmt() { return samd_fmt{0, 0, 0, 0}; }
 
 // Every shared-memory region of the plan lies inside its allocation (checked
@@ -625,7 +642,8 @@ bool layout_ok(const Plan &p) {
          p.off_e <= p.off_bar && 1023 + p.off_bar + bars <= p.smem_bytes && p.op_stride % 1024 == 0 &&
          p.off_b % 1024 == 0 && p.b_bytes % 1024 == 0 && p.off_bar % 8 == 0 && 2 * p.hv * p.mma_n <= 512 &&
          (p.hv == 1 || p.hv == 2 || (p.hv == 4 && p.halo && p.fp8 && p.mma_n <= 64)) && (!p.halo || (p.gdepth >= 2 && p.gdepth <= 4 && (p.hbufs == 2 || p.hbufs == 3))) &&
-         (!p.e_stage || p.off_e + kEpiStageBytes <= p.off_bar) && !(p.e_stage && p.e_flat) && (!p.e_flat || p.nblocks == 1) &&
+         p.off_e + static_cast<size_t>(kEpiWarps) * p.e_words * 4 <= p.off_bar && (!p.e_stage || p.e_words >= 32 * kEpiPitch) &&
+         !(p.e_stage && p.e_flat) && (!p.e_flat || (p.nblocks == 1 && p.e_words > 0)) &&
          (!p.pool || (p.halo && 2 * p.Wp <= BM * p.hv && !p.e_stage && p.pool_pitch >= p.pool_nw &&
                       p.off_e + static_cast<size_t>(2 * BM) * p.pool_pitch * 4 <= p.off_bar));
 }
@@ -769,11 +787,14 @@ samd_status prepare_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa,
 }
 
 // samd_conv2d_prepared (or, with a pooled plan, its fused pool) with its plan.
-samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, const void *act, const void *prepared,
+samd_status run_planned(Plan p, const samd_conv_desc *d, samd_fmt fa, const void *act, const void *prepared,
                         size_t prepared_bytes, int32_t *acc_out, samd_fmt fo, void *packed_out, int shift,
                         cudaStream_t s, bool nchw = false, uint8_t *q8_out = nullptr) {
   if (prepared_bytes < p.ws_bytes) return SAMD_ESHAPE;
   if (p.M == 0) return SAMD_OK;
+  // int32 rows that are not whole 32-byte sectors are staged where there is room
+  const bool acc_stage =
+      acc_out && !nchw && (d->K % 8 != 0 || (reinterpret_cast<uintptr_t>(acc_out) & 31) != 0) && place_acc_stage(p);
   if (!layout_ok(p)) return SAMD_EUNSUP;
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return SAMD_ECUDA;
@@ -887,22 +908,9 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   a.fd_tpi = make_fastdiv(static_cast<uint32_t>(p.pool ? p.pool_tpi : 1));
   a.fd_pnw = make_fastdiv(static_cast<uint32_t>(p.pool ? p.pool_nw : 1));
   a.fd_wo2 = make_fastdiv(static_cast<uint32_t>(p.pool ? p.Wo / 2 : 1));
-  // The epilogue warps' stages: packed rows as planned, and int32 rows that
-  // are not whole 32-byte sectors, where the buffer fits.
-  a.e_words = p.e_flat ? 32 * static_cast<int>(words_per_row(fo, d->K)) : (p.e_stage ? 32 * kEpiPitch : 0);
-  a.acc_stage = 0;
-  size_t off_bar = p.off_bar, smem_bytes = p.smem_bytes;
-  if (acc_out && !nchw && (d->K % 8 != 0 || (reinterpret_cast<uintptr_t>(acc_out) & 31) != 0)) {
-    const int words = a.e_words > 32 * kEpiPitch ? a.e_words : 32 * kEpiPitch;
-    const size_t bar = round_up(p.off_e + static_cast<size_t>(kEpiWarps) * words * 4, 16);
-    if (p.smem_bytes - p.off_bar + bar <= kBudget) {
-      a.acc_stage = 1;
-      a.e_words = words;
-      smem_bytes = p.smem_bytes - p.off_bar + bar;
-      off_bar = bar;
-    }
-  }
-  a.off_bar = static_cast<uint32_t>(off_bar);
+  a.e_words = p.e_words;
+  a.acc_stage = acc_stage ? 1 : 0;
+  a.off_bar = p.off_bar;
   // A small layer gives each CTA at least T reference tiles of work (T from
   // samd_conv2d_set_min_tiles_per_cta; a reference tile is 128 positions of
   // a 3x3 convolution over 64 input and 64 output channels: 9 operand rows of
@@ -941,7 +949,7 @@ samd_status run_planned(const Plan &p, const samd_conv_desc *d, samd_fmt fa, con
   const int wi = fa.word_bits == 64 ? 1 : 0;
   if (p.fp8 && fa.bits > 5) return SAMD_EUNSUP;  // not reached: e4m3 only for |a| <= 16
   const LaunchFn fn = p.fp8 ? kF8[wi][fa.bits - 1] : kF16[wi][fa.bits - 1];
-  const cudaError_t e = fn(fa.is_signed != 0, tmap, a, p.halo != 0, grid, smem_bytes, s);
+  const cudaError_t e = fn(fa.is_signed != 0, tmap, a, p.halo != 0, grid, p.smem_bytes, s);
   return e == cudaSuccess ? SAMD_OK : SAMD_ECUDA;
 }
 
