@@ -215,7 +215,6 @@ struct Plan {
   int nseg, seg_rows, seg_used, row_step;  // halo geometry (see ConvArgs)
   long long grid_m;                        // 128-position tiles along the output
   int stages_a, b_resident;
-  int gdepth;  // HALO: packed staging slots (items gathered gdepth - 1 ahead of the widening)
   int hbufs;   // HALO: widened halo buffers (2 or 3)
   int e_stage; // the epilogue's 3/5/6-bit packed rows are staged, 32 words of each
   int e_flat;  // ConvArgs::e_flat
@@ -241,7 +240,6 @@ size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // 16: 35.1 -> 22.4 us.
 constexpr double kMaxHaloWaste = 1.35;
 constexpr size_t kBudget = 224 * 1024;  // shared memory: below the 227 KB opt-in limit minus static shared memory
-constexpr int kHaloGatherDepth = 2;  // packed staging slots of the halo producers (2..4)
 // minimum 128-pixel tiles per CTA of a launch (samd_conv2d_set_min_tiles_per_cta)
 constexpr int kDefaultMinTiles = 4;
 std::atomic<int> g_min_tiles_per_cta{kDefaultMinTiles};
@@ -339,7 +337,6 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
   p.g_row = grow;
   p.b_bytes = static_cast<uint32_t>(p.mma_n) * p.row_bytes;  // a multiple of 1024
   const size_t bst = p.b_bytes;
-  const size_t e_bytes = 0;  // the epilogue packs in registers
   // mbarriers: full_b and empty_b per weight stage, opfull and opempty per
   // operand stage, two accumulator pairs, the drain barrier and two
   // epilogue group barriers; then the TMEM address word
@@ -350,7 +347,7 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
     p.off_b = static_cast<uint32_t>(op_bytes);
     p.off_g = static_cast<uint32_t>(op_bytes + p.stages * p.tgroup * bst);
     p.off_e = static_cast<uint32_t>(round_up(p.off_g + g_bytes, 16));
-    p.off_bar = static_cast<uint32_t>(round_up(p.off_e + e_bytes, 16));
+    p.off_bar = p.off_e;  // the epilogue packs in registers; stages for it are put in later
     p.smem_bytes = 1024 + p.off_bar + bar_bytes(p.stages, op_stages);  // + alignment slack of the base
   };
   p.taps = d->R * d->S;
@@ -382,7 +379,6 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
     const int bmt = BM * hv;
     p.hv = hv;
     p.halo = 0;
-    p.gdepth = 2;
     p.hbufs = 2;
     p.b_resident = 0;
     p.stages_a = 0;
@@ -416,11 +412,6 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       const size_t stage_g = round_up(static_cast<size_t>(halo_rows) * srow, 16);
       const int ntiles_b = p.nck * p.taps;
       if (halo_rows > kMaxHaloRows || waste > (two_sided ? 1.16 : kMaxHaloWaste)) return false;
-      // The packed staging ring: with depth D the gathers run D - 1 items
-      // ahead of the widening. Depth 2 is used: per-role timelines show the
-      // halo producers finishing a tile's operands microseconds before its
-      // MMAs start, and the sweep step measured 6% slower at depth 4 (the
-      // kernel takes depths up to 4).
       // Widened halo buffers: the producers widen item k into buffer
       // k mod hbufs once the MMAs of item k - hbufs are done. fp16 layers
       // take three when their weights stay resident as well. (A 6-bit sweep
@@ -430,22 +421,17 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       // half as large and cheaper to widen, showed no gain.)
       size_t fixed = 0;
       bool res = false;
-      int depth = kHaloGatherDepth, hbufs = 2;
-      auto fits = [&](int nb, int dp, bool want_res) {
-        fixed = nb * halo_bytes + dp * stage_g + e_bytes + 1024;
+      int hbufs = 2;
+      auto fits = [&](int nb, bool want_res) {
+        fixed = nb * halo_bytes + kHaloGatherSlots * stage_g + 1024;
         if (fixed + 2 * bst + bar_bytes(2, nb) > kBudget) return false;
         res = p.nblocks == 1 && fixed + ntiles_b * bst + bar_bytes(ntiles_b, nb) <= kBudget;
         return !(want_res && !res);
       };
-      bool ok3 = !p.fp8 && fits(3, depth, true);
-      if (ok3) {
+      if (!p.fp8 && fits(3, true))
         hbufs = 3;
-      } else {
-        for (; depth >= 2; --depth)
-          if (fits(2, depth, need_resident)) break;
-        if (depth < 2) return false;
-      }
-      p.gdepth = depth;
+      else if (!fits(2, need_resident))
+        return false;
       p.hbufs = hbufs;
       p.halo = 1;
       p.nchunks = ntiles_b;
@@ -470,13 +456,13 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
       }
       p.op_stride = static_cast<uint32_t>(halo_bytes);
       p.g_stride = static_cast<uint32_t>(stage_g);
-      finish(hbufs * halo_bytes, depth * stage_g, hbufs);
+      finish(hbufs * halo_bytes, kHaloGatherSlots * stage_g, hbufs);
       return true;
     }
     const size_t tile_bytes = static_cast<size_t>(bmt) * p.row_bytes;
     const size_t group_slots = static_cast<size_t>(kGatherDepth) * BM * grow;  // one producer group's ring
     for (int sta = 4; sta >= 2; --sta) {
-      const size_t fixed = sta * tile_bytes + 2 * group_slots + e_bytes + 1024;
+      const size_t fixed = sta * tile_bytes + 2 * group_slots + 1024;
       if (fixed + 2 * bst + bar_bytes(2, sta) > kBudget) continue;
       const bool res = p.nblocks == 1 && fixed + p.nchunks * bst + bar_bytes(p.nchunks, sta) <= kBudget;
       if (need_resident && !res) continue;
@@ -589,21 +575,14 @@ samd_status make_plan(const samd_conv_desc *d, samd_fmt fa, samd_fmt fw, samd_fm
     p.pool_nw = (p.NBc + 32 / fo.bits - 1) / (32 / fo.bits);
     p.pool_pitch = pool_pitch(p.NBc, fo);
     const size_t pool_bytes = static_cast<size_t>(2 * BM) * p.pool_pitch * 4;
-    // the buffer goes after the packed staging ring, made shallower if need
-    // be (the ring's depth does not change the weight layout)
-    int depth = p.gdepth;
-    size_t off_e = 0;
-    for (; depth >= 2; --depth) {
-      off_e = round_up(p.off_g + static_cast<size_t>(depth) * p.g_stride, 16);
-      if (1024 + round_up(off_e + pool_bytes, 16) + bar_bytes(p.stages, p.hbufs) <= kBudget) break;
-    }
-    if (depth < 2) {
+    // the buffer goes after the packed staging slots
+    const size_t off_e = round_up(p.off_g + kHaloGatherSlots * static_cast<size_t>(p.g_stride), 16);
+    if (1024 + round_up(off_e + pool_bytes, 16) + bar_bytes(p.stages, p.hbufs) > kBudget) {
       // a smaller halo may have made room for more weights and left too
       // little for the pool buffer: the placement that was found above fits
       return two_sided ? SAMD_EUNSUP : make_plan(d, fa, fw, fo, p, true, true);
     }
     p.pool = 1;
-    p.gdepth = depth;
     p.grid_m = static_cast<long long>(d->N) * p.pool_tpi;
     p.off_e = static_cast<uint32_t>(off_e);
     p.off_bar = static_cast<uint32_t>(round_up(off_e + pool_bytes, 16));
@@ -638,10 +617,10 @@ bool layout_ok(const Plan &p) {
   const size_t op_bytes = NO * p.op_stride;
   const size_t bars = (2 * static_cast<size_t>(p.stages) + 2 * NO + 7) * 8 + 4;
   return p.stages >= 1 && NO >= 2 && op_bytes <= p.off_b &&
-         p.off_b + static_cast<size_t>(p.stages) * p.tgroup * p.b_bytes <= p.off_g && p.tgroup >= 1 && (p.tgroup == 1 || (p.halo && p.taps % p.tgroup == 0 && !p.b_resident)) && p.off_g + static_cast<size_t>(p.halo ? p.gdepth : 2) * p.g_stride <= p.off_e &&
+         p.off_b + static_cast<size_t>(p.stages) * p.tgroup * p.b_bytes <= p.off_g && p.tgroup >= 1 && (p.tgroup == 1 || (p.halo && p.taps % p.tgroup == 0 && !p.b_resident)) && p.off_g + static_cast<size_t>(p.halo ? kHaloGatherSlots : 2) * p.g_stride <= p.off_e &&
          p.off_e <= p.off_bar && 1023 + p.off_bar + bars <= p.smem_bytes && p.op_stride % 1024 == 0 &&
          p.off_b % 1024 == 0 && p.b_bytes % 1024 == 0 && p.off_bar % 8 == 0 && 2 * p.hv * p.mma_n <= 512 &&
-         (p.hv == 1 || p.hv == 2 || (p.hv == 4 && p.halo && p.fp8 && p.mma_n <= 64)) && (!p.halo || (p.gdepth >= 2 && p.gdepth <= 4 && (p.hbufs == 2 || p.hbufs == 3))) &&
+         (p.hv == 1 || p.hv == 2 || (p.hv == 4 && p.halo && p.fp8 && p.mma_n <= 64)) && (!p.halo || p.hbufs == 2 || p.hbufs == 3) &&
          p.off_e + static_cast<size_t>(kEpiWarps) * p.e_words * 4 <= p.off_bar && (!p.e_stage || p.e_words >= 32 * kEpiPitch) &&
          !(p.e_stage && p.e_flat) && (!p.e_flat || (p.nblocks == 1 && p.e_words > 0)) &&
          (!p.pool || (p.halo && 2 * p.Wp <= BM * p.hv && !p.e_stage && p.pool_pitch >= p.pool_nw &&
@@ -895,7 +874,6 @@ samd_status run_planned(Plan p, const samd_conv_desc *d, samd_fmt fa, const void
   a.b_bytes = p.b_bytes;
   a.off_g = p.off_g;
   a.g_stride = p.g_stride;
-  a.gdepth = p.gdepth;
   a.hbufs = p.hbufs;
   a.off_e = p.off_e;
   a.e_stage = p.e_stage;

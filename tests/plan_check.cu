@@ -26,7 +26,7 @@ using namespace samd;
 // Operand stages, weight stages, packed staging, epilogue stage, barriers, one
 // after the other; sizes are counted again here, not taken from layout_ok.
 bool regions_ok(const conv::Plan &p, const samd_conv_desc &d, samd_fmt fo) {
-  const size_t no = p.halo ? p.hbufs : p.stages_a, ng = p.halo ? p.gdepth : 2;
+  const size_t no = p.halo ? p.hbufs : p.stages_a, ng = 2;
   const size_t weights = static_cast<size_t>(p.stages) * p.tgroup * p.mma_n * p.row_bytes;
   size_t epi = 0;
   if (p.e_flat) epi = 8 * 32 * 4 * static_cast<size_t>(words_per_row(fo, d.K));  // 32 whole rows a warp
@@ -51,7 +51,7 @@ bool regions_ok(const conv::Plan &p, const samd_conv_desc &d, samd_fmt fo) {
 
 int main() {
   long long flat = 0, rows = 0, accs = 0, pools = 0;
-  long long n = 0, bad = 0, halo = 0, seg = 0, fp8 = 0, res = 0, unsup = 0, hv2 = 0, win = 0, deep = 0, estg = 0, hv4 = 0;
+  long long n = 0, bad = 0, halo = 0, seg = 0, fp8 = 0, res = 0, unsup = 0, hv2 = 0, win = 0, estg = 0, hv4 = 0;
   const int Cs[] = {1, 3, 16, 24, 64, 96, 128, 256, 512, 1024};
   const int Ks[] = {1, 16, 40, 64, 96, 128, 256, 300, 512, 1024};
   const int HWs[] = {1, 2, 7, 14, 28, 56, 224};
@@ -87,9 +87,7 @@ int main() {
                           const int srow = (p.WC * wb / 8 + 15) / 16 * 16;
                           ok = ok && maxrow < p.nseg * p.seg_rows &&
                                p.nseg * p.seg_rows * static_cast<long long>(p.row_bytes) <= p.op_stride &&
-                               p.gdepth >= 2 && p.gdepth <= 4 &&
                                static_cast<long long>(p.nseg) * p.seg_rows * srow <= p.g_stride;
-                          if (p.gdepth == conv::kHaloGatherDepth) ++deep;
                         } else {
                           // gather staging: a producer group's ring of kGatherDepth x 128 rows
                           const int chunk_bytes = p.WC * wb / 8;
@@ -130,8 +128,8 @@ int main() {
                       }
                     }
   printf("plans %lld, bad %lld, unsupported %lld, halo %lld (segmented %lld), e4m3 %lld, resident %lld, "
-         "two-half %lld, four-part %lld, window gather %lld, staging at the chosen depth %lld, staged epilogue %lld, "
+         "two-half %lld, four-part %lld, window gather %lld, staged epilogue %lld, "
          "flat epilogue %lld, filter-row stages %lld, int32 stage %lld, pooled %lld\n",
-         n, bad, unsup, halo, seg, fp8, res, hv2, hv4, win, deep, estg, flat, rows, accs, pools);
+         n, bad, unsup, halo, seg, fp8, res, hv2, hv4, win, estg, flat, rows, accs, pools);
   return bad != 0;
 }
