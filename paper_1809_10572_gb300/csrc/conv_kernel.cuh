@@ -1063,11 +1063,11 @@ __device__ __forceinline__ void epilogue_row(const ConvArgs &args, const EpiRow 
 }
 
 // A role's wait on one of the kernel's barriers. A role whose wait gives up
-// (false) stops: the loader and the epilogue at once, the MMA warp and the
-// producers at the end of a tile or a few items, filling and releasing every
-// stage in step until there (with undefined values). The others' waits then
-// give up in turn, within one poll of the failure's being recorded, and the
-// kernel ends with what was in flight drained.
+// (false) stops: the loader at once, the others at the end of their tile or a
+// few items, filling and releasing every stage in step until there (with
+// undefined values). The others' waits then give up in turn, within one poll
+// of the failure's being recorded, and the kernel ends with what was in flight
+// drained.
 __device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, int *status, uint64_t limit_ns = kWaitLimitNs) {
   return ptx::mbar_wait(bar, parity, status, static_cast<int>(SAMD_ETIMEOUT), limit_ns);
 }
@@ -1775,8 +1775,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
     }
     for (uint32_t tile = first_tile + (HV >= 2 ? 0 : set) * tile_step; !pooled && tile < total_tiles;) {
       const int acc_i = HV >= 2 ? static_cast<int>(i & 1) : set;  // accumulator of this tile
+      bool ok = true;
       if (!warm) {
-        if (!warp_wait(accfull(acc_i), (i >> 1) & 1u, status)) break;
+        ok = warp_wait(accfull(acc_i), (i >> 1) & 1u, status);
         ptx::tc_fence_after();
       }
       const uint32_t nbu = fdiv(tile, args.fd_gm);
@@ -1812,6 +1813,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(accempty(acc_i));
+      if (!ok) break;
       tile += kTileStep * tile_step;
       i += kTileStep;
     }
