@@ -272,9 +272,10 @@ SAMD_API samd_status samd_conv2d_noalloc(const samd_conv_desc *desc, samd_fmt fa
  * else SAMD_EUNSUP and nothing is launched): NHWC, stride 1, Ho and Wo even,
  * 2 * (W + 2 * pad) <= 256 (a tile of 256 positions holds whole pairs of
  * padded image rows), fo of 1, 2, 4 or 8 bits in 32-bit words without
- * spacers, and a layer the kernel runs as halo tiles of two halves with
- * room for the tile's packed rows in shared memory. pooled_out: 16-byte
- * aligned, caller-owned.
+ * spacers, and a layer the kernel runs as halo tiles with room for the tile's
+ * packed rows in shared memory. Whether this or the two calls is the faster
+ * depends on the layer (the packed rows take room from its weights): time
+ * both. pooled_out: 16-byte aligned, caller-owned.
  */
 SAMD_API samd_status samd_conv2d_prepared_pool2x2(const samd_conv_desc *desc, samd_fmt fa, const void *act,
                                                   samd_fmt fw, const void *prepared, size_t prepared_bytes,

@@ -234,10 +234,15 @@ long long max_abs(samd_fmt f) { return f.is_signed ? (1LL << (f.bits - 1)) : ((1
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // A halo layer computes the whole virtual grid; a gather layer gathers and
-// widens every operand row once per tap instead. At 7x7 (1.31 grid positions
-// per output) the halo form is still the faster one: 3x3, 512 channels, u6 x
-// s2, batch 64: 58.8 -> 32.9 us; 14x14 (1.15), 512 channels, u4 x s4, batch
-// 16: 35.1 -> 22.4 us.
+// widens every operand row once per tap instead. The line admits 7x7 images
+// (1.31 grid positions per output; 3x3, 512 channels, u6 x s2, batch 64, back
+// to back: 58.8 us by gather, 32.9 by halo) and 14x14 ones (1.15; 512
+// channels, u4 x s4, batch 16: 35.1 and 22.4). It is not where the forms break
+// even, which lies higher: 5x5 images (1.44) of 512 channels, batch 64, take
+// 27.7 us by gather and 15.0 by halo (u4 x s4), 50.4 and 29.7 (u6 x s2), 4x4
+// ones (1.56) 27.5 and 15.0, 49.7 and 29.4, and 7x7 ones with 5x5 filters
+// (1.65) 70.9 and 59.8, 155.8 and 70.3; at 64 channels, batch 256, u4 x s4,
+// gather is ahead by a little at 5x5 and 4x4 (12.8 and 13.7, 12.7 and 13.2).
 constexpr double kMaxHaloWaste = 1.35;
 constexpr size_t kBudget = 224 * 1024;  // shared memory: below the 227 KB opt-in limit minus static shared memory
 // minimum 128-pixel tiles per CTA of a launch (samd_conv2d_set_min_tiles_per_cta)
@@ -909,7 +914,8 @@ samd_status run_planned(Plan p, const samd_conv_desc *d, samd_fmt fa, const void
   if (ctas > sm_count()) ctas = sm_count();
   dim3 grid(static_cast<unsigned>(ctas));
   // The next kernel of the stream may hold SMs while it waits for this one
-  // to drain (one layer after another: ResNet-50 7x7 block 98.3 -> 92.4 us),
+  // to drain (one layer after another: ResNet-50 7x7 block 98.3 -> 92.4 us; a
+  // launch with nothing before it gains nothing),
   // unless more work per SM than the default was asked for, which leaves SMs
   // to layers on other streams (the 32-layer sweep step on eight streams: 124
   // us without, 127 with).

@@ -928,7 +928,9 @@ __device__ __forceinline__ void exact_16(const ConvArgs &args, uint32_t taddr, i
 // int32 outputs: whole sectors of a thread's own row where rows are whole
 // sectors; otherwise 32 columns of the warp's rows are staged (acc_stage) and
 // written row by row, 32 consecutive words a store, or, without room for
-// that, one word at a time. 29 x 51 x 140 positions of 262 channels (217 MB),
+// that, one word at a time. (So do the later channel blocks of whole-sector
+// rows beside 3- and 6-bit packed ones: their first channel is a multiple of
+// 10 or 5, and the stage is planned by K alone.) 29 x 51 x 140 positions of 262 channels (217 MB),
 // with 3-bit packed rows: 451 us one word at a time, 242 this way.
 __device__ __forceinline__ void epilogue_row_acc(const ConvArgs &args, const EpiRow &e, uint32_t *stg) {
   const bool vec_ok = args.K % 4 == 0 && e.ch0 % 4 == 0;
@@ -1445,9 +1447,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const __grid_constant
               }
             };
             // MMAs of up to 64 columns (48 cycles) are the one case where the
-            // predicate costs more than the branch: VGG-16 conv2 39.1 us with
-            // the predicate, 35.0 with the branch; conv4 (128 columns) 27.6
-            // and 30.7
+            // predicate costs more than the branch: VGG-16 conv2, back to
+            // back, 39.1 us with the predicate, 35.0 with the branch; conv4
+            // (128 columns) 27.6 and 30.7
             if (args.mma_n <= 64) {
               if (leader) all_taps(1u);
               __syncwarp();

@@ -69,7 +69,8 @@ int resident_grid(int64_t work_items, int threads, size_t smem = 0) {
 
 // ---- device-side lane helpers ----------------------------------------------
 
-// n / d for 0 <= n < 2^31 by one multiply-high, an add and a shift:
+// n / d for 0 <= n < 2^31 by one multiply-high, an add and a shift (Granlund
+// and Montgomery, "Division by Invariant Integers using Multiplication", 1994):
 // l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1, q = (umulhi(m, n) + n) >> l.
 struct FastDiv {
   uint32_t m;
