@@ -241,10 +241,12 @@ __device__ __forceinline__ void st_global_cs_v8(void *p, const uint32_t *c) {
                : "memory");
 }
 
-// Lanes of 1, 2 and 4 bits: a quad of words fills whole 32-byte sectors of the
+// Lanes of 2 and 4 bits: a quad of words fills whole 32-byte sectors of the
 // output, so a thread stores its 4L bytes itself, 32 at a time; two quads a
 // step, so that two loads are in flight. 51 M signed 4-bit lanes (77 MB
-// moved): 16.4 us through shared memory, 16.1 this way.
+// moved): 16.4 us through shared memory, 16.1 this way; 2^28 2-bit lanes 59.6
+// and 57.1. (1-bit lanes, 128 bytes a thread, 51.3 and 55.3: they stay with
+// unpack32_vec_kernel.)
 template <int BITS, bool SIGNED>
 __global__ void __launch_bounds__(kThreads) unpack32_direct_kernel(const uint32_t *__restrict__ src,
                                                                    int8_t *__restrict__ dst, int64_t nquads) {
@@ -289,9 +291,9 @@ __global__ void __launch_bounds__(kThreads) unpack32_vec_kernel(const uint32_t *
     const uint4 v = __ldcs(reinterpret_cast<const uint4 *>(src) + q);
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     uint32_t c[NC];
-    if constexpr (BITS == 8) {
+    if constexpr (BITS == 1 || BITS == 2 || BITS == 4 || BITS == 8) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k) c[k] = w[k];
+      for (int k = 0; k < 4; ++k) unpack_word32<BITS, SIGNED>(w[k], c + k * (L / 4));
     } else {
 #pragma unroll
       for (int i = 0; i < NC; ++i) c[i] = 0;
@@ -502,7 +504,7 @@ cudaError_t launch_pack32_vec(const int8_t *src, uint32_t *dst, int64_t ntiles, 
 
 template <int BITS, bool SIGNED>
 cudaError_t launch_unpack32_vec(const uint32_t *src, int8_t *dst, int64_t ntiles, cudaStream_t s) {
-  if constexpr (BITS == 1 || BITS == 2 || BITS == 4) {
+  if constexpr (BITS == 2 || BITS == 4) {
     if ((reinterpret_cast<uintptr_t>(dst) & 31) == 0) {  // 32-byte stores (callers align to 16)
       const int grid = resident_grid<unpack32_direct_kernel<BITS, SIGNED>>(ntiles * 32, kThreads);
       unpack32_direct_kernel<BITS, SIGNED><<<grid, kThreads, 0, s>>>(src, dst, ntiles * 32);
