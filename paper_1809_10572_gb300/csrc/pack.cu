@@ -2,10 +2,12 @@
 // b-bit lanes laid side by side in a scalar word; section 7: unpacking to
 // the native 8-bit type).
 //
-// Three layouts:
+// Layouts:
 //   - one row, or rows of whole words, of spacer-free 32-bit words: a thread
 //     moves four words with the widest aligned vectors (pack32_*, unpack32_*);
 //     64-bit words whose lane width divides 32 are pairs of such words;
+//   - spacer formats of 16 and more lanes a word are packed by a thread a word
+//     (pack_generic_kernel);
 //   - anything else (rows that end inside a word, 64-bit words of 3, 5, 6 or
 //     7 bits, spacer bits, and the few words the vector kernels leave): the
 //     bytes of a tile of consecutive words are one contiguous run, staged in
@@ -192,6 +194,28 @@ __global__ void __launch_bounds__(kThreads) pack32_vec_kernel(const int8_t *__re
   }
 }
 
+// Spacer formats of 16 and more lanes a word: a thread packs a word from its
+// bytes one at a time (pack_rows_kernel reads them from shared memory, 16 and
+// more bytes from one thread to the next: 2^26 signed lanes with one spacer
+// bit, 1 bit in 32-bit words 34.8 us and 38.9, in 64-bit words 59.7 and 65.6,
+// 3 bits 36.9 and 41.0; with fewer lanes a word that one is 1.1 to 1.7 times
+// as fast).
+template <typename W>
+__global__ void __launch_bounds__(kThreads) pack_generic_kernel(const int8_t *__restrict__ src, W *__restrict__ dst,
+                                                                int64_t total_words, int64_t inner, int64_t wpr,
+                                                                int bits, int lane_w, int L) {
+  const W mask = (W(1) << bits) - 1;
+  for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < total_words;
+       w += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = w / wpr, wi = w - row * wpr;
+    const int64_t e0 = row * inner + wi * L;
+    const int64_t count = inner - wi * L < L ? inner - wi * L : L;
+    W word = 0;
+    for (int i = 0; i < count; ++i) word |= (W(static_cast<uint8_t>(src[e0 + i])) & mask) << (i * lane_w);
+    dst[w] = word;
+  }
+}
+
 // Unpack of 4 words per thread into 4L bytes, written with the widest aligned
 // vector. b = 8: the word is its bytes. b = 4: the low and high nibbles of
 // each byte are masked apart and interleaved by byte permutes; signed nibbles
@@ -348,6 +372,9 @@ __device__ __forceinline__ uint8_t lane_byte(W word, int i) {
 
 // T words of L lanes: at most 16 KB of bytes, a few words per thread.
 constexpr int tile_words(int L) { return L <= 12 ? 1024 : (L <= 24 ? 512 : 256); }
+// The same for the forms of any format, whose L (at most 32) is known at run
+// time.
+__host__ __device__ constexpr int any_tile_words(int L) { return L <= 16 ? 1024 : 512; }
 
 struct RowsArgs {
   int64_t inner;
@@ -395,12 +422,12 @@ template <typename W, int BITS>
 __global__ void __launch_bounds__(kThreads) pack_rows_kernel(const int8_t *src, W *__restrict__ dst,
                                                              const RowsArgs a) {
   constexpr int kL = BITS ? WordTraits<W>::kBits / (BITS ? BITS : 1) : 0;
-  constexpr int kTile = BITS ? tile_words(kL) : 256;
-  constexpr int kBytes = kTile * (BITS ? kL : 64);
+  constexpr int kBytes = BITS ? tile_words(kL) * kL : 16 * 1024;
   __shared__ __align__(16) uint8_t stage[kBytes + 48];  // 15 bytes before the run, reads up to 8 bytes past it
   const int L = BITS ? kL : a.L;
-  for (uint32_t first = blockIdx.x * kTile; first < a.total_words; first += gridDim.x * kTile) {
-    const RowsTile t(a, first, kTile, L, src);
+  const uint32_t tile = BITS ? tile_words(kL) : any_tile_words(L);
+  for (uint32_t first = blockIdx.x * tile; first < a.total_words; first += gridDim.x * tile) {
+    const RowsTile t(a, first, tile, L, src);
     const int8_t *const p = src + t.b0 - t.lead;
     const int nvec = (t.lead + t.bytes + 15) >> 4;
     for (int v = threadIdx.x; v < nvec; v += kThreads) {
@@ -443,12 +470,12 @@ template <typename W, int BITS, bool SIGNED>
 __global__ void __launch_bounds__(kThreads) unpack_rows_kernel(const W *__restrict__ src, int8_t *dst,
                                                                const RowsArgs a) {
   constexpr int kL = BITS ? WordTraits<W>::kBits / (BITS ? BITS : 1) : 0;
-  constexpr int kTile = BITS ? tile_words(kL) : 256;
-  constexpr int kBytes = kTile * (BITS ? kL : 64);
+  constexpr int kBytes = BITS ? tile_words(kL) * kL : 16 * 1024;
   __shared__ __align__(16) uint8_t stage[kBytes + 32];
   const int L = BITS ? kL : a.L;
-  for (uint32_t first = blockIdx.x * kTile; first < a.total_words; first += gridDim.x * kTile) {
-    const RowsTile t(a, first, kTile, L, dst);
+  const uint32_t tile = BITS ? tile_words(kL) : any_tile_words(L);
+  for (uint32_t first = blockIdx.x * tile; first < a.total_words; first += gridDim.x * tile) {
+    const RowsTile t(a, first, tile, L, dst);
     for (uint32_t w = t.w0 + threadIdx.x; w < t.w1; w += kThreads) {
       int count;
       const int off = t.offset(a, w, L, &count);
@@ -545,7 +572,7 @@ cudaError_t launch_rows(const S *src, D *dst, const RowsArgs &a, int tile, cudaS
 template <typename W>
 cudaError_t pack_rows(samd_fmt f, const int8_t *src, W *dst, int64_t rows, int64_t inner, cudaStream_t s) {
   const RowsArgs a = rows_args(f, rows, inner);
-  if (f.spacer != 0) return launch_rows<pack_rows_kernel<W, 0>>(src, dst, a, 256, s);
+  if (f.spacer != 0) return launch_rows<pack_rows_kernel<W, 0>>(src, dst, a, any_tile_words(a.L), s);
   switch (f.bits) {
 #define SAMD_PACK_CASE(B) \
   case B: return launch_rows<pack_rows_kernel<W, B>>(src, dst, a, tile_words(WordTraits<W>::kBits / B), s);
@@ -559,7 +586,7 @@ cudaError_t pack_rows(samd_fmt f, const int8_t *src, W *dst, int64_t rows, int64
 template <typename W>
 cudaError_t unpack_rows(samd_fmt f, const W *src, int8_t *dst, int64_t rows, int64_t inner, cudaStream_t s) {
   const RowsArgs a = rows_args(f, rows, inner);
-  if (f.spacer != 0) return launch_rows<unpack_rows_kernel<W, 0, false>>(src, dst, a, 256, s);
+  if (f.spacer != 0) return launch_rows<unpack_rows_kernel<W, 0, false>>(src, dst, a, any_tile_words(a.L), s);
   switch (f.bits * 2 + (f.is_signed ? 1 : 0)) {
 #define SAMD_UNPACK_CASE(B)                                                                                           \
   case 2 * B:                                                                                                         \
@@ -607,6 +634,12 @@ int64_t vec_tiles(samd_fmt f, int64_t rows, int64_t inner) {
 
 template <typename W>
 cudaError_t pack_dispatch(samd_fmt f, const int8_t *src, W *dst, int64_t rows, int64_t inner, cudaStream_t s) {
+  if (f.spacer != 0 && lanes_per_word(f) >= 16) {
+    const int64_t wpr = words_per_row(f, inner), total = rows * wpr;
+    pack_generic_kernel<W><<<grid_for(total, kThreads, sm_count() * 16), kThreads, 0, s>>>(
+        src, dst, total, inner, wpr, f.bits, f.bits + f.spacer, lanes_per_word(f));
+    return cudaGetLastError();
+  }
   const int64_t ntiles = vec_tiles(f, rows, inner);
   if (ntiles > 0) {
     cudaError_t e;

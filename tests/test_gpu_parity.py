@@ -449,12 +449,13 @@ def test_requant_format_change_periods(samd_lib, bits, bits_o, word_bits):
 # byte runs of 256, 512 or 1024 words: sizes at the edges of those runs, runs
 # that start at every byte offset, rows shorter than a word, guard bytes.
 @pytest.mark.parametrize("bits,spacer,word_bits", [(1, 0, 32), (3, 0, 32), (6, 0, 32), (7, 0, 32), (8, 0, 32), (1, 0, 64),
-                                                   (3, 0, 64), (5, 0, 64), (7, 0, 64), (2, 1, 32), (4, 2, 64)])
+                                                   (3, 0, 64), (5, 0, 64), (7, 0, 64), (2, 1, 32), (4, 2, 64),
+                                                   (1, 1, 64), (1, 1, 32), (8, 1, 32), (2, 0, 64), (6, 0, 64)])
 def test_pack_unpack_row_runs(samd_lib, bits, spacer, word_bits):
     f = samd.fmt(bits, True, spacer, word_bits)
     L = samd.samd_lanes_per_word(f)
     for rows, inner in [(1023, L + 1), (1025, 1), (513, 3 * L - 1), (257, L + 3), (129, 2 * L + 1), (1, 1024 * L + 1),
-                        (3, 1024 * L - 1), (2049, 3)]:
+                        (3, 1024 * L - 1), (2049, 3), (1, 512 * L + 1), (3, 512 * L - 1), (77, 5 * L), (1, L - 1)]:
         v, b = values_and_bytes(synth.seed_for("run", bits, spacer, word_bits, rows, inner), (rows, inner), bits, True)
         want = oracle.pack(v, bits, True, spacer, word_bits)
         words = torch.full((want.size + 4,), 0x5A5A5A5A, dtype=samd.word_dtype(f), device="cuda")
