@@ -5,7 +5,8 @@
 // Layouts:
 //   - one row, or rows of whole words, of spacer-free 32-bit words: a thread
 //     moves four words with the widest aligned vectors (pack32_*, unpack32_*);
-//     64-bit words whose lane width divides 32 are pairs of such words;
+//     64-bit words whose lane width divides 32 are pairs of such words, except
+//     where a thread packs a 64-bit word faster (pack64_word_kernel);
 //   - spacer formats of 16 and more lanes a word are packed by a thread a word
 //     (pack_generic_kernel);
 //   - anything else (rows that end inside a word, 64-bit words of 3, 5, 6 or
@@ -192,6 +193,53 @@ __global__ void __launch_bounds__(kThreads) pack32_vec_kernel(const int8_t *__re
     }
     __stcs(reinterpret_cast<uint4 *>(dst) + q, make_uint4(w[0], w[1], w[2], w[3]));
   }
+}
+
+// One row, or rows of whole words, of 64-bit words of 1, 2, 5 and 6 bits: a
+// thread packs one word from its L bytes, read with the widest aligned
+// vectors. 2^28 lanes, against pairs of 32-bit words (1 and 2 bits) and
+// pack_rows_kernel (5 and 6): 49.6 us and 51.2, 51.6 and 55.8, 80.2 and 95.2,
+// 97.0 and 110. (At 3 and 7 bits, whose L is odd, that one is the faster: 119
+// and 87, 136 and 115.)
+template <int VB> struct Vec;
+template <> struct Vec<16> { using T = uint4; };
+template <> struct Vec<4> { using T = uint32_t; };
+template <> struct Vec<2> { using T = uint16_t; };
+
+template <int BITS>
+__global__ void __launch_bounds__(kThreads) pack64_word_kernel(const int8_t *__restrict__ src,
+                                                               uint64_t *__restrict__ dst, int64_t nwords, int64_t n) {
+  constexpr int L = 64 / BITS, VB = vec_bytes(L);
+  constexpr uint64_t mask = (1u << BITS) - 1;
+  using T = typename Vec<VB>::T;
+  for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nwords; w += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t e0 = w * L;
+    uint64_t word = 0;
+    if (n - e0 >= L) {
+      const T *const p = reinterpret_cast<const T *>(src + e0);
+      uint8_t buf[L];
+#pragma unroll
+      for (int v = 0; v < L / VB; ++v) {
+        const T t = __ldg(p + v);
+        const uint8_t *const b = reinterpret_cast<const uint8_t *>(&t);
+#pragma unroll
+        for (int j = 0; j < VB; ++j) buf[v * VB + j] = b[j];
+      }
+#pragma unroll
+      for (int i = 0; i < L; ++i) word |= (buf[i] & mask) << (i * BITS);
+    } else {
+      for (int i = 0; i < static_cast<int>(n - e0); ++i) word |= (static_cast<uint8_t>(src[e0 + i]) & mask) << (i * BITS);
+    }
+    dst[w] = word;
+  }
+}
+
+template <int BITS>
+cudaError_t launch_pack64_words(const int8_t *src, uint64_t *dst, int64_t n, cudaStream_t s) {
+  constexpr int L = 64 / BITS;
+  const int64_t nwords = (n + L - 1) / L;
+  pack64_word_kernel<BITS><<<grid_for(nwords, kThreads, sm_count() * 16), kThreads, 0, s>>>(src, dst, nwords, n);
+  return cudaGetLastError();
 }
 
 // Spacer formats of 16 and more lanes a word: a thread packs a word from its
@@ -632,8 +680,24 @@ int64_t vec_tiles(samd_fmt f, int64_t rows, int64_t inner) {
   return rows * inner / (32 / f.bits) / 128;  // warp tiles of 32 quads of words
 }
 
+// Whether 64-bit words go by pack64_word_kernel.
+bool word64_form(samd_fmt f, int64_t rows, int64_t inner) {
+  return f.word_bits == 64 && f.spacer == 0 && (f.bits == 1 || f.bits == 2 || f.bits == 5 || f.bits == 6) &&
+         (rows == 1 || inner % lanes_per_word(f) == 0);
+}
+
 template <typename W>
 cudaError_t pack_dispatch(samd_fmt f, const int8_t *src, W *dst, int64_t rows, int64_t inner, cudaStream_t s) {
+  if constexpr (sizeof(W) == 8)
+    if (word64_form(f, rows, inner)) {
+      const int64_t n = rows * inner;
+      switch (f.bits) {
+        case 1: return launch_pack64_words<1>(src, dst, n, s);
+        case 2: return launch_pack64_words<2>(src, dst, n, s);
+        case 5: return launch_pack64_words<5>(src, dst, n, s);
+        default: return launch_pack64_words<6>(src, dst, n, s);
+      }
+    }
   if (f.spacer != 0 && lanes_per_word(f) >= 16) {
     const int64_t wpr = words_per_row(f, inner), total = rows * wpr;
     pack_generic_kernel<W><<<grid_for(total, kThreads, sm_count() * 16), kThreads, 0, s>>>(
